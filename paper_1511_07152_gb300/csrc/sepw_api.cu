@@ -835,21 +835,22 @@ static int make_residual(sepw_ctx *ctx, int32_t Sr, int32_t OSr, double2 *out64,
     if (ctx->dp.facet)
         return fail(ctx, SEPW_ENOTSUP, "correction table not available in facet mode");
     const DevParams &p = ctx->dp;
-    double2 *X = nullptr, *t64 = nullptr;
-    const size_t nx = (size_t)p.P * OSr * Sr * p.N, nt = (size_t)p.P * p.OS * p.S;
+    unsigned char *work = nullptr;
+    double2 *t64 = nullptr;
+    const size_t nt = (size_t)p.P * p.OS * p.S;
     int rc;
-    if ((rc = grow(ctx, &X, nx)) || (rc = grow(ctx, &t64, nt))) {
-        cudaFree(X);
+    if ((rc = grow(ctx, &work, residual_work_bytes(p, Sr, OSr))) || (rc = grow(ctx, &t64, nt))) {
+        cudaFree(work);
         cudaFree(t64);
         return rc;
     }
     cudaError_t e = launch_taps(p, ctx->d_taper64, ctx->d_tw, t64, nullptr, s);
     if (e == cudaSuccess)
-        e = launch_residual_table(p, Sr, OSr, ctx->d_taper64, ctx->d_tw, t64, X, out64, out32,
+        e = launch_residual_table(p, Sr, OSr, ctx->d_taper64, ctx->d_tw, t64, work, out64, out32,
                                   s);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(s);
-    cudaFree(X);
+    cudaFree(work);
     cudaFree(t64);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "correction table");

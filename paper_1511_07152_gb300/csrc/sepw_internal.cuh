@@ -485,9 +485,11 @@ cudaError_t launch_facet_shift(int64_t nvis, double l0, double m0, int direction
                                const float2 *vin, double *uo, double *vo, float2 *vout,
                                cudaStream_t s);
 
-// sepw_residual.cu (stored correction F_w - F~_w)
+// sepw_residual.cu (stored correction F_w - F~_w); work: residual_work_bytes
+// bytes of device memory
+size_t residual_work_bytes(const DevParams &p, int Sr, int OSr);
 cudaError_t launch_residual_table(const DevParams &p, int Sr, int OSr, const double *taper64,
-                                  const double2 *tw, const double2 *taps64, double2 *X,
+                                  const double2 *tw, const double2 *taps64, void *work,
                                   double2 *out64, float2 *out32, cudaStream_t s);
 cudaError_t launch_grid_residual(const DevParams &p, int Sr, int OSr, const Plan &plan,
                                  const float2 *vis, const float *weight, const float2 *res,

@@ -8,9 +8,24 @@
 // entry c stands for the fine offset c * OS / OSr).  Built in float64:
 //   F_w(d_u, d_v) = (1/N^2) sum_{a,b} c1(nu_a) c1(nu_b) exp(2 pi i w (n_ab - 1))
 //                   exp(-2 pi i (d_u nu_a + d_v nu_b))
-// as two passes over the pixels (rows d_v first, then columns d_u), minus the
-// outer product of the 1-D taps at the same offsets.  The DFT phases reuse
-// the exact integer reduction of the taps kernel (twiddles of N*OS).
+// minus the outer product of the 1-D taps at the same offsets.
+//
+// The build is bound by the FP64 pipe (about 1.3 operations per clock and SM),
+// so the sum is folded by its symmetries.  With alpha = a - N/2 and
+// h(alpha, beta) = c1 c1 exp(2 pi i w (n - 1)), even in alpha and in beta and
+// symmetric in the two, only alpha = -N/2 (and beta = -N/2) has no partner:
+//   F_w = A(|d_v|, |d_u|) + e(d_v) B(|d_u|) + e(d_u) B(|d_v|)
+//         + e(d_v) e(d_u) h(N/2, N/2),                     e(d) = exp(pi i d),
+//   A(x, y) = sum_{alpha, beta = 0}^{N/2 - 1} C(x, beta) h(alpha, beta) C(y, alpha),
+//   B(x)    = sum_{beta = 0}^{N/2 - 1} C(x, beta) h(N/2, beta),
+//   C(x, beta) = (beta ? 2 : 1) cos(2 pi x beta / N)  (real).
+// The offsets are the multiples of 1/OSr from -Sr/2 + 1/OSr to Sr/2, so |d|
+// takes R/2 + 1 values for R = OSr Sr.  That leaves a sixteenth of the direct
+// sum's multiply-adds (half the alphas, betas and offsets, real by complex),
+// and one thread accumulates all rows of its alpha, so that a screen value is
+// computed once per (plane, alpha, beta) up to 33 rows.  N = 1024, 32 planes,
+// 8 x 8 cells, 8 x 8 offsets: the direct sum took 62.1 ms, this takes 2.4
+// (rows 2.21, columns 0.12, edge 0.06, table 0.01).
 //
 // Pass: each warp takes work items of the plan; per visibility the lanes
 // cover the Sr^2 cells.  Gridding adds W V R (conj(R) for w < 0) with float2
@@ -20,9 +35,7 @@
 
 namespace sepw {
 
-constexpr int kResRows = 8;  // table rows accumulated per thread in pass A
-
-// exp(-2 pi i d nu_b) with d * OS = dos (an integer) and nu_b = (b - N/2)/N
+// exp(-2 pi i d nu) at d * OS = dos (an integer) and nu = (b - N/2)/N
 __device__ __forceinline__ double2 dft_tw(const double2 *tw, int64_t M, int64_t dos, int b,
                                           int N)
 {
@@ -40,79 +53,195 @@ __device__ __forceinline__ int64_t row_dos(const DevParams &p, int Sr, int OSr, 
     return (int64_t)(kk - p.S / 2 + 1) * p.OS - (int64_t)c * (p.OS / OSr);
 }
 
-// pass A: X[p][r][a] = sum_b E[r][b] c1(nu_a) c1(nu_b) exp(2 pi i w_p (n_ab - 1))
-// grid (ceil(N / 256), P, ceil(R / kResRows)); block 256
-__global__ void __launch_bounds__(256) residual_rows_kernel(DevParams p, int Sr, int OSr,
-                                                            const double *taper64,
-                                                            const double2 *tw, double2 *X)
+// C[beta][x] for x = 0 .. R2 - 1 (offset x / OSr), beta < N/2; row stride R2
+__global__ void __launch_bounds__(256) residual_cos_kernel(DevParams p, int OSr, int R2,
+                                                           const double2 *tw, double *C)
 {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    const int plane = blockIdx.y;
-    const int R = OSr * Sr;
-    const int r0 = blockIdx.z * kResRows;
-    if (a >= p.N)
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= (int64_t)(p.N / 2) * R2)
         return;
+    const int beta = (int)(e / R2), x = (int)(e % R2);
     const int64_t M = (int64_t)p.N * p.OS;
-    const double wp = p.P > 1 ? (double)plane * p.w_max / (double)(p.P - 1) : 0.0;
-    const double l = (double)(a - p.N / 2) / (double)p.N * p.fov;
-    const double ca = taper64[a];
-    int64_t dos[kResRows];
-    double2 acc[kResRows];
-#pragma unroll
-    for (int q = 0; q < kResRows; ++q) {
-        dos[q] = r0 + q < R ? row_dos(p, Sr, OSr, r0 + q) : 0;
-        acc[q] = make_double2(0.0, 0.0);
-    }
-    for (int b = 0; b < p.N; ++b) {
-        const double m = (double)(b - p.N / 2) / (double)p.N * p.fov;
-        const double r2 = l * l + m * m;
-        const double nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
-        double s, c;
-        sincospi(2.0 * (wp * nm1), &s, &c);
-        const double h = ca * taper64[b];
-        const double hr = h * c, hi = h * s;
-#pragma unroll
-        for (int q = 0; q < kResRows; ++q) {
-            const double2 e = dft_tw(tw, M, dos[q], b, p.N);
-            acc[q].x += e.x * hr - e.y * hi;
-            acc[q].y += e.x * hi + e.y * hr;
-        }
-    }
-    const int64_t base = (int64_t)plane * R * p.N;
-#pragma unroll
-    for (int q = 0; q < kResRows; ++q)
-        if (r0 + q < R)
-            X[base + (int64_t)(r0 + q) * p.N + a] = acc[q];
+    const int64_t m = ((int64_t)x * (p.OS / OSr) * beta) % M;
+    C[e] = (beta ? 2.0 : 1.0) * tw[m].x;
 }
 
-// pass B: K[(rv, ru)] = (1/N^2) sum_a X[rv][a] E[ru][a], minus the separable
-// product; writes the table.  grid (ceil(R*R / 256), P); block 256
-__global__ void __launch_bounds__(256) residual_cols_kernel(DevParams p, int Sr, int OSr,
-                                                            const double2 *tw, const double2 *X,
-                                                            const double2 *taps64,
-                                                            double2 *out64, float2 *out32)
+__device__ __forceinline__ double2 screen(double wp, double l, double m)
+{
+    const double r2 = l * l + m * m;
+    const double nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
+    double s, c;
+    sincospi(2.0 * (wp * nm1), &s, &c);
+    return make_double2(c, s);
+}
+
+__device__ __forceinline__ double plane_w(const DevParams &p, int plane)
+{
+    return p.P > 1 ? (double)plane * p.w_max / (double)(p.P - 1) : 0.0;
+}
+
+// Rows: Y[p][z][x][alpha] = sum over the z-th part of beta of C(x, beta)
+// h(alpha, beta), for G values of x from x0 (x >= R2: not written).
+// grid (ceil(N/2 / 64), P, parts * groups); block 64
+constexpr int kResRowThreads = 64;
+
+template <int G>
+__global__ void __launch_bounds__(kResRowThreads) residual_rows_kernel(
+    DevParams p, int R2, int parts, const double *__restrict__ taper64,
+    const double *__restrict__ C, double2 *__restrict__ Y)
+{
+    const int H = p.N / 2;
+    const int alpha = blockIdx.x * kResRowThreads + threadIdx.x;
+    const int plane = blockIdx.y;
+    const int z = blockIdx.z % parts, x0 = (blockIdx.z / parts) * G;
+    if (alpha >= H)
+        return;
+    const int len = (H + parts - 1) / parts;
+    const int b0 = z * len, b1 = min(H, b0 + len);
+    const double wp = plane_w(p, plane);
+    const double l = (double)alpha / (double)p.N * p.fov;
+    const double ca = taper64[H + alpha];
+    double2 acc[G];
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+        acc[q] = make_double2(0.0, 0.0);
+    for (int beta = b0; beta < b1; ++beta) {
+        const double2 e = screen(wp, l, (double)beta / (double)p.N * p.fov);
+        const double t = ca * taper64[H + beta];
+        const double hr = t * e.x, hi = t * e.y;
+        const double *c = C + (int64_t)beta * R2 + x0;
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            const double cq = x0 + q < R2 ? __ldg(c + q) : 0.0;
+            acc[q].x = fma(cq, hr, acc[q].x);
+            acc[q].y = fma(cq, hi, acc[q].y);
+        }
+    }
+    double2 *y = Y + (((int64_t)plane * parts + z) * R2 + x0) * H + alpha;
+#pragma unroll
+    for (int q = 0; q < G; ++q)
+        if (x0 + q < R2)
+            y[(int64_t)q * H] = acc[q];
+}
+
+// B[p][x] = sum_beta C(x, beta) h(N/2, beta); B[p][R2] = h(N/2, N/2).
+// grid (P); block 256
+__global__ void __launch_bounds__(256) residual_edge_kernel(DevParams p, int R2,
+                                                            const double *__restrict__ taper64,
+                                                            const double *__restrict__ C,
+                                                            double2 *__restrict__ B)
+{
+    __shared__ double2 h[1024];
+    const int H = p.N / 2, plane = blockIdx.x;
+    const double wp = plane_w(p, plane);
+    const double l = 0.5 * p.fov, ca = taper64[0];
+    for (int xb = 0; xb < R2; xb += blockDim.x) {
+        const int x = xb + threadIdx.x;
+        double2 acc = make_double2(0.0, 0.0);
+        for (int c0 = 0; c0 < H; c0 += 1024) {
+            __syncthreads();
+            for (int i = threadIdx.x; i < 1024 && c0 + i < H; i += blockDim.x) {
+                const double2 e = screen(wp, l, (double)(c0 + i) / (double)p.N * p.fov);
+                const double t = ca * taper64[H + c0 + i];
+                h[i] = make_double2(t * e.x, t * e.y);
+            }
+            __syncthreads();
+            const int lim = min(1024, H - c0);
+            if (x < R2)
+                for (int i = 0; i < lim; ++i) {
+                    const double cq = __ldg(C + (int64_t)(c0 + i) * R2 + x);
+                    acc.x = fma(cq, h[i].x, acc.x);
+                    acc.y = fma(cq, h[i].y, acc.y);
+                }
+        }
+        if (x < R2)
+            B[(int64_t)plane * (R2 + 1) + x] = acc;
+    }
+    if (threadIdx.x == 0) {
+        const double2 e = screen(wp, l, l);
+        B[(int64_t)plane * (R2 + 1) + R2] = make_double2(ca * ca * e.x, ca * ca * e.y);
+    }
+}
+
+// Columns: A[p][x][y] = sum_alpha Y[p][.][x][alpha] C(y, alpha).  A block
+// takes one (plane, x): the parts of Y are summed into shared memory, then
+// thread (g, y) sums its quarter of each chunk of alphas.
+// grid (R2, P); block (64, 4)
+__global__ void __launch_bounds__(256) residual_cols_kernel(DevParams p, int R2, int parts,
+                                                            const double *__restrict__ C,
+                                                            const double2 *__restrict__ Y,
+                                                            double2 *__restrict__ A)
+{
+    constexpr int kCh = 512;
+    __shared__ double2 ys[kCh];
+    __shared__ double2 red[4][64];
+    const int H = p.N / 2, x = blockIdx.x, plane = blockIdx.y;
+    const int g = threadIdx.y, tid = g * 64 + threadIdx.x;
+    const double2 *y0 = Y + ((int64_t)plane * parts * R2 + x) * H;
+    for (int yb = 0; yb < R2; yb += 64) {
+        const int y = yb + threadIdx.x;
+        double2 acc = make_double2(0.0, 0.0);
+        for (int c0 = 0; c0 < H; c0 += kCh) {
+            __syncthreads();
+            for (int i = tid; i < kCh && c0 + i < H; i += 256) {
+                double2 v = y0[c0 + i];
+                for (int z = 1; z < parts; ++z) {
+                    const double2 w = y0[(int64_t)z * R2 * H + c0 + i];
+                    v.x += w.x;
+                    v.y += w.y;
+                }
+                ys[i] = v;
+            }
+            __syncthreads();
+            const int lim = min(kCh, H - c0);
+            if (y < R2)
+                for (int i = g; i < lim; i += 4) {
+                    const double cq = __ldg(C + (int64_t)(c0 + i) * R2 + y);
+                    acc.x = fma(cq, ys[i].x, acc.x);
+                    acc.y = fma(cq, ys[i].y, acc.y);
+                }
+        }
+        red[g][threadIdx.x] = acc;
+        __syncthreads();
+        if (g == 0 && y < R2) {
+            for (int q = 1; q < 4; ++q) {
+                acc.x += red[q][threadIdx.x].x;
+                acc.y += red[q][threadIdx.x].y;
+            }
+            A[((int64_t)plane * R2 + x) * R2 + y] = acc;
+        }
+    }
+}
+
+// F_w from A and B, minus the separable product; writes the table.
+// grid (ceil(R*R / 256), P); block 256
+__global__ void __launch_bounds__(256) residual_table_kernel(
+    DevParams p, int Sr, int OSr, int R2, const double2 *__restrict__ tw,
+    const double2 *__restrict__ A, const double2 *__restrict__ B,
+    const double2 *__restrict__ taps64, double2 *out64, float2 *out32)
 {
     const int R = OSr * Sr;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int plane = blockIdx.y;
-    if (e >= R * R)
+    if (e >= (int64_t)R * R)
         return;
-    const int rv = e / R, ru = e % R;
+    const int rv = (int)(e / R), ru = (int)(e % R);
     const int64_t M = (int64_t)p.N * p.OS;
-    const int64_t dos = row_dos(p, Sr, OSr, ru);
-    const double2 *x = X + ((int64_t)plane * R + rv) * p.N;
-    double kr = 0.0, ki = 0.0;
-    for (int a = 0; a < p.N; ++a) {
-        const double2 t = dft_tw(tw, M, dos, a, p.N);
-        const double2 v = x[a];
-        kr += v.x * t.x - v.y * t.y;
-        ki += v.x * t.y + v.y * t.x;
-    }
+    const int step = p.OS / OSr, k0 = (p.S - Sr) / 2;
+    const int64_t dv = row_dos(p, Sr, OSr, rv), du = row_dos(p, Sr, OSr, ru);
+    const int xv = (int)((dv < 0 ? -dv : dv) / step), xu = (int)((du < 0 ? -du : du) / step);
+    const double2 ev = dft_tw(tw, M, dv, 0, p.N), eu = dft_tw(tw, M, du, 0, p.N);
+    const double2 *b = B + (int64_t)plane * (R2 + 1);
+    const double2 bu = b[xu], bv = b[xv], h = b[R2];
+    const double2 a = A[((int64_t)plane * R2 + xv) * R2 + xu];
+    // e(dv) (B(du) + e(du) h) + e(du) B(dv) + A
+    const double tr = bu.x + (eu.x * h.x - eu.y * h.y), ti = bu.y + (eu.x * h.y + eu.y * h.x);
+    double kr = a.x + (ev.x * tr - ev.y * ti) + (eu.x * bv.x - eu.y * bv.y);
+    double ki = a.y + (ev.x * ti + ev.y * tr) + (eu.x * bv.y + eu.y * bv.x);
     const double inv = 1.0 / ((double)p.N * (double)p.N);
     kr *= inv;
     ki *= inv;
     // separable product at the same offsets: taps[p][o][kk]
-    const int step = p.OS / OSr, k0 = (p.S - Sr) / 2;
     const int cv = rv / Sr, k = rv % Sr, cu = ru / Sr, j = ru % Sr;
     const double2 tv = taps64[((int64_t)plane * p.OS + cv * step) * p.S + k0 + k];
     const double2 tu = taps64[((int64_t)plane * p.OS + cu * step) * p.S + k0 + j];
@@ -125,18 +254,67 @@ __global__ void __launch_bounds__(256) residual_cols_kernel(DevParams p, int Sr,
         out32[idx] = make_float2((float)kr, (float)ki);
 }
 
+// workspace: C, then Y, A and B (double2)
+struct ResidualWork {
+    int R2, parts;
+    size_t nC, nY, nA, nB;
+    size_t bytes() const { return sizeof(double2) * ((nC + 1) / 2 + nY + nA + nB); }
+};
+
+static ResidualWork residual_work(const DevParams &p, int Sr, int OSr)
+{
+    ResidualWork w;
+    const size_t H = p.N / 2;
+    w.R2 = OSr * Sr / 2 + 1;
+    // parts of the beta sum: enough warps for the FP64 pipes, at most 4 (the
+    // partial sums then take no more memory than the R x N sums they replace)
+    const size_t threads = (size_t)p.P * H;
+    w.parts = threads >= 200000 ? 1 : threads >= 100000 ? 2 : 4;
+    w.nC = H * w.R2;
+    w.nY = (size_t)p.P * w.parts * w.R2 * H;
+    w.nA = (size_t)p.P * w.R2 * w.R2;
+    w.nB = (size_t)p.P * (w.R2 + 1);
+    return w;
+}
+
+size_t residual_work_bytes(const DevParams &p, int Sr, int OSr)
+{
+    return residual_work(p, Sr, OSr).bytes();
+}
+
 cudaError_t launch_residual_table(const DevParams &p, int Sr, int OSr, const double *taper64,
-                                  const double2 *tw, const double2 *taps64, double2 *X,
+                                  const double2 *tw, const double2 *taps64, void *work,
                                   double2 *out64, float2 *out32, cudaStream_t s)
 {
-    const int R = OSr * Sr;
-    dim3 ga((p.N + 255) / 256, p.P, (R + kResRows - 1) / kResRows);
-    residual_rows_kernel<<<ga, 256, 0, s>>>(p, Sr, OSr, taper64, tw, X);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess)
+    const ResidualWork w = residual_work(p, Sr, OSr);
+    double2 *Y = (double2 *)work, *A = Y + w.nY, *B = A + w.nA;
+    double *C = (double *)(B + w.nB);
+    const int R = OSr * Sr, R2 = w.R2, H = p.N / 2;
+    cudaError_t e;
+    residual_cos_kernel<<<(unsigned)(((int64_t)H * R2 + 255) / 256), 256, 0, s>>>(p, OSr, R2, tw,
+                                                                                C);
+    if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    dim3 gb((R * R + 255) / 256, p.P);
-    residual_cols_kernel<<<gb, 256, 0, s>>>(p, Sr, OSr, tw, X, taps64, out64, out32);
+    const unsigned gx = (H + kResRowThreads - 1) / kResRowThreads;
+    if (R2 <= 9)
+        residual_rows_kernel<9><<<dim3(gx, p.P, w.parts), kResRowThreads, 0, s>>>(
+            p, R2, w.parts, taper64, C, Y);
+    else if (R2 <= 17)
+        residual_rows_kernel<17><<<dim3(gx, p.P, w.parts), kResRowThreads, 0, s>>>(
+            p, R2, w.parts, taper64, C, Y);
+    else
+        residual_rows_kernel<33><<<dim3(gx, p.P, w.parts * ((R2 + 32) / 33)), kResRowThreads, 0,
+                                   s>>>(p, R2, w.parts, taper64, C, Y);
+    if ((e = cudaGetLastError()) != cudaSuccess)
+        return e;
+    residual_edge_kernel<<<p.P, 256, 0, s>>>(p, R2, taper64, C, B);
+    if ((e = cudaGetLastError()) != cudaSuccess)
+        return e;
+    residual_cols_kernel<<<dim3(R2, p.P), dim3(64, 4), 0, s>>>(p, R2, w.parts, C, Y, A);
+    if ((e = cudaGetLastError()) != cudaSuccess)
+        return e;
+    residual_table_kernel<<<dim3((unsigned)(((int64_t)R * R + 255) / 256), p.P), 256, 0, s>>>(
+        p, Sr, OSr, R2, tw, A, B, taps64, out64, out32);
     return cudaGetLastError();
 }
 

@@ -118,3 +118,25 @@ def test_correction_rejects(env):
     with pytest.raises(S.SepwError) as e:
         S.sepw_grid_residual_planned(ctx, table, d["vis"], None, grid)
     assert e.value.status == S.ENOTSUP
+
+
+@pytest.mark.parametrize("N,S_,OS,Sr,OSr", [
+    (50, 8, 4, 4, 4),      # 9 folded offsets: the smallest row group, full
+    (50, 8, 4, 8, 4),      # 17: the next
+    (50, 12, 8, 12, 8),    # 49: two groups, the second partly empty
+    (16, 2, 3, 2, 1),      # smallest grid and support, odd oversampling
+    (1040, 8, 2, 8, 2),    # more pixels than one chunk of the column sums
+])
+def test_correction_table_sizes(env, N, S_, OS, Sr, OSr):
+    """The folded sums at the edges of their row groups and chunks (float64,
+    the bar of test_correction_table)."""
+    torch, S = env
+    wl = synth.random_case(113, 10, N, S_, OS, 3, w_max=700.0, fov=math.radians(5.0))
+    p = O.params_from(wl.params())
+    K, T = O.exact_table(p), O.taps(p)
+    ctx = S.sepw_create(S.make_params(**wl.params(), form=S.FORM_TILED))
+    want = O.residual_table(p, Sr, OSr, K=K, T=T)
+    got = S.sepw_make_residual_f64(ctx, Sr, OSr).cpu().numpy()
+    assert np.max(np.abs(got - want)) <= 1e-10 * np.max(np.abs(K))
+    t64 = S.sepw_make_taps_f64(ctx).cpu().numpy()
+    assert np.max(np.abs(t64 - T)) <= 1e-12 * max(1.0, np.max(np.abs(T)))
