@@ -320,98 +320,305 @@ cudaError_t launch_residual_table(const DevParams &p, int Sr, int OSr, const dou
 
 // ---------------------------------------------------------------------------
 // correction passes over the plan's work items
+//
+// A table entry (the Sr x Sr cells of one plane and offset pair) is read once
+// per visibility and used once, so the passes are bound by the L2 reads of
+// the entries (8 Sr^2 bytes a visibility; the table exceeds L1).  Two things
+// keep them near that:
+//   * lane l owns the cell pairs l, l + 32, ... (Sr is even, so a pair never
+//     straddles two rows): an entry arrives as whole 16-byte loads of
+//     consecutive lanes, several visibilities' loads in flight at a time;
+//   * the plan's slots come in runs of one (origin, conj) key: gridding sums a
+//     run in registers and adds it to the grid once, degridding reads its
+//     cells once per run.
+// A warp takes one of `parts` consecutive parts of an item, so that plans with
+// few items still fill the chip.  One visibility at a time with the cells
+// re-read (added by atomics) for each, 8 x 8 cells at 4M visibilities took
+// 1.90 ms (gridding) and 2.92 ms (degridding); see the figures below.
 // ---------------------------------------------------------------------------
 
 constexpr int kResWarps = 8;
+constexpr int kResBlocksPerSM = 4;
+// units a pass aims at per resident warp, and the fewest visibilities in one
+constexpr int kResUnitsPerWarp = 8;
+constexpr int kResMinUnit = 32;
 
+// parts of an item such that n_items * parts units fill the grid several times
+__device__ __forceinline__ int res_parts(int n_items, int chunk)
+{
+    const int want = gridDim.x * kResWarps * kResUnitsPerWarp;
+    return max(1, min(chunk / kResMinUnit, want / max(n_items, 1)));
+}
+
+// two adjacent cells of a table entry; VEC: the table is 16-byte aligned
+template <bool VEC>
+__device__ __forceinline__ float4 load_pair(const float2 *p)
+{
+    if constexpr (VEC)
+        return __ldg(reinterpret_cast<const float4 *>(p));
+    const float2 a = __ldg(p), b = __ldg(p + 1);
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// index of a record's table entry (fits 32 bits unsigned: P OSr^2 <= 2^31)
+__device__ __forceinline__ uint32_t res_entry(uint64_t r, int OSr, int step)
+{
+    return ((uint32_t)rec_plane(r) * OSr + rec_ov(r) / step) * OSr + rec_ou(r) / step;
+}
+
+// PPL: cell pairs per lane, ceil(Sr^2 / 64)
+template <int PPL, bool VEC>
 __global__ void __launch_bounds__(kResWarps * 32) grid_residual_kernel(
     DevParams p, int Sr, int OSr, const WorkItem *__restrict__ items,
     const int32_t *__restrict__ nitems, int32_t *counter, const uint64_t *__restrict__ rec,
     const int32_t *__restrict__ perm, const float2 *__restrict__ vis,
     const float *__restrict__ weight, const float2 *__restrict__ res, float2 *grid)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ float4 s_meta[kResWarps * 32];  // entry, key, W V
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4 *const meta = s_meta + warp * 32;
     const int n_items = *nitems;
-    const int step = p.OS / OSr, k0 = (p.S - Sr) / 2, cells = Sr * Sr;
+    const int step = p.OS / OSr, k0 = (p.S - Sr) / 2, cells = Sr * Sr, pairs = cells / 2;
+    const int parts = res_parts(n_items, p.chunk);
+    int off[PPL];  // grid offset of the lane's pairs from the footprint's first kept cell
+#pragma unroll
+    for (int q = 0; q < PPL; ++q) {
+        const int c = 2 * (lane + 32 * q);
+        off[q] = (c / Sr) * p.N + c % Sr;
+    }
     for (;;) {
-        int item = 0;
+        int unit = 0;
         if (lane == 0)
-            item = atomicAdd(counter, 1);
-        item = __shfl_sync(0xffffffffu, item, 0);
+            unit = atomicAdd(counter, 1);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        const int item = unit / parts, part = unit % parts;
         if (item >= n_items)
             break;
         const WorkItem it = items[item];
+        const int len = max(kResMinUnit, (it.count + parts - 1) / parts);
+        const int b0 = it.start + part * len, b1 = min(it.start + it.count, b0 + len);
+        if (b0 >= b1)
+            continue;
         const TileOrigin o = tile_origin(p, it.tile);
         float2 *const tg = grid + o.base + (o.gy0 + k0) * p.N + o.gx0 + k0;
-        for (int s = it.start; s < it.start + it.count; ++s) {
-            const uint64_t r = rec[s];
-            const int i = perm[s];
-            const float wt = weight ? __ldg(weight + i) : 1.0f;
-            const float2 x = __ldg(vis + i);
-            const float wr = wt * x.x, wi = wt * x.y;
-            const float sg = rec_conj(r) ? -1.f : 1.f;
-            const float2 *R = res + (((int64_t)rec_plane(r) * OSr + rec_ov(r) / step) * OSr +
-                                     rec_ou(r) / step) * cells;
-            float2 *g = tg + (int64_t)rec_ly(r) * p.N + rec_lx(r);
-            for (int c = lane; c < cells; c += 32) {
-                const float2 t = __ldg(R + c);
-                const float ti = sg * t.y;
-                atomicAdd(g + (int64_t)(c / Sr) * p.N + (c % Sr),
-                          make_float2(wr * t.x - wi * ti, wr * ti + wi * t.x));
+        float4 acc[PPL];
+#pragma unroll
+        for (int q = 0; q < PPL; ++q)
+            acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        int cur = -1;
+        // conj visibilities accumulated conj(W V) R: conjugated here
+        auto flush = [&]() {
+            if (cur < 0)
+                return;
+            const float sg = (cur & 1) ? -1.f : 1.f;
+            float2 *const g = tg + (int64_t)(cur >> 7) * p.N + ((cur >> 1) & 63);
+#pragma unroll
+            for (int q = 0; q < PPL; ++q) {
+                if (lane + 32 * q < pairs) {
+                    atomicAdd(g + off[q], make_float2(acc[q].x, sg * acc[q].y));
+                    atomicAdd(g + off[q] + 1, make_float2(acc[q].z, sg * acc[q].w));
+                }
+                acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
+        };
+        for (int base = b0; base < b1; base += 32) {
+            const int s = base + lane;
+            int kq = -1;
+            if (s < b1) {
+                const uint64_t r = rec[s];
+                const int i = perm[s];
+                const float wt = weight ? __ldg(weight + i) : 1.0f;
+                const float2 x = __ldg(vis + i);
+                const bool cj = rec_conj(r);
+                kq = ((rec_ly(r) * 64 + rec_lx(r)) << 1) | (cj ? 1 : 0);
+                meta[lane] = make_float4(__uint_as_float(res_entry(r, OSr, step)),
+                                         __int_as_float(kq), wt * x.x,
+                                         cj ? -wt * x.y : wt * x.y);
+            }
+            __syncwarp();
+            const int n = min(32, b1 - base);
+            const int kp = __shfl_up_sync(0xffffffffu, kq, 1);
+            const unsigned starts = __ballot_sync(0xffffffffu, lane < n && (lane == 0 || kq != kp));
+            for (int q = 0; q < n;) {
+                const unsigned later = starts & ~((2u << q) - 1u);
+                const int q1 = later ? __ffs(later) - 1 : n;
+                const int key = __float_as_int(meta[q].y);
+                if (key != cur) {
+                    flush();
+                    cur = key;
+                }
+#pragma unroll(PPL <= 2 ? 4 : 1)
+                for (; q < q1; ++q) {
+                    const float4 m = meta[q];
+                    const float2 *R = res + (size_t)__float_as_uint(m.x) * cells + 2 * lane;
+#pragma unroll
+                    for (int c = 0; c < PPL; ++c) {
+                        float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (lane + 32 * c < pairs)
+                            t = load_pair<VEC>(R + 64 * c);
+                        acc[c].x = fmaf(m.z, t.x, acc[c].x);
+                        acc[c].x = fmaf(-m.w, t.y, acc[c].x);
+                        acc[c].y = fmaf(m.z, t.y, acc[c].y);
+                        acc[c].y = fmaf(m.w, t.x, acc[c].y);
+                        acc[c].z = fmaf(m.z, t.z, acc[c].z);
+                        acc[c].z = fmaf(-m.w, t.w, acc[c].z);
+                        acc[c].w = fmaf(m.z, t.w, acc[c].w);
+                        acc[c].w = fmaf(m.w, t.z, acc[c].w);
+                    }
+                }
+            }
+            __syncwarp();
         }
+        flush();
     }
 }
 
+// Sum of v[e] over the 32 lanes for e = 0..7; v[0] then holds the sum for
+// e = lane >> 2.
+__device__ __forceinline__ void res_reduce8(float (&v)[8], int lane)
+{
+#pragma unroll
+    for (int h = 4; h > 0; h >>= 1) {
+        const bool up = lane & (4 * h);
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float send = up ? v[i] : v[i + h];
+            const float keep = up ? v[i + h] : v[i];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
+        }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+template <int PPL, bool VEC>
 __global__ void __launch_bounds__(kResWarps * 32) degrid_residual_kernel(
     DevParams p, int Sr, int OSr, const WorkItem *__restrict__ items,
     const int32_t *__restrict__ nitems, int32_t *counter, const uint64_t *__restrict__ rec,
     const int32_t *__restrict__ perm, const float2 *__restrict__ grid,
     const float *__restrict__ weight, const float2 *__restrict__ res, float2 *vis_out)
 {
-    const int lane = threadIdx.x & 31;
+    constexpr int G = PPL == 1 ? 8 : PPL == 2 ? 4 : PPL <= 4 ? 2 : 1;  // entries in flight
+    __shared__ uint2 s_meta[kResWarps * 32];  // entry, key
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint2 *const meta = s_meta + warp * 32;
     const int n_items = *nitems;
-    const int step = p.OS / OSr, k0 = (p.S - Sr) / 2, cells = Sr * Sr;
+    const int step = p.OS / OSr, k0 = (p.S - Sr) / 2, cells = Sr * Sr, pairs = cells / 2;
+    const int parts = res_parts(n_items, p.chunk);
+    int off[PPL];
+#pragma unroll
+    for (int q = 0; q < PPL; ++q) {
+        const int c = 2 * (lane + 32 * q);
+        off[q] = (c / Sr) * p.N + c % Sr;
+    }
     for (;;) {
-        int item = 0;
+        int unit = 0;
         if (lane == 0)
-            item = atomicAdd(counter, 1);
-        item = __shfl_sync(0xffffffffu, item, 0);
+            unit = atomicAdd(counter, 1);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
+        const int item = unit / parts, part = unit % parts;
         if (item >= n_items)
             break;
         const WorkItem it = items[item];
+        const int len = max(kResMinUnit, (it.count + parts - 1) / parts);
+        const int b0 = it.start + part * len, b1 = min(it.start + it.count, b0 + len);
+        if (b0 >= b1)
+            continue;
         const TileOrigin o = tile_origin(p, it.tile);
         const float2 *const tg = grid + o.base + (o.gy0 + k0) * p.N + o.gx0 + k0;
-        for (int s = it.start; s < it.start + it.count; ++s) {
-            const uint64_t r = rec[s];
-            const float sg = rec_conj(r) ? 1.f : -1.f;  // conj of the gridding kernel
-            const float2 *R = res + (((int64_t)rec_plane(r) * OSr + rec_ov(r) / step) * OSr +
-                                     rec_ou(r) / step) * cells;
-            const float2 *g = tg + (int64_t)rec_ly(r) * p.N + rec_lx(r);
-            float ar = 0.f, ai = 0.f;
-            for (int c = lane; c < cells; c += 32) {
-                const float2 t = __ldg(R + c);
-                const float ti = sg * t.y;
-                const float2 x = __ldg(g + (int64_t)(c / Sr) * p.N + (c % Sr));
-                ar += t.x * x.x - ti * x.y;
-                ai += t.x * x.y + ti * x.x;
-            }
+        float4 x[PPL];
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                ar += __shfl_xor_sync(0xffffffffu, ar, off);
-                ai += __shfl_xor_sync(0xffffffffu, ai, off);
+        for (int q = 0; q < PPL; ++q)
+            x[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        int cur = -1;
+        for (int base = b0; base < b1; base += 32) {
+            const int s = base + lane;
+            int i = -1;
+            float wt = 0.f;
+            float2 old = make_float2(0.f, 0.f);
+            if (s < b1) {
+                const uint64_t r = rec[s];
+                i = perm[s];
+                wt = weight ? __ldg(weight + i) : 1.0f;
+                old = vis_out[i];
+                meta[lane] = make_uint2(res_entry(r, OSr, step),
+                                        ((rec_ly(r) * 64 + rec_lx(r)) << 1) |
+                                            (rec_conj(r) ? 1 : 0));
             }
-            if (lane == 0) {
-                const int i = perm[s];
-                const float wt = weight ? __ldg(weight + i) : 1.0f;
-                float2 v = vis_out[i];
-                v.x += wt * ar;
-                v.y += wt * ai;
-                vis_out[i] = v;
+            __syncwarp();
+            const int n = min(32, b1 - base);
+            for (int qb = 0; qb < n; qb += 8) {
+                float vr[8], vi[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e)
+                    vr[e] = vi[e] = 0.f;
+#pragma unroll
+                for (int eb = 0; eb < 8; eb += G) {
+                    float4 t[G][PPL];
+#pragma unroll
+                    for (int e = 0; e < G; ++e) {
+                        const int q = qb + eb + e;
+                        const bool ok = q < n;
+                        const float2 *R = res + (size_t)(ok ? meta[q].x : 0u) * cells + 2 * lane;
+#pragma unroll
+                        for (int c = 0; c < PPL; ++c) {
+                            t[e][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (ok && lane + 32 * c < pairs)
+                                t[e][c] = load_pair<VEC>(R + 64 * c);
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < G; ++e) {
+                        if (qb + eb + e >= n)
+                            continue;
+                        const int key = (int)meta[qb + eb + e].y;
+                        if (key != cur) {
+                            cur = key;
+                            // plain-kernel runs work on conj(X)
+                            const float sg = (cur & 1) ? 1.f : -1.f;
+                            const float2 *g = tg + (int64_t)(cur >> 7) * p.N + ((cur >> 1) & 63);
+#pragma unroll
+                            for (int c = 0; c < PPL; ++c)
+                                if (lane + 32 * c < pairs) {
+                                    const float2 a = __ldg(g + off[c]), b = __ldg(g + off[c] + 1);
+                                    x[c] = make_float4(a.x, sg * a.y, b.x, sg * b.y);
+                                }
+                        }
+                        float sr = 0.f, si = 0.f;
+#pragma unroll
+                        for (int c = 0; c < PPL; ++c) {
+                            sr = fmaf(t[e][c].x, x[c].x, sr);
+                            sr = fmaf(-t[e][c].y, x[c].y, sr);
+                            si = fmaf(t[e][c].x, x[c].y, si);
+                            si = fmaf(t[e][c].y, x[c].x, si);
+                            sr = fmaf(t[e][c].z, x[c].z, sr);
+                            sr = fmaf(-t[e][c].w, x[c].w, sr);
+                            si = fmaf(t[e][c].z, x[c].w, si);
+                            si = fmaf(t[e][c].w, x[c].z, si);
+                        }
+                        vr[eb + e] = sr;
+                        vi[eb + e] = si;
+                    }
+                }
+                res_reduce8(vr, lane);
+                res_reduce8(vi, lane);
+                // visibility qb + e was staged by lane qb + e and summed on
+                // lanes 4 e .. 4 e + 3
+                const int src = 4 * (lane - qb);
+                const float re = __shfl_sync(0xffffffffu, vr[0], src & 31);
+                const float im = __shfl_sync(0xffffffffu, vi[0], src & 31);
+                if (lane >= qb && lane < qb + 8 && i >= 0) {
+                    const bool cj = meta[lane].y & 1;
+                    vis_out[i] = make_float2(fmaf(wt, re, old.x), fmaf(wt, cj ? im : -im, old.y));
+                }
             }
+            __syncwarp();
         }
     }
 }
+
+// X(ceil(pairs / 32) bound): the instantiated pairs per lane, Sr <= 32
+#define SEPW_FOR_EACH_PPL(X) X(1) X(2) X(3) X(4) X(8) X(16)
 
 cudaError_t launch_grid_residual(const DevParams &p, int Sr, int OSr, const Plan &plan,
                                  const float2 *vis, const float *weight, const float2 *res,
@@ -420,10 +627,19 @@ cudaError_t launch_grid_residual(const DevParams &p, int Sr, int OSr, const Plan
     cudaError_t e = cudaMemsetAsync(plan.d_item_counter, 0, sizeof(int32_t), s);
     if (e != cudaSuccess)
         return e;
-    grid_residual_kernel<<<num_sms * 4, kResWarps * 32, 0, s>>>(
-        p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec, plan.d_perm,
-        vis, weight, res, grid);
-    return cudaGetLastError();
+    const int ppl = (Sr * Sr / 2 + 31) / 32;
+    const bool vec = ((uintptr_t)res & 15) == 0;
+#define X(PPL)                                                                              \
+    if (ppl <= PPL) {                                                                       \
+        (vec ? grid_residual_kernel<PPL, true> : grid_residual_kernel<PPL, false>)          \
+            <<<num_sms * kResBlocksPerSM, kResWarps * 32, 0, s>>>(                          \
+                p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec,   \
+                plan.d_perm, vis, weight, res, grid);                                       \
+        return cudaGetLastError();                                                          \
+    }
+    SEPW_FOR_EACH_PPL(X)
+#undef X
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_degrid_residual(const DevParams &p, int Sr, int OSr, const Plan &plan,
@@ -433,10 +649,19 @@ cudaError_t launch_degrid_residual(const DevParams &p, int Sr, int OSr, const Pl
     cudaError_t e = cudaMemsetAsync(plan.d_item_counter + 1, 0, sizeof(int32_t), s);
     if (e != cudaSuccess)
         return e;
-    degrid_residual_kernel<<<num_sms * 4, kResWarps * 32, 0, s>>>(
-        p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec,
-        plan.d_perm, grid, weight, res, vis_out);
-    return cudaGetLastError();
+    const int ppl = (Sr * Sr / 2 + 31) / 32;
+    const bool vec = ((uintptr_t)res & 15) == 0;
+#define X(PPL)                                                                              \
+    if (ppl <= PPL) {                                                                       \
+        (vec ? degrid_residual_kernel<PPL, true> : degrid_residual_kernel<PPL, false>)      \
+            <<<num_sms * kResBlocksPerSM, kResWarps * 32, 0, s>>>(                          \
+                p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec, \
+                plan.d_perm, grid, weight, res, vis_out);                                   \
+        return cudaGetLastError();                                                          \
+    }
+    SEPW_FOR_EACH_PPL(X)
+#undef X
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace sepw

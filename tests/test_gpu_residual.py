@@ -140,3 +140,40 @@ def test_correction_table_sizes(env, N, S_, OS, Sr, OSr):
     assert np.max(np.abs(got - want)) <= 1e-10 * np.max(np.abs(K))
     t64 = S.sepw_make_taps_f64(ctx).cpu().numpy()
     assert np.max(np.abs(t64 - T)) <= 1e-12 * max(1.0, np.max(np.abs(T)))
+
+
+@pytest.mark.parametrize("form,S_,Sr,OSr", [
+    ("tiled", 24, 2, 2), ("tiled", 24, 8, 1), ("tiled", 24, 10, 4), ("tiled", 24, 12, 2),
+    ("tiled", 24, 16, 4), ("tiled", 24, 24, 2), ("tiled", 32, 32, 1), ("tc_bf16x2", 16, 14, 4)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_correction_pass_cells_per_lane(env, form, S_, Sr, OSr, aligned):
+    """The correction passes for every number of cell pairs per lane, with
+    entries on and off 16-byte boundaries, runs of one origin and conj mixed,
+    and plans in origin order and not; any table serves (FP32 bar 1e-5)."""
+    torch, S = env
+    wl = synth.random_case(114, 5000, 96, S_, 4, 5, w_max=800.0, radius_cells=12.0)
+    p = O.params_from(wl.params())
+    ctx = S.sepw_create(S.make_params(**wl.params(),
+                                      form=S.FORM_TILED if form == "tiled" else S.FORM_TC_BF16X2))
+    rng = np.random.default_rng(Sr)
+    shape = (p.P, OSr, OSr, Sr, Sr)
+    R = (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+    buf = torch.empty(R.size + 1, dtype=torch.complex64, device="cuda")
+    table = (buf[:-1] if aligned else buf[1:]).view(shape)
+    table.copy_(torch.from_numpy(R))
+    assert (table.data_ptr() % 16 == 0) == aligned
+    d = {k: torch.from_numpy(getattr(wl, k)).cuda() for k in ("u", "v", "w", "vis", "weight")}
+    S.sepw_plan(ctx, d["u"], d["v"], d["w"])
+    N = wl.grid_size
+    X = (rng.standard_normal((N, N)) + 1j * rng.standard_normal((N, N))).astype(np.complex64)
+    loc = O.locate(p, wl.u, wl.v, wl.w)
+    for weight in (wl.weight, None):
+        wt = None if weight is None else d["weight"]
+        grid = torch.from_numpy(X).cuda()
+        S.sepw_grid_residual_planned(ctx, table, d["vis"], wt, grid)
+        want = O.grid_residual(p, loc, wl.vis, weight, R)
+        assert rel_l2(grid.cpu().numpy() - X, want) <= 1e-5
+        out = d["vis"].clone()  # the pass adds
+        S.sepw_degrid_residual_planned(ctx, table, torch.from_numpy(X).cuda(), wt, out)
+        want = O.degrid_residual(p, loc, X, weight, R)
+        assert rel_l2(out.cpu().numpy() - wl.vis, want) <= 1e-5
