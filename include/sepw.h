@@ -263,9 +263,9 @@ SEPW_API int sepw_set_wait_limit(sepw_ctx *ctx, uint64_t limit_ns);
 /* Schedule of the tiled and tensor-core plans (the visibility-per-tile
  * schedule of a batch of W-stacking layers or channels with uneven counts,
  * Sec. 4.3): `chunk` visibilities per work item (64 .. 2048, a multiple of
- * 32; 0 = 2048, the default) and the number of parts a warp of the FP32
- * block gridder (S = 8, 16) takes of an item at a time (1 .. 16; 0 = 8 on
- * plans of at least 256 visibilities per tile, else 1, the default).  Takes
+ * 32; 0 = 2048, the default) and the number of parts the FP32 tiled
+ * gridders cut an item into, one per warp at a time (1 .. 16; 0 = parts of 32
+ * to 256 visibilities by the plan's size, the default).  Takes
  * effect at the next sepw_plan (the current plan is invalidated); results
  * do not depend on it beyond FP32 rounding order.  Host only. */
 SEPW_API int sepw_set_schedule(sepw_ctx *ctx, int32_t chunk, int32_t grid_parts);
@@ -450,7 +450,7 @@ SEPW_API int sepw_wstack_model_grids(sepw_ctx *ctx, const float *image, float *s
  * Same result as sepw_grid with the tiled FP32 form (p->form is ignored: the
  * parameters are checked as for SEPW_FORM_TILED, tile 0 meaning 32), but no
  * context is needed and nothing is allocated: the binning workspace is one
- * file-scope device array of about 26 MB compiled into the library, which
+ * file-scope device array of about 40 MB compiled into the library, which
  * every GPU that loads the library keeps until the process exits.  The call
  * makes no cudaMalloc / cudaFree and no allocating library call.
  *   - p, taps, u, v, w, vis, weight (NULL = 1), grid (accumulated, +=):

@@ -3,6 +3,7 @@
 // contract of every function.
 #include <cufft.h>
 #include <math.h>
+#include <algorithm>
 #include <new>
 #include <vector>
 #include <stdarg.h>
@@ -41,9 +42,11 @@ struct sepw_ctx {
     // workspace of the contraction gridder's pre-shifted tap tables
     unsigned char *d_tc2 = nullptr;
     size_t tc2_cap = 0;
-    // workspace of the tiled gridder's planar copy of the caller's tap
-    // table(s) (two tables: facet mode)
+    // workspace of the tiled gridders' copies of the caller's tap table(s):
+    // the block gridder's planar copy (two tables in facet mode) or the
+    // window gridder's padded ones
     float *d_planar = nullptr;
+    bool window = false;  // the tiled form grids with the window gridder
     Plan plan;
     cufftHandle fft = 0;
     bool fft_ready = false;
@@ -134,6 +137,7 @@ DevParams sepw::make_dev_params(const sepw_params *p)
     d.T = effective_tile(p);
     d.ntx = (d.N - d.S) / d.T + 1;
     d.t_inv = tile_reciprocal(d.T);
+    set_bins(d, kBinsSorted);
     d.fov = p->fov;
     d.half = (double)(d.N / 2);
     d.os_d = (double)d.OS;
@@ -179,13 +183,13 @@ void free_plan(Plan &pl)
     cudaFree(pl.d_rec);
     cudaFree(pl.d_perm);
     cudaFree(pl.d_drop_list);
-    cudaFree(pl.d_bin);
+    cudaFree(pl.d_bin_base);  // holds d_dropped
     cudaFree(pl.d_tile_count);
-    cudaFree(pl.d_tile_cursor);
+    cudaFree(pl.d_blocks);
     cudaFree(pl.d_items);
-    cudaFree(pl.d_nitems);
+    cudaFree(pl.d_units);
+    cudaFree(pl.d_nitems);  // holds d_nunits
     cudaFree(pl.d_item_counter);
-    cudaFree(pl.d_dropped);
     cudaFree(pl.d_offsets);
     pl = Plan();
 }
@@ -216,20 +220,39 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     Plan &pl = ctx->plan;
     int rc;
     const int64_t ntiles64 = (int64_t)ctx->dp.ntx * ctx->dp.ntx * ngrids;
-    if (ntiles64 > (1ll << 26))  // bin ids (tile * kSubBins + sub) stay in int32
+    if (ntiles64 > (1ll << 26))
         return fail(ctx, SEPW_EINVAL, "too many tiles (%lld)", (long long)ntiles64);
     const int ntiles = (int)ntiles64;
+    // the window gridder's bins unless their ids (tile * nsub + bin) leave int32
+    const bool sorts = ctx->p.form == SEPW_FORM_TILED || ctx->p.form == SEPW_FORM_TC_TF32;
+    set_bins(ctx->dp, ctx->window ? kBinsWindow : sorts ? kBinsSorted : kBinsTile);
+    if (ntiles64 * ctx->dp.nsub > INT32_MAX)
+        set_bins(ctx->dp, kBinsSorted);
+    if (ntiles64 * ctx->dp.nsub > INT32_MAX)
+        return fail(ctx, SEPW_EINVAL, "too many bins (%lld tiles)", (long long)ntiles64);
     if (!pl.d_nitems) {
-        if ((rc = grow(ctx, &pl.d_nitems, 1)) || (rc = grow(ctx, &pl.d_item_counter, 2)) ||
-            (rc = grow(ctx, &pl.d_dropped, 1)))
+        if ((rc = grow(ctx, &pl.d_nitems, 2)) || (rc = grow(ctx, &pl.d_item_counter, 2)))
             return rc;
+        pl.d_nunits = pl.d_nitems + 1;
     }
     if (pl.tiles_capacity < ntiles) {
-        if ((rc = grow(ctx, &pl.d_tile_count, ntiles)) ||
-            (rc = grow(ctx, &pl.d_tile_cursor, ntiles)) ||
-            (rc = grow(ctx, &pl.d_bin, (size_t)ntiles * kSubBins)))
+        pl.tiles_capacity = 0;
+        unsigned char *blocks = (unsigned char *)pl.d_blocks;
+        pl.d_blocks = nullptr;
+        rc = grow(ctx, &blocks, plan_block_bytes(ntiles));
+        pl.d_blocks = blocks;
+        if (rc || (rc = grow(ctx, &pl.d_tile_count, ntiles)))
             return rc;
         pl.tiles_capacity = ntiles;
+    }
+    const size_t bin_bytes = plan_bin_bytes(ntiles, ctx->dp);
+    if (pl.bins_capacity < bin_bytes) {
+        pl.bins_capacity = 0;
+        pl.d_dropped = nullptr;
+        if ((rc = grow(ctx, &pl.d_bin_base, bin_bytes)))
+            return rc;
+        pl.bins_capacity = bin_bytes;
+        pl.d_dropped = (unsigned long long *)pl.d_bin_base;
     }
     pl.ntiles = ntiles;
     if (ctx->p.form == SEPW_FORM_PLAIN)
@@ -251,7 +274,31 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
             return rc;
         pl.items_capacity = (int32_t)items;
     }
+    pl.unit = plan_unit(ctx->dp, nvis, ctx->num_sms);
+    if (ctx->p.form == SEPW_FORM_TILED) {
+        const int64_t units = (int64_t)ntiles + nvis / pl.unit + 1;
+        if (units > INT32_MAX)
+            return fail(ctx, SEPW_EINVAL, "too many work units");
+        if (pl.units_capacity < units) {
+            pl.units_capacity = 0;
+            if ((rc = grow(ctx, &pl.d_units, (size_t)units)))
+                return rc;
+            pl.units_capacity = (int32_t)units;
+        }
+    }
+    pl.window = ctx->dp.sub_log2 == 2;  // kBinsWindow
+    // for the kernels that walk runs of one origin: the tiled form's block and
+    // column gridders, and the tiled degridder of the TF32 form
+    pl.sorted = sorts && !pl.window;
     return SEPW_OK;
+}
+
+// The tiled form's gridder: the block gridder for S = 8 and 16, whose plans
+// are sorted by origin, and the window gridder for the other supports where
+// its tables can be had.
+bool use_window(const DevParams &p)
+{
+    return p.S != 8 && p.S != 16 && window_tables_bytes(p) > 0;
 }
 
 }  // namespace
@@ -339,10 +386,13 @@ int sepw_create(sepw_ctx **out, const sepw_params *p)
         return SEPW_ECUDA;
     }
     const int N = p->grid_size;
+    ctx->window = p->form == SEPW_FORM_TILED && use_window(ctx->dp);
     if ((rc = grow(ctx, &ctx->d_taper64, N)) || (rc = grow(ctx, &ctx->d_taper32, N)) ||
         (rc = grow(ctx, &ctx->d_tw, (size_t)N * p->oversample)) ||
         (rc = grow(ctx, &ctx->d_status, 1)) ||
-        (rc = grow(ctx, &ctx->d_planar, 2 * 2 * sepw_taps_count(p)))) {
+        (rc = grow(ctx, &ctx->d_planar,
+                   std::max(2 * 2 * sepw_taps_count(p),
+                            ctx->window ? window_tables_bytes(ctx->dp) / sizeof(float) : 0)))) {
         sepw_destroy(ctx);
         return rc;
     }
@@ -491,7 +541,7 @@ static int plan_impl(sepw_ctx *ctx, int32_t ngrids, const int64_t *offsets_host,
                 ctx->tc2_cap = need;
             }
         }
-        SEPW_CUDA(ctx, launch_plan(ctx->dp, nvis, u, v, w, pl, s));
+        SEPW_CUDA(ctx, launch_plan(ctx->dp, nvis, u, v, w, pl, ctx->num_sms, s));
     }
     pl.valid = true;
     return SEPW_OK;

@@ -1,15 +1,15 @@
 // Plan construction for the tiled forms: locate every visibility, bin it by
 // the T x T tile that holds its footprint origin and, inside the tile, by the
-// 4 x 4 sub-block of the origin and conj (counting sort with warp-aggregated
-// atomics), cut each tile into work items of at most kChunk visibilities, and
-// sort each item by (footprint origin, conj) so that consecutive visibilities
-// with the same origin and kernel conjugation can be accumulated in one
-// register block.
+// block of origins (set_bins; counting sort with warp-aggregated atomics), cut each tile into work items of at most kChunk visibilities (and
+// into the smaller units of the tiled gridders), and, for the kernels that
+// walk runs of one origin, sort each item by (footprint origin, conj).
 //
 // The update structure this serves is Sec. 5: every visibility adds a
 // separable S x S block at its own offset; visibilities that share a tile
 // share one shared-memory window, and visibilities that share an origin share
 // one register block.
+#include <algorithm>
+
 #include "sepw_internal.cuh"
 
 namespace sepw {
@@ -51,7 +51,7 @@ __global__ void __launch_bounds__(256) locate_bin_kernel(
                 g = lo;
             }
             const int lx = fx - tx * p.T, ly = fy - ty * p.T;
-            bin = ((g * p.ntx + ty) * p.ntx + tx) * kSubBins + sub_bin(lx, ly, L.conj, p);
+            bin = ((g * p.ntx + ty) * p.ntx + tx) * p.nsub + sub_bin(lx, ly, L.conj, p);
             rec0[i] = pack_rec(lx, ly, L.ou, L.ov, L.plane, L.conj);
         }
         bin_of[i] = bin;
@@ -80,158 +80,250 @@ __global__ void __launch_bounds__(256) locate_bin_kernel(
     }
 }
 
-// Pass 1b (one warp per tile): the tile's visibility count, and each bin's
-// count replaced by its offset inside the tile (exclusive scan of the 32).
-__global__ void __launch_bounds__(256) bin_scan_kernel(int32_t ntiles,
-                                                       int32_t *__restrict__ bin,
-                                                       int32_t *__restrict__ tile_count)
+// Passes 1b and 2: tile totals, then exclusive scans of the visibilities and
+// of the items and units over all tiles.  Full pieces (`chunk` or `unit`
+// visibilities) are listed before the partial ones, so that dynamically
+// scheduled workers take the heavy ones first; within each list the pieces
+// are in tile order.
+//
+// Pass 1b sums every tile's bins (a warp per tile) and every block's totals;
+// the last block to finish scans the totals of all blocks, so pass 2 starts
+// from its block's prefix with no launch in between.  The scan ran in a
+// single block before and took 426 us for the 524,288 tiles of a 128-grid
+// batch (now 20 us for its share of pass 2).
+struct Totals {
+    int32_t n, full_items, part_items, full_units, part_units;
+};
+__device__ __forceinline__ Totals operator+(const Totals &a, const Totals &b)
 {
-    static_assert(kSubBins == 32, "one lane per bin");
-    const int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (t >= ntiles)
-        return;
-    const int c = bin[t * kSubBins + lane];
-    int incl = c;
+    return {a.n + b.n, a.full_items + b.full_items, a.part_items + b.part_items,
+            a.full_units + b.full_units, a.part_units + b.part_units};
+}
+__device__ __forceinline__ Totals operator-(const Totals &a, const Totals &b)
+{
+    return {a.n - b.n, a.full_items - b.full_items, a.part_items - b.part_items,
+            a.full_units - b.full_units, a.part_units - b.part_units};
+}
+__device__ __forceinline__ Totals tile_totals(int n, int chunk, int unit)
+{
+    const int fi = n / chunk, fu = n / unit;
+    return {n, fi, n != fi * chunk, fu, n != fu * unit};
+}
+__device__ __forceinline__ Totals shfl_up(const Totals &v, int d)
+{
+    return {__shfl_up_sync(0xffffffffu, v.n, d), __shfl_up_sync(0xffffffffu, v.full_items, d),
+            __shfl_up_sync(0xffffffffu, v.part_items, d),
+            __shfl_up_sync(0xffffffffu, v.full_units, d),
+            __shfl_up_sync(0xffffffffu, v.part_units, d)};
+}
+__device__ __forceinline__ Totals warp_scan(Totals v, int lane)  // inclusive
+{
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, off);
+        const Totals y = shfl_up(v, off);
         if (lane >= off)
-            incl += y;
+            v = v + y;
     }
-    bin[t * kSubBins + lane] = incl - c;
+    return v;
+}
+// Inclusive scan over the block's threads; `total` gets the block's sum.
+// warps: one entry per warp and one more (shared).
+__device__ __forceinline__ Totals block_scan(Totals v, Totals *warps, Totals &total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    v = warp_scan(v, lane);
+    __syncthreads();
     if (lane == 31)
-        tile_count[t] = incl;
-}
-
-// Pass 2 (one block of 1024 threads): exclusive scans of the tile counts
-// (-> slot cursors) and of the per-tile chunk counts (-> work items).  Full
-// chunks (`chunk` visibilities) are listed before the partial ones, so that
-// dynamically scheduled workers take the heavy items first; within each list
-// the items are in tile order.  Warp w owns the tiles [w R, (w + 1) R) and
-// walks them 32 at a time, one tile per lane, so that its loads and its
-// cursor and item stores are coalesced: a first walk sums the range, a block
-// scan gives every warp its bases, and a second walk writes the cursors and
-// items from warp-shuffle scans of each group of 32 tiles.
-constexpr int kScanThreads = 1024;
-constexpr int kScanWarps = kScanThreads / 32;
-
-__device__ __forceinline__ void warp_scan3(int64_t &a, int32_t &b, int32_t &c, int lane)
-{
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int64_t x = __shfl_up_sync(0xffffffffu, a, off);
-        const int32_t y = __shfl_up_sync(0xffffffffu, b, off);
-        const int32_t z = __shfl_up_sync(0xffffffffu, c, off);
-        if (lane >= off) {
-            a += x;
-            b += y;
-            c += z;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kScanThreads) scan_kernel(
-    int32_t ntiles, int32_t chunk, const int32_t *__restrict__ tile_count,
-    int32_t *__restrict__ cursor, WorkItem *__restrict__ items, int32_t *nitems)
-{
-    __shared__ int64_t s_cnt[kScanWarps];
-    __shared__ int32_t s_full[kScanWarps], s_part[kScanWarps];
-    __shared__ int32_t s_tot_full, s_tot_part;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int R = (((ntiles + kScanWarps - 1) / kScanWarps) + 31) & ~31;  // tiles per warp
-    const int lo = min(ntiles, warp * R), hi = min(ntiles, lo + R);
-    // walk 1: the range's totals (visibilities, full chunks, partial chunks)
-    int64_t c = 0;
-    int32_t nf = 0, np = 0;
-    for (int i0 = lo; i0 < hi; i0 += 32 * 4) {
-        int n[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const int i = i0 + 32 * k + lane;
-            n[k] = i < hi ? tile_count[i] : 0;
-        }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            c += n[k];
-            nf += n[k] / chunk;
-            np += (n[k] % chunk) != 0;
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        c += __shfl_xor_sync(0xffffffffu, c, off);
-        nf += __shfl_xor_sync(0xffffffffu, nf, off);
-        np += __shfl_xor_sync(0xffffffffu, np, off);
-    }
-    if (lane == 0) {
-        s_cnt[warp] = c;
-        s_full[warp] = nf;
-        s_part[warp] = np;
-    }
+        warps[warp] = v;
     __syncthreads();
     if (warp == 0) {
-        int64_t wc = s_cnt[lane];
-        int32_t wf = s_full[lane], wp = s_part[lane];
-        const int64_t c0 = wc;
-        const int32_t f0 = wf, p0 = wp;
-        warp_scan3(wc, wf, wp, lane);
-        s_cnt[lane] = wc - c0;  // exclusive warp bases
-        s_full[lane] = wf - f0;
-        s_part[lane] = wp - p0;
-        if (lane == 31) {
-            s_tot_full = wf;
-            s_tot_part = wp;
-        }
+        const Totals w = lane < nw ? warps[lane] : Totals{0, 0, 0, 0, 0};
+        const Totals x = warp_scan(w, lane);
+        if (lane < nw)
+            warps[lane] = x - w;
+        if (lane == 31)
+            warps[32] = x;
     }
     __syncthreads();
-    const int32_t total_full = s_tot_full;
-    int64_t base_c = s_cnt[warp];
-    int32_t base_f = s_full[warp], base_p = total_full + s_part[warp];
-    // walk 2: cursors and items, 32 tiles at a time
-    for (int i0 = lo; i0 < hi; i0 += 32) {
-        const int i = i0 + lane;
-        const int n = i < hi ? tile_count[i] : 0;
-        const int nk = n / chunk, part = (n % chunk) != 0;
-        int64_t ic = n;
-        int32_t ik = nk, ipt = part;
-        warp_scan3(ic, ik, ipt, lane);
-        const int64_t off_c = base_c + ic - n;  // exclusive
-        const int32_t off_f = base_f + ik - nk, off_p = base_p + ipt - part;
-        if (i < hi) {
-            cursor[i] = (int32_t)off_c;
-            for (int q = 0; q < nk; ++q) {
-                WorkItem it;
-                it.tile = i;
-                it.start = (int32_t)(off_c + (int64_t)q * chunk);
-                it.count = chunk;
-                it.pad = 0;
-                items[off_f + q] = it;
-            }
-            if (part) {
-                WorkItem it;
-                it.tile = i;
-                it.start = (int32_t)(off_c + (int64_t)nk * chunk);
-                it.count = n % chunk;
-                it.pad = 0;
-                items[off_p] = it;
-            }
-        }
-        base_c += __shfl_sync(0xffffffffu, ic, 31);
-        base_f += __shfl_sync(0xffffffffu, ik, 31);
-        base_p += __shfl_sync(0xffffffffu, ipt, 31);
-    }
-    if (t == 0)
-        *nitems = total_full + s_tot_part;
+    total = warps[32];
+    return v + warps[warp];
 }
 
-// Pass 3: scatter visibility ids and records to their slots: tile start +
-// offset of the bin inside the tile + rank inside the bin.
+// Tiles a block of passes 1b and 2 takes: 32 (one per warp; 256 where a thread
+// takes a tile) as long as that leaves at most 1024 blocks to scan, then more.
+static int plan_block(int64_t ntiles, int nsub)
+{
+    int tb = nsub <= 4 ? 256 : 32;
+    while (tb < 1024 && ntiles > 1024ll * tb)
+        tb *= 2;
+    return tb;
+}
+constexpr int kPlanThreads = 1024, kPlanWarps = kPlanThreads / 32;
+
+__global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
+    int32_t ntiles, int32_t tb, int32_t nsub, int32_t chunk, int32_t unit,
+    const int32_t *__restrict__ bin, int32_t *__restrict__ tile_count,
+    Totals *__restrict__ blocks, unsigned *ticket)
+{
+    __shared__ Totals s_warps[33];
+    __shared__ int32_t s_n[1024];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t0 = blockIdx.x * tb;
+    if (nsub <= 4) {  // a thread per tile
+        if ((int)threadIdx.x < tb) {
+            int c = 0;
+            if (t0 + (int)threadIdx.x < ntiles)
+                for (int q = 0; q < nsub; ++q)
+                    c += bin[(int64_t)(t0 + threadIdx.x) * nsub + q];
+            s_n[threadIdx.x] = c;
+        }
+    }
+#pragma unroll 2
+    for (int k = nsub <= 4 ? tb : warp; k < tb; k += kPlanWarps) {  // a warp per tile
+        int c = 0;
+        if (t0 + k < ntiles) {
+            const int32_t *b = bin + (int64_t)(t0 + k) * nsub;
+            if (lane < nsub)
+                c = b[lane];
+            if (lane + 32 < nsub)
+                c += b[lane + 32];
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        if (lane == 0)
+            s_n[k] = c;
+    }
+    __syncthreads();
+    const int n = (int)threadIdx.x < tb ? s_n[threadIdx.x] : 0;
+    if ((int)threadIdx.x < tb && t0 + (int)threadIdx.x < ntiles)
+        tile_count[t0 + threadIdx.x] = n;
+    Totals total;
+    block_scan(tile_totals(n, chunk, unit), s_warps, total);
+    if (threadIdx.x == 0) {
+        blocks[blockIdx.x] = total;
+        __threadfence();
+        s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last)
+        return;
+    // exclusive prefixes of the blocks' totals, the sum of all at the end
+    __threadfence();
+    const int nb = gridDim.x;
+    Totals run{0, 0, 0, 0, 0};
+    for (int b0 = 0; b0 < nb; b0 += kPlanThreads) {
+        const int b = b0 + threadIdx.x;
+        Totals v{0, 0, 0, 0, 0};
+        if (b < nb) {
+            const volatile Totals *w = blocks + b;  // written by other blocks
+            v = {w->n, w->full_items, w->part_items, w->full_units, w->part_units};
+        }
+        Totals sum;
+        const Totals x = block_scan(v, s_warps, sum);
+        if (b < nb)
+            blocks[b] = run + x - v;
+        run = run + sum;
+    }
+    if (threadIdx.x == 0)
+        blocks[nb] = run;
+}
+
+// Lists the full pieces of size `size` of the block's tb tiles (tile tile0 +
+// k: those from piece pre[k] on, the first at slot first[k]; total pieces),
+// consecutive threads writing consecutive pieces.
+__device__ __forceinline__ void list_full(WorkItem *__restrict__ out, int tile0, int tb,
+                                          int total, int size, const int32_t *pre,
+                                          const int32_t *first)
+{
+    for (int e = threadIdx.x; e < total; e += kPlanThreads) {
+        int k = 0;  // the last tile with pre[k] <= e
+        for (int h = tb >> 1; h > 0; h >>= 1)
+            if (pre[k + h] <= e)
+                k += h;
+        out[e] = {tile0 + k, first[k] + (e - pre[k]) * size, size, 0};
+    }
+}
+
+// Pass 2: every bin's count replaced by its first slot; items and units.
+__global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
+    int32_t ntiles, int32_t tb, int32_t nsub, int32_t chunk, int32_t unit,
+    const int32_t *__restrict__ tile_count, const Totals *__restrict__ blocks,
+    int32_t *__restrict__ bin, WorkItem *__restrict__ items, int32_t *nitems,
+    WorkItem *__restrict__ units, int32_t *nunits)
+{
+    __shared__ Totals s_warps[33];
+    __shared__ int32_t s_n[1024], s_at[1024], s_items[1024], s_units[1024];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t0 = blockIdx.x * tb, t = t0 + threadIdx.x;
+    const int n = (int)threadIdx.x < tb && t < ntiles ? tile_count[t] : 0;
+    const Totals mine = tile_totals(n, chunk, unit);
+    Totals sum;
+    const Totals before = blocks[blockIdx.x];  // exclusive prefix of the block
+    const Totals in = block_scan(mine, s_warps, sum) - mine, at = before + in;
+    const Totals all = blocks[gridDim.x];
+    if (t == 0) {
+        *nitems = all.full_items + all.part_items;
+        if (units)
+            *nunits = all.full_units + all.part_units;
+    }
+    if ((int)threadIdx.x < tb) {
+        s_n[threadIdx.x] = n;
+        s_at[threadIdx.x] = at.n;
+        s_items[threadIdx.x] = in.full_items;
+        s_units[threadIdx.x] = in.full_units;
+        if (mine.part_items)
+            items[all.full_items + at.part_items] = {t, at.n + mine.full_items * chunk,
+                                                     n - mine.full_items * chunk, 0};
+        if (units && mine.part_units)
+            units[all.full_units + at.part_units] = {t, at.n + mine.full_units * unit,
+                                                     n - mine.full_units * unit, 0};
+    }
+    __syncthreads();
+    list_full(items + before.full_items, t0, tb, sum.full_items, chunk, s_items, s_at);
+    if (units)
+        list_full(units + before.full_units, t0, tb, sum.full_units, unit, s_units, s_at);
+    if (nsub <= 4) {  // a thread per tile
+        if ((int)threadIdx.x < tb && n > 0) {
+            int32_t *b = bin + (int64_t)t * nsub;
+            for (int q = 0, run = at.n; q < nsub; ++q) {
+                const int c = b[q];
+                b[q] = run;
+                run += c;
+            }
+        }
+        return;
+    }
+#pragma unroll 2
+    for (int k = warp; k < tb; k += kPlanWarps) {
+        if (s_n[k] == 0)
+            continue;  // nobody looks up the slots of an empty tile
+        int32_t *b = bin + (int64_t)(t0 + k) * nsub;
+        const int c0 = lane < nsub ? b[lane] : 0, c1 = lane + 32 < nsub ? b[lane + 32] : 0;
+        int i0 = c0, i1 = c1;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y0 = __shfl_up_sync(0xffffffffu, i0, off);
+            const int y1 = __shfl_up_sync(0xffffffffu, i1, off);
+            if (lane >= off) {
+                i0 += y0;
+                i1 += y1;
+            }
+        }
+        const int at0 = s_at[k], at1 = at0 + __shfl_sync(0xffffffffu, i0, 31);
+        if (lane < nsub)
+            b[lane] = at0 + i0 - c0;
+        if (lane + 32 < nsub)
+            b[lane + 32] = at1 + i1 - c1;
+    }
+}
+static_assert(kMaxSubBins == 64, "two bins per lane");
+
+// Pass 3: scatter visibility ids and records to their slots: first slot of the
+// bin + rank inside the bin.
 __global__ void __launch_bounds__(256) scatter_kernel(
     int64_t nvis, const int32_t *__restrict__ bin_of, const int32_t *__restrict__ rank_of,
-    const uint64_t *__restrict__ rec0, const int32_t *__restrict__ tile_start,
-    const int32_t *__restrict__ bin_off, int32_t *__restrict__ perm,
-    uint64_t *__restrict__ rec)
+    const uint64_t *__restrict__ rec0, const int32_t *__restrict__ bin_first,
+    int32_t *__restrict__ perm, uint64_t *__restrict__ rec)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nvis)
@@ -239,31 +331,27 @@ __global__ void __launch_bounds__(256) scatter_kernel(
     const int b = bin_of[i];
     if (b < 0)
         return;
-    const int slot = __ldg(tile_start + b / kSubBins) + __ldg(bin_off + b) + rank_of[i];
+    const int slot = __ldg(bin_first + b) + rank_of[i];
     perm[slot] = (int32_t)i;
     rec[slot] = rec0[i];
 }
 
 // Pass 4: inside each work item, counting sort by (footprint origin, conj),
-// sub-block major: the key orders by the 4 x 4 sub-block of the origin and
-// conj (the bin of pass 1), then by the origin's row and column inside the
-// sub-block (edge at most E = ceil(T / 4)), 32 E^2 <= 8192 keys.
-// Visibilities that share a key share one register block in the tiled
-// kernels, and the block never mixes conjugated and plain kernels; the
-// sub-blocks stay contiguous inside an item, so a run of slots that starts
-// and ends in one sub-block lies inside it.  One block per item; the item's
-// slots are rewritten in place.  The order among equal keys is arbitrary.
+// bin major: the key orders by the bin of pass 1 (block of origins and conj),
+// then by the origin's row and column inside the block.  Visibilities that
+// share a key share one register block in the tiled kernels, and the block
+// never mixes conjugated and plain kernels; the bins stay contiguous inside an
+// item, so a run of slots that starts and ends in one bin lies inside it.  One
+// block of threads per item; the item's slots are rewritten in place.  The
+// order among equal keys is arbitrary.
 constexpr int kSortThreads = 512;
 constexpr int kMaxSortBins = 2 * 64 * 64;
 constexpr int kMaxBinsPerThread = kMaxSortBins / kSortThreads;
 
-__device__ __forceinline__ int sort_key(uint64_t r, const DevParams &p, int E)
+__device__ __forceinline__ int sort_key(uint64_t r, const DevParams &p)
 {
-    const int lx = rec_lx(r), ly = rec_ly(r);
-    const int sx = div_tile(lx * 4, p), sy = div_tile(ly * 4, p);
-    const int x0 = (sx * p.T + 3) >> 2, y0 = (sy * p.T + 3) >> 2;  // first cell
-    const int sub = ((sx * 4 + sy) << 1) | (rec_conj(r) ? 1 : 0);  // as sub_bin
-    return (sub * E + (ly - y0)) * E + (lx - x0);
+    const int lx = rec_lx(r), ly = rec_ly(r), lg = p.sub_log2, m = (1 << lg) - 1;
+    return (sub_bin(lx, ly, rec_conj(r), p) << lg | (ly & m)) << lg | (lx & m);
 }
 
 __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
@@ -280,8 +368,7 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     const WorkItem it = items[item];
     const int n = it.count;
-    const int E = (p.T + 3) / 4;
-    const int nb = 32 * E * E;
+    const int nb = p.nsub << (2 * p.sub_log2);
     const int per = (nb + kSortThreads - 1) / kSortThreads;
     for (int b = threadIdx.x; b < per * kSortThreads; b += kSortThreads)
         hist[b] = 0;
@@ -297,7 +384,7 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
             const uint64_t r = rec[it.start + q];
             s_rec[q] = r;
             s_perm[q] = perm[it.start + q];
-            key = sort_key(r, p, E);
+            key = sort_key(r, p);
         }
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         if (act && lane_id == __ffs(peers) - 1)
@@ -353,7 +440,7 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
         int key = -1;
         if (act) {
             r = s_rec[q];
-            key = sort_key(r, p, E);
+            key = sort_key(r, p);
         }
         const unsigned peers = __match_any_sync(0xffffffffu, key);
         const int leader = __ffs(peers) - 1;
@@ -388,57 +475,78 @@ cudaError_t launch_zero_dropped(const Plan &plan, float2 *vis, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Visibilities in a unit of the tiled gridders: about eight units for each of
+// the ~40 warps an SM holds, 32 to 256.  Whole items of 2048 gave 524,288
+// visibilities to 400 warps (S = 16, 758 us; 155 us now); 4M visibilities at
+// S = 8: 190 us with two units per warp, 178 us with eight.  Above 256 the
+// last warps work alone on 32M visibilities (2.13 ms for 256, 2.16 for 512,
+// 2.24 for 1024, 2.38 for 2048); below, sparse tiles fall into more units
+// (128 grids at S = 12: 8.97 ms for 256, 9.55 for 128).
+int32_t plan_unit(const DevParams &p, int64_t nvis, int num_sms)
+{
+    if (p.grid_parts > 0)
+        return std::max(32, ((p.chunk + p.grid_parts - 1) / p.grid_parts + 31) & ~31);
+    const int64_t u = (nvis / std::max(1, 320 * num_sms) + 31) & ~31ll;
+    return (int32_t)std::min<int64_t>(256, std::max<int64_t>(32, u));
+}
+
+size_t plan_bin_bytes(int64_t ntiles, const DevParams &p)
+{
+    return kBinHeader + sizeof(int32_t) * (size_t)p.nsub * (size_t)ntiles;
+}
+size_t plan_block_bytes(int64_t ntiles)
+{
+    const int tb = plan_block(ntiles, kMaxSubBins);  // the most blocks
+    return sizeof(Totals) * (size_t)((ntiles + tb - 1) / tb + 1);
+}
+
 cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
-                        const double *v, const double *w, Plan &plan, cudaStream_t s)
+                        const double *v, const double *w, Plan &plan, int num_sms,
+                        cudaStream_t s)
 {
     cudaError_t e;
-    e = cudaMemsetAsync(plan.d_bin, 0, sizeof(int32_t) * kSubBins * (size_t)plan.ntiles, s);
+    // one clear for the dropped count, the ticket and the bins
+    e = cudaMemsetAsync(plan.d_bin_base, 0, plan_bin_bytes(plan.ntiles, p), s);
     if (e != cudaSuccess)
         return e;
-    e = cudaMemsetAsync(plan.d_dropped, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess)
-        return e;
+    int32_t *const bin = (int32_t *)(plan.d_bin_base + kBinHeader);
     if (nvis > 0) {
         locate_bin_kernel<<<(unsigned)((nvis + 255) / 256), 256, 0, s>>>(
-            p, nvis, u, v, w, plan.d_tile, plan.d_rank, plan.d_rec0, plan.d_bin,
+            p, nvis, u, v, w, plan.d_tile, plan.d_rank, plan.d_rec0, bin,
             plan.d_dropped, plan.d_drop_list, plan.ngrids, plan.d_offsets);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }
-    bin_scan_kernel<<<(unsigned)(((int64_t)plan.ntiles * 32 + 255) / 256), 256, 0, s>>>(
-        plan.ntiles, plan.d_bin, plan.d_tile_count);
+    const int tb = plan_block(plan.ntiles, p.nsub), nblk = (plan.ntiles + tb - 1) / tb;
+    Totals *const blocks = (Totals *)plan.d_blocks;
+    tile_count_kernel<<<nblk, kPlanThreads, 0, s>>>(plan.ntiles, tb, p.nsub, p.chunk, plan.unit, bin,
+                                          plan.d_tile_count, blocks,
+                                          (unsigned *)(plan.d_bin_base + kBinTicket));
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    scan_kernel<<<1, kScanThreads, 0, s>>>(plan.ntiles, p.chunk, plan.d_tile_count,
-                                           plan.d_tile_cursor, plan.d_items, plan.d_nitems);
+    tile_items_kernel<<<nblk, kPlanThreads, 0, s>>>(plan.ntiles, tb, p.nsub, p.chunk, plan.unit,
+                                          plan.d_tile_count, blocks, bin, plan.d_items,
+                                          plan.d_nitems, plan.d_units, plan.d_nunits);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     if (nvis > 0) {
         scatter_kernel<<<(unsigned)((nvis + 255) / 256), 256, 0, s>>>(
-            nvis, plan.d_tile, plan.d_rank, plan.d_rec0, plan.d_tile_cursor, plan.d_bin,
-            plan.d_perm, plan.d_rec);
+            nvis, plan.d_tile, plan.d_rank, plan.d_rec0, bin, plan.d_perm, plan.d_rec);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
-        // the per-item sort by (sub-block, conj, origin) serves the kernels
-        // that walk runs of one origin (the tiled FP32 gridder and
-        // degridder); the 16-bit tensor-core forms (one-part and hi + lo)
-        // grid and degrid in any order within an item and skip it
-        if (plan.form == SEPW_FORM_TC_BF16 || plan.form == SEPW_FORM_TC_FP16 ||
-            plan.form == SEPW_FORM_TC_FP16X2 || plan.form == SEPW_FORM_TC_BF16X2)
+        // the per-item sort by (block, origin, conj) serves the kernels that
+        // walk runs of one origin; the 16-bit tensor-core forms and the
+        // window gridder take any order within a block and skip it
+        if (!plan.sorted)
             return cudaSuccess;
-        const int E = (p.T + 3) / 4;
-        const int nb = 32 * E * E;
+        const int nb = p.nsub << (2 * p.sub_log2);
         const size_t shm =
             sizeof(int32_t) * kSortThreads * ((nb + kSortThreads - 1) / kSortThreads);
         e = cudaFuncSetAttribute(item_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)shm);
         if (e != cudaSuccess)
             return e;
-        int dev = 0, sms = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-            (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-            return e;
-        const int nblk = std::max(1, std::min(plan.items_capacity, 16 * sms));
+        const int nblk = std::max(1, std::min(plan.items_capacity, 16 * num_sms));
         item_sort_kernel<<<nblk, kSortThreads, shm, s>>>(p, plan.d_items, plan.d_nitems,
                                                          plan.d_perm, plan.d_rec);
         if ((e = cudaGetLastError()) != cudaSuccess)

@@ -16,6 +16,10 @@ struct DevParams {
     int32_t N, S, OS, P, T;
     int32_t ntx;      // tiles per axis for the tiled forms
     uint32_t t_inv;   // ceil(2^32 / T), see div_tile
+    int32_t sub_log2; // log2 of the edge of a plan's blocks of origins
+    int32_t sub_n;    // blocks along a tile's edge
+    int32_t sub_conj; // 1: a block's conj visibilities are a bin of their own
+    int32_t nsub;     // bins of a tile
     double fov;       // inverse cell size: x = u * fov + N/2
     double half;      // N/2 as a double
     double os_d;      // OS as a double
@@ -306,13 +310,32 @@ __device__ __forceinline__ bool record_ok(const DevParams &p, uint64_t r, int i,
 constexpr int kChunk = 2048;      // largest work item (visibilities), the default
 constexpr int kMaxWindow = 64;    // T + S - 1 <= kMaxWindow
 
-// Plan workspace (owned by the context).
-// Binning below the tile: each tile's visibilities are grouped by the 4 x 4
-// sub-block of the tile that holds their footprint origin and by conj, 32
-// bins per tile, before the tile is cut into work items.  An item then spans
-// few sub-blocks, so after the per-item sort its runs of one origin are long
-// (one register block accumulates a whole run).
-constexpr int kSubBins = 32;
+// Binning below the tile: each tile's visibilities are grouped by the block
+// of origins (edge 2^sub_log2) that holds their footprint origin before the
+// tile is cut into work items.
+//   kBinsWindow: edge 4, the window gridder's (its registers cover a block's
+//     footprints); T <= 32, so at most 64 bins.
+//   kBinsSorted: edge 8 (16 for T > 32) and conj apart, for plans whose items
+//     are sorted by origin: an item then spans few bins and its runs of one
+//     key are long.  Edge 4 made the scatter of 32M visibilities slower (535
+//     against 438 us: its writes go to four times as many places) and the
+//     runs no longer; without conj apart the S = 8 gridder took 190 us
+//     against 181 us (4M visibilities).
+//   kBinsTile: one bin, for the tensor-core forms, which take any order
+//     (8M visibilities, T = 16: plan 308 -> 178 us with 32 bins -> 1).
+enum PlanBins { kBinsWindow, kBinsSorted, kBinsTile };
+inline void set_bins(DevParams &d, PlanBins b)
+{
+    d.sub_log2 = b == kBinsWindow ? 2 : b == kBinsTile ? 6 : d.T <= 32 ? 3 : 4;
+    d.sub_n = (d.T + (1 << d.sub_log2) - 1) >> d.sub_log2;
+    d.sub_conj = b == kBinsSorted ? 1 : 0;
+    d.nsub = (d.sub_n * d.sub_n) << d.sub_conj;
+}
+constexpr int kMaxSubBins = 64;
+
+// the plan's bins follow a header that is cleared with them: the dropped
+// count (8 bytes), then the tile passes' ticket
+constexpr size_t kBinHeader = 64, kBinTicket = 8;
 
 // ceil(2^32 / T) for the tile edge T (8 <= T <= 64)
 // Bounds of locate_axis's integer path for grid size N and OS = 2^os_log2
@@ -346,33 +369,42 @@ __device__ __forceinline__ int div_tile(int n, const DevParams &p)
     return (int)__umulhi((unsigned)n, p.t_inv);
 }
 
-// column-major: the eight bins of one column of sub-blocks are consecutive
+// column-major: the blocks of one column are consecutive, downwards
 __device__ __forceinline__ int sub_bin(int lx, int ly, bool conj, const DevParams &p)
 {
-    return ((div_tile(lx * 4, p) * 4 + div_tile(ly * 4, p)) << 1) | (conj ? 1 : 0);
+    const int b = (lx >> p.sub_log2) * p.sub_n + (ly >> p.sub_log2);
+    return p.sub_conj ? b << 1 | (conj ? 1 : 0) : b;
 }
 
+// Plan workspace (owned by the context).
 struct Plan {
     int64_t nvis = 0;
     int64_t capacity = 0;       // allocated visibility slots
     int32_t ntiles = 0;
     int32_t tiles_capacity = 0;
+    size_t bins_capacity = 0;   // bytes at d_bin_base
     int32_t items_capacity = 0;
+    int32_t units_capacity = 0;
+    int32_t unit = 256;         // visibilities per unit
     bool valid = false;
+    bool sorted = true;         // items sorted by (block, origin, conj)
+    bool window = false;        // gridding by the window gridder
     int form = 0;
     // tiled forms
     int32_t *d_tile = nullptr;      // [nvis] bin id per visibility (-1 dropped)
     int32_t *d_rank = nullptr;      // [nvis] rank of the visibility inside its bin
-    int32_t *d_bin = nullptr;       // [ntiles * kSubBins] bin counts, then cursors
+    unsigned char *d_bin_base = nullptr;  // header, then [ntiles * nsub] counts, then slots
     uint64_t *d_rec0 = nullptr;     // [nvis] record, input order
     uint64_t *d_rec = nullptr;      // [nvis] record, slot order
     int32_t *d_perm = nullptr;      // [nvis] slot -> visibility index
     int32_t *d_tile_count = nullptr;   // [ntiles]
-    int32_t *d_tile_cursor = nullptr;  // [ntiles]
+    void *d_blocks = nullptr;          // totals of the tile passes' blocks
     WorkItem *d_items = nullptr;       // [items_capacity]
-    int32_t *d_nitems = nullptr;       // [1]
+    WorkItem *d_units = nullptr;       // [units_capacity], tiled form only
+    int32_t *d_nitems = nullptr;       // [2]: items, units
+    int32_t *d_nunits = nullptr;       // d_nitems + 1
     int32_t *d_item_counter = nullptr; // [2] persistent-kernel work counters
-    unsigned long long *d_dropped = nullptr;  // [1]
+    unsigned long long *d_dropped = nullptr;  // in d_bin_base's header
     int32_t *d_drop_list = nullptr;           // [nvis] indices of dropped visibilities
     int32_t ngrids = 1;                // batched plans: grids in the batch
     int64_t *d_offsets = nullptr;      // [ngrids + 1] visibility offsets per grid
@@ -413,8 +445,13 @@ cudaError_t launch_degrid_plain(const DevParams &p, int64_t nvis, const double *
                                 unsigned long long *dropped, cudaStream_t s);
 
 // sepw_bin.cu
+// sizes of Plan::d_bin_base and Plan::d_blocks, and the unit for nvis
+size_t plan_bin_bytes(int64_t ntiles, const DevParams &p);
+size_t plan_block_bytes(int64_t ntiles);
+int32_t plan_unit(const DevParams &p, int64_t nvis, int num_sms);
 cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
-                        const double *v, const double *w, Plan &plan, cudaStream_t s);
+                        const double *v, const double *w, Plan &plan, int num_sms,
+                        cudaStream_t s);
 // batched: plan.ngrids > 1 and plan.d_offsets hold the per-grid ranges
 cudaError_t launch_zero_dropped(const Plan &plan, float2 *vis, cudaStream_t s);
 
@@ -429,6 +466,14 @@ cudaError_t launch_degrid_tiled(const DevParams &p, const Plan &plan,
                                 const float2 *grid, const float *weight,
                                 const float2 *taps, float2 *vis, int num_sms,
                                 cudaStream_t s);
+
+// sepw_window.cu: gridder of the tiled form for the supports the block gridder
+// does not take (plan.window).  tables: window_tables_bytes(p) bytes for the
+// per-call tap tables, 0 if it does not take these parameters.
+size_t window_tables_bytes(const DevParams &p);
+cudaError_t launch_grid_window(const DevParams &p, const Plan &plan, const float2 *vis,
+                               const float *weight, const float2 *taps, float *tables,
+                               float2 *grid, int num_sms, cudaStream_t s);
 
 // Control of the tensor-core kernels: the limit of every bounded mbarrier
 // wait, and a test hook (stall != 0: the MMA thread issues and commits

@@ -7,7 +7,7 @@
 // raw allocations from plugins.  This entry point serves them: instead of a
 // context's workspace it uses one fixed scratch array compiled into the
 // library as a file-scope __device__ variable, so every GPU that loads the
-// library holds that array (kNoallocBytes, about 26 MB) until the process
+// library holds that array (kNoallocBytes, about 40 MB) until the process
 // exits.
 //
 // The scratch holds the same plan as the context path (bin ids and ranks,
@@ -38,14 +38,21 @@ constexpr size_t kOffRec0 = align256(kOffRank + sizeof(int32_t) * kMaxVis);
 constexpr size_t kOffRec = align256(kOffRec0 + sizeof(uint64_t) * kMaxVis);
 constexpr size_t kOffPerm = align256(kOffRec + sizeof(uint64_t) * kMaxVis);
 constexpr size_t kOffDrop = align256(kOffPerm + sizeof(int32_t) * kMaxVis);
+constexpr int64_t kMaxUnits = kMaxTiles + kMaxVis / 32 + 1;
 constexpr size_t kOffCount = align256(kOffDrop + sizeof(int32_t) * kMaxVis);
-constexpr size_t kOffCursor = align256(kOffCount + sizeof(int32_t) * kMaxTiles);
-constexpr size_t kOffBin = align256(kOffCursor + sizeof(int32_t) * kMaxTiles);
-constexpr size_t kOffItems = align256(kOffBin + sizeof(int32_t) * kSubBins * kMaxTiles);
-constexpr size_t kOffNitems = align256(kOffItems + sizeof(WorkItem) * kMaxItems);
-constexpr size_t kOffCounter = align256(kOffNitems + sizeof(int32_t));
-constexpr size_t kOffDropped = align256(kOffCounter + 2 * sizeof(int32_t));
-constexpr size_t kNoallocBytes = align256(kOffDropped + sizeof(unsigned long long));
+constexpr size_t kOffBlocks = align256(kOffCount + sizeof(int32_t) * kMaxTiles);
+constexpr size_t kBlocksBytes = 64 * 1024;  // plan_block_bytes(kMaxTiles), checked per call
+constexpr size_t kOffBin = align256(kOffBlocks + kBlocksBytes);
+constexpr size_t kOffItems =
+    align256(kOffBin + kBinHeader + sizeof(int32_t) * kMaxSubBins * kMaxTiles);
+constexpr size_t kOffUnits = align256(kOffItems + sizeof(WorkItem) * kMaxItems);
+constexpr size_t kOffNitems = align256(kOffUnits + sizeof(WorkItem) * kMaxUnits);
+constexpr size_t kOffCounter = align256(kOffNitems + 2 * sizeof(int32_t));
+// the gridder's copy of the tap table; callers with larger ones get the
+// kernels that read theirs directly
+constexpr size_t kTablesBytes = (size_t)4 << 20;
+constexpr size_t kOffTables = align256(kOffCounter + 2 * sizeof(int32_t));
+constexpr size_t kNoallocBytes = align256(kOffTables + kTablesBytes);
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
@@ -117,7 +124,7 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     if (nvis > kMaxVis)
         return SEPW_ETOOLARGE;
 
-    const DevParams dp = make_dev_params(&tp);
+    DevParams dp = make_dev_params(&tp);
     const int64_t ntiles = (int64_t)dp.ntx * dp.ntx;
     if (ntiles > kMaxTiles)
         return SEPW_ETOOLARGE;
@@ -159,20 +166,32 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     pl.d_perm = (int32_t *)(b + kOffPerm);
     pl.d_drop_list = (int32_t *)(b + kOffDrop);
     pl.d_tile_count = (int32_t *)(b + kOffCount);
-    pl.d_tile_cursor = (int32_t *)(b + kOffCursor);
-    pl.d_bin = (int32_t *)(b + kOffBin);
+    pl.d_blocks = b + kOffBlocks;
+    pl.d_bin_base = b + kOffBin;
     pl.d_items = (WorkItem *)(b + kOffItems);
+    pl.d_units = (WorkItem *)(b + kOffUnits);
     pl.d_nitems = (int32_t *)(b + kOffNitems);
+    pl.d_nunits = pl.d_nitems + 1;
     pl.d_item_counter = (int32_t *)(b + kOffCounter);
-    pl.d_dropped = (unsigned long long *)(b + kOffDropped);
+    pl.d_dropped = (unsigned long long *)pl.d_bin_base;
+    if (plan_block_bytes(ntiles) > kBlocksBytes)
+        return SEPW_ETOOLARGE;
+    pl.unit = plan_unit(dp, nvis, num_sms);
+    const size_t wbytes = window_tables_bytes(dp);
+    pl.window = dp.S != 8 && dp.S != 16 && wbytes > 0 && wbytes <= kTablesBytes;
+    pl.sorted = !pl.window;
+    set_bins(dp, pl.window ? kBinsWindow : kBinsSorted);
+    float *tables = (float *)(b + kOffTables);
+    if (!pl.window && sizeof(float2) * dp.P * dp.OS * (size_t)dp.S > kTablesBytes)
+        tables = nullptr;
 
     cudaStream_t s = (cudaStream_t)stream;
-    if (launch_plan(dp, nvis, u, v, w, pl, s) != cudaSuccess) {
+    if (launch_plan(dp, nvis, u, v, w, pl, num_sms, s) != cudaSuccess) {
         cudaGetLastError();
         return SEPW_ECUDA;
     }
     if (nvis > 0 && launch_grid_tiled(dp, pl, (const float2 *)vis, weight,
-                                      (const float2 *)taps, nullptr, (float2 *)grid, num_sms,
+                                      (const float2 *)taps, tables, (float2 *)grid, num_sms,
                                       s) != cudaSuccess) {
         cudaGetLastError();
         return SEPW_ECUDA;

@@ -66,9 +66,23 @@ __device__ __forceinline__ int meta_dv(int y) { return y >> 13; }
 constexpr int kTiledThreads = 256;
 constexpr int kTiledWarps = kTiledThreads / 32;
 constexpr int kTiledBlocksPerSM = 4;
-// block gridder on dense plans: work units per item (see its work loop)
-constexpr int kGridParts = 8;
-constexpr int kGridPartsMinDensity = 256;  // visibilities per tile
+// The degridders' CTAs take consecutive parts of an item on plans with few
+// items: as many as give each CTA about kDegridParts, none below
+// kDegridMinPart visibilities (the window is loaded once per part).
+constexpr int kDegridParts = 4, kDegridMinPart = 128;
+__device__ __forceinline__ int degrid_parts(int n_items, int chunk)
+{
+    return max(1, min(chunk / kDegridMinPart,
+                      kDegridParts * (int)gridDim.x / max(n_items, 1)));
+}
+// the part `u % parts` of item `u / parts`; false when it is empty
+__device__ __forceinline__ bool take_part(WorkItem &it, int part, int parts)
+{
+    const int len = max(kDegridMinPart, (it.count + parts - 1) / parts);
+    it.start += part * len;
+    it.count = min(len, it.count - part * len);
+    return it.count > 0;
+}
 
 __device__ __forceinline__ int key_ly(int key) { return (key >> 1) >> 6; }
 __device__ __forceinline__ int key_lx(int key) { return (key >> 1) & 63; }
@@ -247,16 +261,19 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled
     const int rg = lane / S, j = lane % S;
     const bool lane_ok = Layout<S>::ALL_LANES || rg < RG;
     const int n_items = *nitems;
+    const int parts = degrid_parts(n_items, p.chunk);
 
     for (;;) {
         __syncthreads();
         if (threadIdx.x == 0)
             s_item = atomicAdd(counter, 1);
         __syncthreads();
-        const int item = s_item;
+        const int item = s_item / parts;
         if (item >= n_items)
             break;
-        const WorkItem it = items[item];
+        WorkItem it = items[item];
+        if (!take_part(it, s_item - item * parts, parts))
+            continue;
         const TileOrigin o = tile_origin(p, it.tile);
         for (int rr = warp; rr < W; rr += kTiledWarps) {
             const int64_t gy = o.gy0 + rr;
@@ -437,6 +454,7 @@ __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block
     const unsigned ocol = (unsigned)cg;
     const unsigned orow = (unsigned)(p.voff + rg);
     const int n_items = *nitems;
+    const int parts = degrid_parts(n_items, p.chunk);
     // this lane's first window cell relative to the footprint origin
     const float2 *const lwin = win + rg * WP + cg;
 
@@ -445,10 +463,12 @@ __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block
         if (threadIdx.x == 0)
             s_item = atomicAdd(counter, 1);
         __syncthreads();
-        const int item = s_item;
+        const int item = s_item / parts;
         if (item >= n_items)
             break;
-        const WorkItem it = items[item];
+        WorkItem it = items[item];
+        if (!take_part(it, s_item - item * parts, parts))
+            continue;
         if (!work_item_ok(p, it))
             continue;  // checked build only (uniform over the CTA)
         const TileOrigin o = tile_origin(p, it.tile);
@@ -600,11 +620,10 @@ constexpr int kGridBlkPerSM = 5;
 
 template <int S, bool PLANAR>
 __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block_kernel(
-    DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
+    DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
     int32_t *counter, const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
     const float2 *__restrict__ vis, const float *__restrict__ weight,
-    const float2 *__restrict__ taps, const float *__restrict__ planar, float2 *grid,
-    int parts)
+    const float2 *__restrict__ taps, const float *__restrict__ planar, float2 *grid)
 {
     constexpr int RB = Blk2<S>::RB, RP = Blk2<S>::RP, CB = Blk2<S>::CB;
     constexpr bool FULL = Blk2<S>::FULL;
@@ -620,30 +639,17 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
     const float2 *const tcol = taps + cg;
     const float2 *const trow = taps + p.voff + rg;
     const float *const prow = PLANAR ? planar + 2 * p.voff + RB * rg : nullptr;
-    const int n_items = *nitems;
+    const int n_units = *nunits;
 
-    for (;;) {
-        // a warp takes one of `parts` consecutive parts of an item: on dense
-        // plans whole 2048-visibility items per warp left the end of the
-        // launch to few warps (parts: 1 -> 2.38 ms, 2 -> 2.24, 4 -> 2.16,
-        // 8 -> 2.13, 16 -> 2.14 on 32M visibilities; runs break only at part
-        // edges).  Sparse plans (many small items) keep parts = 1: split
-        // units there only add atomics on the one counter.
-        int unit = 0;
-        if (lane == 0)
-            unit = atomicAdd(counter, 1);
-        unit = __shfl_sync(0xffffffffu, unit, 0);
-        const int item = unit / parts, part = unit % parts;
-        if (item >= n_items)
-            break;
-        const WorkItem it = items[item];
+    // the first unit by the warp's number, the others from the counter
+    const int n_warps = gridDim.x * kTiledWarps;
+    for (int unit = blockIdx.x * kTiledWarps + warp, next; unit < n_units; unit = next) {
+        next = lane == 0 ? atomicAdd(counter, 1) : 0;
+        next = n_warps + __shfl_sync(0xffffffffu, next, 0);
+        const WorkItem it = units[unit];
         if (!work_item_ok(p, it))
             continue;  // checked build only
-        const int len = (it.count + parts - 1) / parts;
-        const int b0 = it.start + part * len;
-        const int b1 = min(it.start + it.count, b0 + len);
-        if (b0 >= b1)
-            continue;
+        const int b0 = it.start, b1 = it.start + it.count;
         const TileOrigin o = tile_origin(p, it.tile);
         float2 *const tgrid = grid + o.base + (o.gy0 + rg) * p.N + o.gx0 + cg;
 
@@ -848,9 +854,6 @@ static cudaError_t launch_grid_S(const DevParams &p, const Plan &plan, const flo
         return e;
     if constexpr (Blk2<S>::OK) {
         const unsigned nb = (unsigned)(num_sms * kGridBlkPerSM);
-        const int parts =
-            p.grid_parts > 0 ? p.grid_parts
-            : plan.nvis >= (int64_t)kGridPartsMinDensity * plan.ntiles ? kGridParts : 1;
         if (planar) {  // rebuilt per call: the caller's table may have changed
             const int64_t n = (p.facet ? 2 : 1) * (int64_t)p.P * p.OS * S;
             if ((e = launch_planar_taps(taps, planar, n, S, s)) != cudaSuccess)
@@ -858,12 +861,12 @@ static cudaError_t launch_grid_S(const DevParams &p, const Plan &plan, const flo
         }
         if (planar)
             grid_tiled_block_kernel<S, true><<<nb, kTiledThreads, 0, s>>>(
-                p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec, plan.d_perm,
-                vis, weight, taps, planar, grid, parts);
+                p, plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm,
+                vis, weight, taps, planar, grid);
         else
             grid_tiled_block_kernel<S, false><<<nb, kTiledThreads, 0, s>>>(
-                p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec, plan.d_perm,
-                vis, weight, taps, nullptr, grid, parts);
+                p, plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm,
+                vis, weight, taps, nullptr, grid);
     } else
         grid_tiled_kernel<S><<<num_sms * kTiledBlocksPerSM, kTiledThreads, 0, s>>>(
             p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec, plan.d_perm, vis,
@@ -917,6 +920,8 @@ cudaError_t launch_grid_tiled(const DevParams &p0, const Plan &plan, const float
                               float2 *grid, int num_sms, cudaStream_t s)
 {
     const DevParams p = with_plan_bounds(p0, plan);
+    if (plan.window)
+        return launch_grid_window(p, plan, vis, weight, taps, planar, grid, num_sms, s);
     switch (p.S) {
 #define X(SS) \
     case SS: return launch_grid_S<SS>(p, plan, vis, weight, taps, planar, grid, num_sms, s);
