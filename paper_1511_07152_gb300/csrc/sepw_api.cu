@@ -46,7 +46,7 @@ struct sepw_ctx {
     // the block gridder's planar copy (two tables in facet mode) or the
     // window gridder's padded ones
     float *d_planar = nullptr;
-    bool window = false;  // the tiled form grids with the window gridder
+    bool window = false;  // the tiled form can grid with the window gridder
     Plan plan;
     cufftHandle fft = 0;
     bool fft_ready = false;
@@ -225,7 +225,8 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     const int ntiles = (int)ntiles64;
     // the window gridder's bins unless their ids (tile * nsub + bin) leave int32
     const bool sorts = ctx->p.form == SEPW_FORM_TILED || ctx->p.form == SEPW_FORM_TC_TF32;
-    set_bins(ctx->dp, ctx->window ? kBinsWindow : sorts ? kBinsSorted : kBinsTile);
+    const bool window = ctx->window && plan_window(ctx->dp, nvis, ngrids);
+    set_bins(ctx->dp, window ? kBinsWindow : sorts ? kBinsSorted : kBinsTile);
     if (ntiles64 * ctx->dp.nsub > INT32_MAX)
         set_bins(ctx->dp, kBinsSorted);
     if (ntiles64 * ctx->dp.nsub > INT32_MAX)
@@ -274,9 +275,11 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
             return rc;
         pl.items_capacity = (int32_t)items;
     }
-    pl.unit = plan_unit(ctx->dp, nvis, ctx->num_sms);
+    pl.nvis = nvis;
+    pl.window = ctx->dp.sub_log2 == 2;  // kBinsWindow
+    set_units(ctx->dp, ctx->num_sms, pl);
     if (ctx->p.form == SEPW_FORM_TILED) {
-        const int64_t units = (int64_t)ntiles + nvis / pl.unit + 1;
+        const int64_t units = max_units(pl);
         if (units > INT32_MAX)
             return fail(ctx, SEPW_EINVAL, "too many work units");
         if (pl.units_capacity < units) {
@@ -286,20 +289,12 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
             pl.units_capacity = (int32_t)units;
         }
     }
-    pl.window = ctx->dp.sub_log2 == 2;  // kBinsWindow
     // for the kernels that walk runs of one origin: the tiled form's block and
     // column gridders, and the tiled degridder of the TF32 form
     pl.sorted = sorts && !pl.window;
     return SEPW_OK;
 }
 
-// The tiled form's gridder: the block gridder for S = 8 and 16, whose plans
-// are sorted by origin, and the window gridder for the other supports where
-// its tables can be had.
-bool use_window(const DevParams &p)
-{
-    return p.S != 8 && p.S != 16 && window_tables_bytes(p) > 0;
-}
 
 }  // namespace
 
@@ -386,7 +381,7 @@ int sepw_create(sepw_ctx **out, const sepw_params *p)
         return SEPW_ECUDA;
     }
     const int N = p->grid_size;
-    ctx->window = p->form == SEPW_FORM_TILED && use_window(ctx->dp);
+    ctx->window = p->form == SEPW_FORM_TILED && window_tables_bytes(ctx->dp) > 0;
     if ((rc = grow(ctx, &ctx->d_taper64, N)) || (rc = grow(ctx, &ctx->d_taper32, N)) ||
         (rc = grow(ctx, &ctx->d_tw, (size_t)N * p->oversample)) ||
         (rc = grow(ctx, &ctx->d_status, 1)) ||
@@ -943,6 +938,22 @@ static int residual_pass_check(sepw_ctx *ctx, int32_t Sr, int32_t OSr, const flo
     return check_dev(ctx, table, "table", false);
 }
 
+// Sorts the items of a plan made without it before the first correction pass,
+// whose kernels walk runs of one origin, if there is a visibility per four
+// cells to make runs (2M visibilities on 1024^2 at S = 12: step 1366 -> 513
+// us).  The order inside a bin is free, so every other kernel can use the plan
+// as before.  (The tiled degridder did not gain by it: 1440 us either way for
+// a step of 8M at S = 12.)
+static int sort_for_runs(sepw_ctx *ctx, cudaStream_t s)
+{
+    Plan &pl = ctx->plan;
+    if (pl.sorted || 4 * pl.nvis < (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N)
+        return SEPW_OK;
+    SEPW_CUDA(ctx, launch_item_sort(ctx->dp, pl, ctx->num_sms, s));
+    pl.sorted = true;
+    return SEPW_OK;
+}
+
 int sepw_grid_residual_planned(sepw_ctx *ctx, int32_t support_r, int32_t oversample_r,
                                const float *table, const float *vis, const float *weight,
                                float *grid, sepw_stream_t stream)
@@ -957,6 +968,8 @@ int sepw_grid_residual_planned(sepw_ctx *ctx, int32_t support_r, int32_t oversam
     if (ctx->plan.nvis == 0)
         return SEPW_OK;
     if ((rc = check_dev(ctx, vis, "vis", false)) || (rc = check_dev(ctx, weight, "weight", true)))
+        return rc;
+    if ((rc = sort_for_runs(ctx, (cudaStream_t)stream)))
         return rc;
     SEPW_CUDA(ctx, launch_grid_residual(ctx->dp, support_r, oversample_r, ctx->plan,
                                         (const float2 *)vis, weight, (const float2 *)table,
@@ -979,6 +992,8 @@ int sepw_degrid_residual_planned(sepw_ctx *ctx, int32_t support_r, int32_t overs
         return SEPW_OK;
     if ((rc = check_dev(ctx, vis_out, "vis_out", false)) ||
         (rc = check_dev(ctx, weight, "weight", true)))
+        return rc;
+    if ((rc = sort_for_runs(ctx, (cudaStream_t)stream)))
         return rc;
     SEPW_CUDA(ctx, launch_degrid_residual(ctx->dp, support_r, oversample_r, ctx->plan,
                                           (const float2 *)grid, weight, (const float2 *)table,

@@ -104,10 +104,19 @@ __device__ __forceinline__ Totals operator-(const Totals &a, const Totals &b)
     return {a.n - b.n, a.full_items - b.full_items, a.part_items - b.part_items,
             a.full_units - b.full_units, a.part_units - b.part_units};
 }
-__device__ __forceinline__ Totals tile_totals(int n, int chunk, int unit)
+// How tiles are cut: items of `chunk`; units of a `parts`-th of the tile, at
+// most `unit` and a multiple of 32 (all of them `unit` when parts is 1).
+struct Cut {
+    int32_t chunk, unit, parts;
+    __device__ __forceinline__ int unit_of(int n) const
+    {
+        return parts > 1 ? max(32, min(unit, (n / parts + 31) & ~31)) : unit;
+    }
+};
+__device__ __forceinline__ Totals tile_totals(int n, const Cut &cut)
 {
-    const int fi = n / chunk, fu = n / unit;
-    return {n, fi, n != fi * chunk, fu, n != fu * unit};
+    const int u = cut.unit_of(n), fi = n / cut.chunk, fu = n / u;
+    return {n, fi, n != fi * cut.chunk, fu, n != fu * u};
 }
 __device__ __forceinline__ Totals shfl_up(const Totals &v, int d)
 {
@@ -161,7 +170,7 @@ static int plan_block(int64_t ntiles, int nsub)
 constexpr int kPlanThreads = 1024, kPlanWarps = kPlanThreads / 32;
 
 __global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
-    int32_t ntiles, int32_t tb, int32_t nsub, int32_t chunk, int32_t unit,
+    int32_t ntiles, int32_t tb, int32_t nsub, Cut cut,
     const int32_t *__restrict__ bin, int32_t *__restrict__ tile_count,
     Totals *__restrict__ blocks, unsigned *ticket)
 {
@@ -198,7 +207,7 @@ __global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
     if ((int)threadIdx.x < tb && t0 + (int)threadIdx.x < ntiles)
         tile_count[t0 + threadIdx.x] = n;
     Totals total;
-    block_scan(tile_totals(n, chunk, unit), s_warps, total);
+    block_scan(tile_totals(n, cut), s_warps, total);
     if (threadIdx.x == 0) {
         blocks[blockIdx.x] = total;
         __threadfence();
@@ -228,11 +237,12 @@ __global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
         blocks[nb] = run;
 }
 
-// Lists the full pieces of size `size` of the block's tb tiles (tile tile0 +
-// k: those from piece pre[k] on, the first at slot first[k]; total pieces),
+// Lists the full pieces of the block's tb tiles (tile tile0 + k: those from
+// piece pre[k] on, of size_of(k), the first at slot first[k]; total pieces),
 // consecutive threads writing consecutive pieces.
+template <typename F>
 __device__ __forceinline__ void list_full(WorkItem *__restrict__ out, int tile0, int tb,
-                                          int total, int size, const int32_t *pre,
+                                          int total, F size_of, const int32_t *pre,
                                           const int32_t *first)
 {
     for (int e = threadIdx.x; e < total; e += kPlanThreads) {
@@ -240,13 +250,14 @@ __device__ __forceinline__ void list_full(WorkItem *__restrict__ out, int tile0,
         for (int h = tb >> 1; h > 0; h >>= 1)
             if (pre[k + h] <= e)
                 k += h;
+        const int size = size_of(k);
         out[e] = {tile0 + k, first[k] + (e - pre[k]) * size, size, 0};
     }
 }
 
 // Pass 2: every bin's count replaced by its first slot; items and units.
 __global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
-    int32_t ntiles, int32_t tb, int32_t nsub, int32_t chunk, int32_t unit,
+    int32_t ntiles, int32_t tb, int32_t nsub, Cut cut,
     const int32_t *__restrict__ tile_count, const Totals *__restrict__ blocks,
     int32_t *__restrict__ bin, WorkItem *__restrict__ items, int32_t *nitems,
     WorkItem *__restrict__ units, int32_t *nunits)
@@ -256,7 +267,8 @@ __global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t0 = blockIdx.x * tb, t = t0 + threadIdx.x;
     const int n = (int)threadIdx.x < tb && t < ntiles ? tile_count[t] : 0;
-    const Totals mine = tile_totals(n, chunk, unit);
+    const Totals mine = tile_totals(n, cut);
+    const int chunk = cut.chunk, unit = cut.unit_of(n);
     Totals sum;
     const Totals before = blocks[blockIdx.x];  // exclusive prefix of the block
     const Totals in = block_scan(mine, s_warps, sum) - mine, at = before + in;
@@ -279,9 +291,11 @@ __global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
                                                      n - mine.full_units * unit, 0};
     }
     __syncthreads();
-    list_full(items + before.full_items, t0, tb, sum.full_items, chunk, s_items, s_at);
+    list_full(items + before.full_items, t0, tb, sum.full_items, [&](int) { return chunk; },
+              s_items, s_at);
     if (units)
-        list_full(units + before.full_units, t0, tb, sum.full_units, unit, s_units, s_at);
+        list_full(units + before.full_units, t0, tb, sum.full_units,
+                  [&](int k) { return cut.unit_of(s_n[k]); }, s_units, s_at);
     if (nsub <= 4) {  // a thread per tile
         if ((int)threadIdx.x < tb && n > 0) {
             int32_t *b = bin + (int64_t)t * nsub;
@@ -351,7 +365,13 @@ constexpr int kMaxBinsPerThread = kMaxSortBins / kSortThreads;
 __device__ __forceinline__ int sort_key(uint64_t r, const DevParams &p)
 {
     const int lx = rec_lx(r), ly = rec_ly(r), lg = p.sub_log2, m = (1 << lg) - 1;
-    return (sub_bin(lx, ly, rec_conj(r), p) << lg | (ly & m)) << lg | (lx & m);
+    const int k = (sub_bin(lx, ly, rec_conj(r), p) << lg | (ly & m)) << lg | (lx & m);
+    return p.sub_conj ? k : k << 1 | (rec_conj(r) ? 1 : 0);
+}
+// keys of a tile: at most 2 x 64 x 64
+static int sort_keys(const DevParams &p)
+{
+    return p.nsub << (2 * p.sub_log2 + (p.sub_conj ? 0 : 1));
 }
 
 __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
@@ -368,7 +388,7 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     const WorkItem it = items[item];
     const int n = it.count;
-    const int nb = p.nsub << (2 * p.sub_log2);
+    const int nb = p.nsub << (2 * p.sub_log2 + (p.sub_conj ? 0 : 1));
     const int per = (nb + kSortThreads - 1) / kSortThreads;
     for (int b = threadIdx.x; b < per * kSortThreads; b += kSortThreads)
         hist[b] = 0;
@@ -475,19 +495,50 @@ cudaError_t launch_zero_dropped(const Plan &plan, float2 *vis, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// Visibilities in a unit of the tiled gridders: about eight units for each of
-// the ~40 warps an SM holds, 32 to 256.  Whole items of 2048 gave 524,288
-// visibilities to 400 warps (S = 16, 758 us; 155 us now); 4M visibilities at
-// S = 8: 190 us with two units per warp, 178 us with eight.  Above 256 the
-// last warps work alone on 32M visibilities (2.13 ms for 256, 2.16 for 512,
-// 2.24 for 1024, 2.38 for 2048); below, sparse tiles fall into more units
-// (128 grids at S = 12: 8.97 ms for 256, 9.55 for 128).
-int32_t plan_unit(const DevParams &p, int64_t nvis, int num_sms)
+// The units of the tiled gridders: 32 to 256 visibilities, about two for each
+// of the ~40 warps an SM holds; for the block gridders also an eighth of their
+// tile, as long as that does not make more units than those warps can use
+// (sparse tiles then weigh as little as dense ones at the end of the launch,
+// and dense ones keep their runs).  Whole items of 2048 gave 524,288
+// visibilities to 400 warps (S = 16, 758 us; 155 us so).  Above 256 the last
+// warps work alone on 32M visibilities (2.13 ms for 256, 2.16 for 512, 2.24
+// for 1024, 2.38 for 2048); the window gridder adds whole windows at the ends
+// of a unit (128 grids at S = 12: 8.97 ms for 256, 9.55 for 128).
+void set_units(const DevParams &p, int num_sms, Plan &plan)
 {
-    if (p.grid_parts > 0)
-        return std::max(32, ((p.chunk + p.grid_parts - 1) / p.grid_parts + 31) & ~31);
-    const int64_t u = (nvis / std::max(1, 320 * num_sms) + 31) & ~31ll;
-    return (int32_t)std::min<int64_t>(256, std::max<int64_t>(32, u));
+    plan.unit_parts = 1;
+    if (p.grid_parts > 0) {
+        plan.unit = std::max(32, ((p.chunk + p.grid_parts - 1) / p.grid_parts + 31) & ~31);
+        return;
+    }
+    const int64_t per = plan.window ? 320 : 80;
+    const int64_t u = (plan.nvis / std::max<int64_t>(1, per * num_sms) + 31) & ~31ll;
+    plan.unit = (int32_t)std::min<int64_t>(256, std::max<int64_t>(32, u));
+    if (!plan.window)
+        plan.unit_parts = (int32_t)std::min<int64_t>(
+            8, std::max<int64_t>(1, 640ll * num_sms / std::max(1, plan.ntiles)));
+}
+
+// units of any plan that set_units cuts: a full one takes unit visibilities or
+// more than a ninth of its tile
+int64_t max_units(const Plan &plan)
+{
+    const int64_t cut = plan.nvis / (plan.unit_parts > 1 ? 32 : plan.unit);
+    return std::min(cut, plan.nvis / plan.unit + (int64_t)plan.unit_parts * plan.ntiles) +
+           plan.ntiles + 1;
+}
+
+// Whether the tiled form grids with the window gridder (where its tables can
+// be had): every support without a block gridder, and S = 16 below a
+// visibility per four cells, where runs of one origin are short (524,288
+// visibilities on 2048^2: 155 us with the block gridder, 86 us with the window
+// gridder; 4M: 355 and 468 us).  At S = 8 the block gridder is the faster one (1M on 1024^2: 62 and
+// 74 us; 8M on 15 x 4096^2: 475 and 556 us).
+bool plan_window(const DevParams &p, int64_t nvis, int ngrids)
+{
+    if (p.S == 16)
+        return 4 * nvis < (int64_t)ngrids * p.N * p.N;
+    return p.S != 8;
 }
 
 size_t plan_bin_bytes(int64_t ntiles, const DevParams &p)
@@ -519,14 +570,15 @@ cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
     }
     const int tb = plan_block(plan.ntiles, p.nsub), nblk = (plan.ntiles + tb - 1) / tb;
     Totals *const blocks = (Totals *)plan.d_blocks;
-    tile_count_kernel<<<nblk, kPlanThreads, 0, s>>>(plan.ntiles, tb, p.nsub, p.chunk, plan.unit, bin,
-                                          plan.d_tile_count, blocks,
-                                          (unsigned *)(plan.d_bin_base + kBinTicket));
+    const Cut cut{p.chunk, plan.unit, plan.unit_parts};
+    tile_count_kernel<<<nblk, kPlanThreads, 0, s>>>(
+        plan.ntiles, tb, p.nsub, cut, bin, plan.d_tile_count, blocks,
+        (unsigned *)(plan.d_bin_base + kBinTicket));
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
-    tile_items_kernel<<<nblk, kPlanThreads, 0, s>>>(plan.ntiles, tb, p.nsub, p.chunk, plan.unit,
-                                          plan.d_tile_count, blocks, bin, plan.d_items,
-                                          plan.d_nitems, plan.d_units, plan.d_nunits);
+    tile_items_kernel<<<nblk, kPlanThreads, 0, s>>>(
+        plan.ntiles, tb, p.nsub, cut, plan.d_tile_count, blocks, bin, plan.d_items, plan.d_nitems,
+        plan.d_units, plan.d_nunits);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     if (nvis > 0) {
@@ -534,25 +586,27 @@ cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
             nvis, plan.d_tile, plan.d_rank, plan.d_rec0, bin, plan.d_perm, plan.d_rec);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
-        // the per-item sort by (block, origin, conj) serves the kernels that
-        // walk runs of one origin; the 16-bit tensor-core forms and the
-        // window gridder take any order within a block and skip it
-        if (!plan.sorted)
-            return cudaSuccess;
-        const int nb = p.nsub << (2 * p.sub_log2);
-        const size_t shm =
-            sizeof(int32_t) * kSortThreads * ((nb + kSortThreads - 1) / kSortThreads);
-        e = cudaFuncSetAttribute(item_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)shm);
-        if (e != cudaSuccess)
-            return e;
-        const int nblk = std::max(1, std::min(plan.items_capacity, 16 * num_sms));
-        item_sort_kernel<<<nblk, kSortThreads, shm, s>>>(p, plan.d_items, plan.d_nitems,
-                                                         plan.d_perm, plan.d_rec);
-        if ((e = cudaGetLastError()) != cudaSuccess)
-            return e;
+        if (plan.sorted)
+            return launch_item_sort(p, plan, num_sms, s);
     }
     return cudaSuccess;
+}
+
+// The per-item sort serves the kernels that walk runs of one origin; the
+// 16-bit tensor-core forms and the window gridder take any order within a bin
+// and leave it out until a call that gains by it (sort_for_runs).
+cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, cudaStream_t s)
+{
+    const int nb = sort_keys(p);
+    const size_t shm = sizeof(int32_t) * kSortThreads * ((nb + kSortThreads - 1) / kSortThreads);
+    cudaError_t e = cudaFuncSetAttribute(item_sort_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+    if (e != cudaSuccess)
+        return e;
+    const int nblk = std::max(1, std::min(plan.items_capacity, 16 * num_sms));
+    item_sort_kernel<<<nblk, kSortThreads, shm, s>>>(p, plan.d_items, plan.d_nitems, plan.d_perm,
+                                                     plan.d_rec);
+    return cudaGetLastError();
 }
 
 }  // namespace sepw

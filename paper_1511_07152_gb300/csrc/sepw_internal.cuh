@@ -385,7 +385,8 @@ struct Plan {
     size_t bins_capacity = 0;   // bytes at d_bin_base
     int32_t items_capacity = 0;
     int32_t units_capacity = 0;
-    int32_t unit = 256;         // visibilities per unit
+    int32_t unit = 256;         // most visibilities per unit
+    int32_t unit_parts = 1;     // units are at most this part of their tile
     bool valid = false;
     bool sorted = true;         // items sorted by (block, origin, conj)
     bool window = false;        // gridding by the window gridder
@@ -445,13 +446,16 @@ cudaError_t launch_degrid_plain(const DevParams &p, int64_t nvis, const double *
                                 unsigned long long *dropped, cudaStream_t s);
 
 // sepw_bin.cu
-// sizes of Plan::d_bin_base and Plan::d_blocks, and the unit for nvis
+// sizes of Plan::d_bin_base and Plan::d_blocks, and the units
 size_t plan_bin_bytes(int64_t ntiles, const DevParams &p);
 size_t plan_block_bytes(int64_t ntiles);
-int32_t plan_unit(const DevParams &p, int64_t nvis, int num_sms);
+void set_units(const DevParams &p, int num_sms, Plan &plan);  // from nvis, ntiles, window
+int64_t max_units(const Plan &plan);
+bool plan_window(const DevParams &p, int64_t nvis, int ngrids);
 cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
                         const double *v, const double *w, Plan &plan, int num_sms,
                         cudaStream_t s);
+cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, cudaStream_t s);
 // batched: plan.ngrids > 1 and plan.d_offsets hold the per-grid ranges
 cudaError_t launch_zero_dropped(const Plan &plan, float2 *vis, cudaStream_t s);
 

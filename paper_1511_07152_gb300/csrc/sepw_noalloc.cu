@@ -176,10 +176,10 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     pl.d_dropped = (unsigned long long *)pl.d_bin_base;
     if (plan_block_bytes(ntiles) > kBlocksBytes)
         return SEPW_ETOOLARGE;
-    pl.unit = plan_unit(dp, nvis, num_sms);
     const size_t wbytes = window_tables_bytes(dp);
-    pl.window = dp.S != 8 && dp.S != 16 && wbytes > 0 && wbytes <= kTablesBytes;
+    pl.window = wbytes > 0 && wbytes <= kTablesBytes && plan_window(dp, nvis, 1);
     pl.sorted = !pl.window;
+    set_units(dp, num_sms, pl);
     set_bins(dp, pl.window ? kBinsWindow : kBinsSorted);
     float *tables = (float *)(b + kOffTables);
     if (!pl.window && sizeof(float2) * dp.P * dp.OS * (size_t)dp.S > kTablesBytes)

@@ -641,11 +641,15 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
     const float *const prow = PLANAR ? planar + 2 * p.voff + RB * rg : nullptr;
     const int n_units = *nunits;
 
-    // the first unit by the warp's number, the others from the counter
+    // the first unit by the warp's number, neighbours (which add to the same
+    // cells) on different SMs; the others from the counter, taken when the
+    // warp is free: claimed ahead they would wait for a busy one
     const int n_warps = gridDim.x * kTiledWarps;
-    for (int unit = blockIdx.x * kTiledWarps + warp, next; unit < n_units; unit = next) {
-        next = lane == 0 ? atomicAdd(counter, 1) : 0;
-        next = n_warps + __shfl_sync(0xffffffffu, next, 0);
+    auto next_unit = [&]() {
+        const int k = lane == 0 ? atomicAdd(counter, 1) : 0;
+        return n_warps + __shfl_sync(0xffffffffu, k, 0);
+    };
+    for (int unit = warp * gridDim.x + blockIdx.x; unit < n_units; unit = next_unit()) {
         const WorkItem it = units[unit];
         if (!work_item_ok(p, it))
             continue;  // checked build only

@@ -141,6 +141,39 @@ def test_non_finite_values_stay_in_their_footprints(env, support):
     assert rel_l2(got[1][ok], got[0][ok]) <= TOL
 
 
+@pytest.mark.parametrize("support,nvis", [(16, 4095), (16, 4097), (12, 4097)])
+def test_correction_after_an_unsorted_plan(env, support, nvis):
+    """The sort that the correction passes add to a plan made without it (dense
+    enough or not), and the separable kernels on that plan before and after;
+    S = 16 on both sides of the window gridder's density."""
+    torch, S = env
+    wl = synth.random_case(345, nvis, 128, support, 4, 3)
+    p = O.params_from(wl.params())
+    T, loc = O.taps(p), O.locate(p, wl.u, wl.v, wl.w)
+    ctx = S.sepw_create(S.make_params(**wl.params(), form=S.FORM_TILED))
+    taps = S.sepw_make_taps(ctx)
+    d = _dev(torch, wl)
+    rng = np.random.default_rng(7)
+    R = (rng.standard_normal((p.P, 2, 2, 8, 8)) + 1j * rng.standard_normal((p.P, 2, 2, 8, 8)))
+    table = torch.from_numpy(R.astype(np.complex64)).cuda()
+    S.sepw_plan(ctx, d["u"], d["v"], d["w"])
+    grid = torch.zeros((p.N, p.N), dtype=torch.complex64, device="cuda")
+    out = torch.zeros(nvis, dtype=torch.complex64, device="cuda")
+    S.sepw_grid_residual_planned(ctx, table, d["vis"], d["weight"], grid)
+    want = O.grid_residual(p, loc, wl.vis, wl.weight, R.astype(np.complex64))
+    assert rel_l2(grid.cpu().numpy(), want) <= TOL
+    model = grid.clone()
+    S.sepw_degrid_residual_planned(ctx, table, model, d["weight"], out)
+    host = model.cpu().numpy()
+    assert rel_l2(out.cpu().numpy(), O.degrid_residual(p, loc, host, wl.weight,
+                                                       R.astype(np.complex64))) <= TOL
+    grid.zero_()
+    S.sepw_grid_planned(ctx, taps, d["vis"], d["weight"], grid)
+    assert rel_l2(grid.cpu().numpy(), O.grid_separable(p, loc, wl.vis, wl.weight, T)) <= TOL
+    S.sepw_degrid_planned(ctx, taps, model, d["weight"], out)
+    assert rel_l2(out.cpu().numpy(), O.degrid_separable(p, loc, host, wl.weight, T)) <= TOL
+
+
 def test_facet_tables(env):
     """Separate u and v tables (the v taps come from the second one)."""
     torch, S = env
