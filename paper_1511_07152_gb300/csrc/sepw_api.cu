@@ -50,6 +50,9 @@ struct sepw_ctx {
     Plan plan;
     cufftHandle fft = 0;
     bool fft_ready = false;
+    cufftHandle fft_cols = 0;  // N column transforms, where the rows are ours
+    bool cols_ready = false;
+    float2 *d_rows_tab = nullptr;  // twiddles of our row transforms (cols_ready)
     // hybrid W stacking: slice centres of the last sepw_wstack_plan and the
     // workspace of the slice sort
     std::vector<double> ws_centres;
@@ -417,6 +420,8 @@ void sepw_destroy(sepw_ctx *ctx)
     cudaDeviceSynchronize();
     if (ctx->fft_ready)
         cufftDestroy(ctx->fft);
+    if (ctx->cols_ready)
+        cufftDestroy(ctx->fft_cols);
     if (ctx->fft_batch_n)
         cufftDestroy(ctx->fft_batch);
     cudaFree(ctx->d_ws_c64);
@@ -432,6 +437,7 @@ void sepw_destroy(sepw_ctx *ctx)
     cudaFree(ctx->d_tw);
     cudaFree(ctx->d_status);
     cudaFree(ctx->d_planar);
+    cudaFree(ctx->d_rows_tab);
     cudaFree(ctx->d_tc2);
     free_plan(ctx->plan);
     cudaSetDevice(cur);
@@ -816,6 +822,49 @@ int sepw_test_stall_mma(sepw_ctx *ctx, int enable)
     return SEPW_OK;
 }
 
+// The context's 2-D transform, on stream s
+static int ensure_fft(sepw_ctx *ctx, cudaStream_t s)
+{
+    if (!ctx->fft_ready) {
+        const cufftResult r =
+            cufftPlan2d(&ctx->fft, ctx->p.grid_size, ctx->p.grid_size, CUFFT_C2C);
+        if (r != CUFFT_SUCCESS)
+            return fail(ctx, SEPW_ECUDA, "cufftPlan2d failed (%d)", (int)r);
+        ctx->fft_ready = true;
+    }
+    if (cufftSetStream(ctx->fft, s) != CUFFT_SUCCESS)
+        return fail(ctx, SEPW_ECUDA, "cufftSetStream failed");
+    return SEPW_OK;
+}
+
+// The column transforms of one grid, on stream s, and the rows' twiddles
+static int ensure_cols(sepw_ctx *ctx, cudaStream_t s)
+{
+    if (!ctx->cols_ready) {
+        int n = ctx->p.grid_size, rc;
+        if (!ctx->d_rows_tab &&
+            (rc = grow(ctx, &ctx->d_rows_tab, rows_table_bytes(n) / sizeof(float2))))
+            return rc;
+        SEPW_CUDA(ctx, launch_rows_tables(ctx->dp, ctx->d_tw, ctx->d_rows_tab, s));
+        // later calls may come on other streams
+        SEPW_CUDA(ctx, cudaStreamSynchronize(s));
+        const cufftResult r =
+            cufftPlanMany(&ctx->fft_cols, 1, &n, &n, n, 1, &n, n, 1, CUFFT_C2C, n);
+        if (r != CUFFT_SUCCESS)
+            return fail(ctx, SEPW_ECUDA, "cufftPlanMany (columns) failed (%d)", (int)r);
+        ctx->cols_ready = true;
+    }
+    if (cufftSetStream(ctx->fft_cols, s) != CUFFT_SUCCESS)
+        return fail(ctx, SEPW_ECUDA, "cufftSetStream failed");
+    return SEPW_OK;
+}
+
+static int fft_exec(sepw_ctx *ctx, cufftHandle fft, float2 *g, int direction)
+{
+    const cufftResult r = cufftExecC2C(fft, (cufftComplex *)g, (cufftComplex *)g, direction);
+    return r == CUFFT_SUCCESS ? SEPW_OK : fail(ctx, SEPW_ECUDA, "cufftExecC2C failed (%d)", (int)r);
+}
+
 int sepw_image(sepw_ctx *ctx, int direction, float *buf, sepw_stream_t stream)
 {
     Range range_("sepw_image");
@@ -828,20 +877,20 @@ int sepw_image(sepw_ctx *ctx, int direction, float *buf, sepw_stream_t stream)
     if (rc)
         return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    if (!ctx->fft_ready) {
-        cufftResult r = cufftPlan2d(&ctx->fft, ctx->p.grid_size, ctx->p.grid_size, CUFFT_C2C);
-        if (r != CUFFT_SUCCESS)
-            return fail(ctx, SEPW_ECUDA, "cufftPlan2d failed (%d)", (int)r);
-        ctx->fft_ready = true;
+    if (direction != SEPW_IMAGE_TO_GRID && rows_supported(ctx->p.grid_size)) {
+        if ((rc = ensure_cols(ctx, s)) ||
+            (rc = fft_exec(ctx, ctx->fft_cols, (float2 *)buf, CUFFT_INVERSE)))
+            return rc;
+        SEPW_CUDA(ctx, launch_rows_to_image(ctx->dp, direction == SEPW_GRID_TO_IMAGE ? 1 : 2,
+                                            ctx->d_taper32, ctx->d_rows_tab, (float2 *)buf, s));
+        return SEPW_OK;
     }
-    if (cufftSetStream(ctx->fft, s) != CUFFT_SUCCESS)
-        return fail(ctx, SEPW_ECUDA, "cufftSetStream failed");
+    if ((rc = ensure_fft(ctx, s)))
+        return rc;
     SEPW_CUDA(ctx, launch_image_pre(ctx->dp, direction, ctx->d_taper32, (float2 *)buf, s));
-    cufftResult r = cufftExecC2C(ctx->fft, (cufftComplex *)buf, (cufftComplex *)buf,
-                                 direction == SEPW_IMAGE_TO_GRID ? CUFFT_FORWARD
-                                                                 : CUFFT_INVERSE);
-    if (r != CUFFT_SUCCESS)
-        return fail(ctx, SEPW_ECUDA, "cufftExecC2C failed (%d)", (int)r);
+    if ((rc = fft_exec(ctx, ctx->fft, (float2 *)buf,
+                       direction == SEPW_IMAGE_TO_GRID ? CUFFT_FORWARD : CUFFT_INVERSE)))
+        return rc;
     SEPW_CUDA(ctx, launch_image_post(ctx->dp, direction, ctx->d_taper32, (float2 *)buf, s));
     return SEPW_OK;
 }
@@ -1150,6 +1199,17 @@ static int ensure_fft_batch(sepw_ctx *ctx, int L)
     return SEPW_OK;
 }
 
+// W stacking by our row transforms: their sizes, whole 16-byte pieces of the
+// slice grids, and an image apart from them (a row of the image is written
+// while other rows are still to be read).
+static bool wstack_rows(const sepw_ctx *ctx, const float *slice_grids, const float *image)
+{
+    const uintptr_t n2 = sizeof(float2) * ctx->p.grid_size * (uintptr_t)ctx->p.grid_size;
+    const uintptr_t g = (uintptr_t)slice_grids, i = (uintptr_t)image;
+    return rows_supported(ctx->p.grid_size) && (g & 15) == 0 &&
+           (i + n2 <= g || g + n2 * ctx->ws_centres.size() <= i);
+}
+
 int sepw_wstack_image(sepw_ctx *ctx, float *slice_grids, float *image, sepw_stream_t stream)
 {
     Range range_("sepw_wstack_image");
@@ -1162,9 +1222,21 @@ int sepw_wstack_image(sepw_ctx *ctx, float *slice_grids, float *image, sepw_stre
         (rc = check_dev(ctx, image, "image", false)))
         return rc;
     const int L = (int)ctx->ws_centres.size();
+    cudaStream_t s = (cudaStream_t)stream;
+    if (wstack_rows(ctx, slice_grids, image)) {
+        const size_t n2 = (size_t)ctx->p.grid_size * ctx->p.grid_size;
+        if ((rc = ensure_cols(ctx, s)))
+            return rc;
+        for (int c = 0; c < L; ++c)
+            if ((rc = fft_exec(ctx, ctx->fft_cols, (float2 *)slice_grids + c * n2, CUFFT_INVERSE)))
+                return rc;
+        SEPW_CUDA(ctx, launch_slices_to_image(ctx->dp, L, ctx->d_taper32, ctx->d_ws_c32,
+                                              ctx->d_rows_tab, (const float2 *)slice_grids,
+                                              (float2 *)image, s));
+        return SEPW_OK;
+    }
     if ((rc = ensure_fft_batch(ctx, L)))
         return rc;
-    cudaStream_t s = (cudaStream_t)stream;
     if (cufftSetStream(ctx->fft_batch, s) != CUFFT_SUCCESS)
         return fail(ctx, SEPW_ECUDA, "cufftSetStream failed");
     SEPW_CUDA(ctx, launch_wstack_sign(ctx->dp, L, (float2 *)slice_grids, s));
@@ -1190,9 +1262,22 @@ int sepw_wstack_model_grids(sepw_ctx *ctx, const float *image, float *slice_grid
         (rc = check_dev(ctx, image, "image", false)))
         return rc;
     const int L = (int)ctx->ws_centres.size();
+    cudaStream_t s = (cudaStream_t)stream;
+    if (wstack_rows(ctx, slice_grids, image)) {
+        const size_t n2 = (size_t)ctx->p.grid_size * ctx->p.grid_size;
+        if ((rc = ensure_cols(ctx, s)))
+            return rc;
+        SEPW_CUDA(ctx, launch_image_to_slices(ctx->dp, L, ctx->d_taper32, ctx->d_ws_c32,
+                                              ctx->d_rows_tab, (const float2 *)image,
+                                              (float2 *)slice_grids, s));
+        for (int c = 0; c < L; ++c)
+            if ((rc = fft_exec(ctx, ctx->fft_cols, (float2 *)slice_grids + c * n2,
+                               CUFFT_FORWARD)))
+                return rc;
+        return SEPW_OK;
+    }
     if ((rc = ensure_fft_batch(ctx, L)))
         return rc;
-    cudaStream_t s = (cudaStream_t)stream;
     if (cufftSetStream(ctx->fft_batch, s) != CUFFT_SUCCESS)
         return fail(ctx, SEPW_ECUDA, "cufftSetStream failed");
     SEPW_CUDA(ctx, launch_wstack_split(ctx->dp, L, ctx->d_taper32, ctx->d_ws_c32,

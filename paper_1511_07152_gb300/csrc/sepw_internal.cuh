@@ -547,7 +547,24 @@ cudaError_t launch_degrid_residual(const DevParams &p, int Sr, int OSr, const Pl
                                    const float2 *grid, const float *weight, const float2 *res,
                                    float2 *vis_out, int num_sms, cudaStream_t s);
 
-// sepw_image.cu
+// sepw_fft.cu: row transforms with the image side's passes folded in, for the
+// N of rows_supported; column transforms of the grid side run before
+// (to image) or after (to grid).  tab: rows_table_bytes(N) bytes filled by
+// launch_rows_tables.  mode 1: n / (c c), 2: 1 / (n c c).  launch_slices_to_image
+// wants g 16-byte aligned.
+bool rows_supported(int N);
+size_t rows_table_bytes(int N);
+cudaError_t launch_rows_tables(const DevParams &p, const double2 *tw, float2 *tab, cudaStream_t s);
+cudaError_t launch_rows_to_image(const DevParams &p, int mode, const float *taper,
+                                 const float2 *tab, float2 *buf, cudaStream_t s);
+cudaError_t launch_slices_to_image(const DevParams &p, int L, const float *taper, const float *wc,
+                                   const float2 *tab, const float2 *g, float2 *image,
+                                   cudaStream_t s);
+cudaError_t launch_image_to_slices(const DevParams &p, int L, const float *taper, const float *wc,
+                                   const float2 *tab, const float2 *image, float2 *g,
+                                   cudaStream_t s);
+
+// sepw_image.cu (other N, and towards the grid: around a 2-D transform)
 cudaError_t launch_image_pre(const DevParams &p, int direction, const float *taper,
                              float2 *buf, cudaStream_t s);
 cudaError_t launch_image_post(const DevParams &p, int direction, const float *taper,
