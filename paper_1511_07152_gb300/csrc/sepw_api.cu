@@ -279,6 +279,7 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
         pl.items_capacity = (int32_t)items;
     }
     pl.nvis = nvis;
+    ctx->dp.early = nvis <= kEarlyVis ? 1 : 0;
     pl.window = ctx->dp.sub_log2 == 2;  // kBinsWindow
     set_units(ctx->dp, ctx->num_sms, pl);
     if (ctx->p.form == SEPW_FORM_TILED) {
@@ -298,6 +299,26 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     return SEPW_OK;
 }
 
+
+// Runs a gridding or degridding call on the plan just made and copies the
+// plan's dropped count to n_dropped (device, may be NULL): the tiled form's
+// launches write it on their way, the others leave it to a copy.
+template <typename F>
+int with_dropped(sepw_ctx *ctx, int64_t *n_dropped, cudaStream_t s, F call)
+{
+    int rc = check_dev(ctx, n_dropped, "n_dropped", true);
+    if (rc)
+        return rc;
+    const bool folded = n_dropped && ctx->plan.form == SEPW_FORM_TILED && ctx->plan.nvis > 0;
+    ctx->plan.dropped_out = folded ? n_dropped : nullptr;
+    rc = call();
+    ctx->plan.dropped_out = nullptr;
+    if (rc || folded || !n_dropped)
+        return rc;
+    SEPW_CUDA(ctx, cudaMemcpyAsync(n_dropped, ctx->plan.d_dropped, sizeof(int64_t),
+                                   cudaMemcpyDeviceToDevice, s));
+    return SEPW_OK;
+}
 
 }  // namespace
 
@@ -690,18 +711,6 @@ int sepw_degrid_planned(sepw_ctx *ctx, const float *taps, const float *grid,
     return SEPW_OK;
 }
 
-static int copy_dropped(sepw_ctx *ctx, int64_t *n_dropped, cudaStream_t s)
-{
-    if (!n_dropped)
-        return SEPW_OK;
-    int rc = check_dev(ctx, n_dropped, "n_dropped", false);
-    if (rc)
-        return rc;
-    SEPW_CUDA(ctx, cudaMemcpyAsync(n_dropped, ctx->plan.d_dropped, sizeof(int64_t),
-                                   cudaMemcpyDeviceToDevice, s));
-    return SEPW_OK;
-}
-
 int sepw_grid(sepw_ctx *ctx, const float *taps, int64_t nvis, const double *u,
               const double *v, const double *w, const float *vis, const float *weight,
               float *grid, int64_t *n_dropped, sepw_stream_t stream)
@@ -711,9 +720,9 @@ int sepw_grid(sepw_ctx *ctx, const float *taps, int64_t nvis, const double *u,
     int rc = sepw_plan(ctx, nvis, u, v, w, stream);
     if (rc)
         return rc;
-    if ((rc = sepw_grid_planned(ctx, taps, vis, weight, grid, stream)))
-        return rc;
-    return copy_dropped(ctx, n_dropped, (cudaStream_t)stream);
+    return with_dropped(ctx, n_dropped, (cudaStream_t)stream, [&] {
+        return sepw_grid_planned(ctx, taps, vis, weight, grid, stream);
+    });
 }
 
 int sepw_grid_batched(sepw_ctx *ctx, const float *taps, int32_t ngrids,
@@ -726,9 +735,9 @@ int sepw_grid_batched(sepw_ctx *ctx, const float *taps, int32_t ngrids,
     int rc = sepw_plan_batched(ctx, ngrids, vis_offsets, u, v, w, stream);
     if (rc)
         return rc;
-    if ((rc = sepw_grid_planned(ctx, taps, vis, weight, grids, stream)))
-        return rc;
-    return copy_dropped(ctx, n_dropped, (cudaStream_t)stream);
+    return with_dropped(ctx, n_dropped, (cudaStream_t)stream, [&] {
+        return sepw_grid_planned(ctx, taps, vis, weight, grids, stream);
+    });
 }
 
 int sepw_degrid(sepw_ctx *ctx, const float *taps, int64_t nvis, const double *u,
@@ -740,9 +749,9 @@ int sepw_degrid(sepw_ctx *ctx, const float *taps, int64_t nvis, const double *u,
     int rc = sepw_plan(ctx, nvis, u, v, w, stream);
     if (rc)
         return rc;
-    if ((rc = sepw_degrid_planned(ctx, taps, grid, weight, vis_out, stream)))
-        return rc;
-    return copy_dropped(ctx, n_dropped, (cudaStream_t)stream);
+    return with_dropped(ctx, n_dropped, (cudaStream_t)stream, [&] {
+        return sepw_degrid_planned(ctx, taps, grid, weight, vis_out, stream);
+    });
 }
 
 int sepw_device_status(sepw_ctx *ctx, int *status, sepw_stream_t stream)

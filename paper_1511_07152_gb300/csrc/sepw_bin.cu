@@ -30,6 +30,7 @@ __global__ void __launch_bounds__(256) locate_bin_kernel(
     unsigned long long *dropped, int32_t *__restrict__ drop_list, int ngrids,
     const int64_t *__restrict__ offsets)
 {
+    pdl_enter();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool active = i < nvis;
     int bin = -1;
@@ -168,17 +169,13 @@ static int plan_block(int64_t ntiles, int nsub)
     return tb;
 }
 constexpr int kPlanThreads = 1024, kPlanWarps = kPlanThreads / 32;
+constexpr int kOneBlockTiles = 256;  // up to here one block makes both passes
 
-__global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
-    int32_t ntiles, int32_t tb, int32_t nsub, Cut cut,
-    const int32_t *__restrict__ bin, int32_t *__restrict__ tile_count,
-    Totals *__restrict__ blocks, unsigned *ticket)
+// s_n[k] = visibilities of tile t0 + k, k < tb
+__device__ __forceinline__ void count_tiles(int t0, int tb, int ntiles, int nsub,
+                                            const int32_t *bin, int32_t *s_n)
 {
-    __shared__ Totals s_warps[33];
-    __shared__ int32_t s_n[1024];
-    __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t0 = blockIdx.x * tb;
     if (nsub <= 4) {  // a thread per tile
         if ((int)threadIdx.x < tb) {
             int c = 0;
@@ -187,9 +184,10 @@ __global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
                     c += bin[(int64_t)(t0 + threadIdx.x) * nsub + q];
             s_n[threadIdx.x] = c;
         }
+        return;
     }
 #pragma unroll 2
-    for (int k = nsub <= 4 ? tb : warp; k < tb; k += kPlanWarps) {  // a warp per tile
+    for (int k = warp; k < tb; k += kPlanWarps) {  // a warp per tile
         int c = 0;
         if (t0 + k < ntiles) {
             const int32_t *b = bin + (int64_t)(t0 + k) * nsub;
@@ -202,6 +200,19 @@ __global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
         if (lane == 0)
             s_n[k] = c;
     }
+}
+
+__global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
+    int32_t ntiles, int32_t tb, int32_t nsub, Cut cut,
+    const int32_t *__restrict__ bin, int32_t *__restrict__ tile_count,
+    Totals *__restrict__ blocks, unsigned *ticket)
+{
+    __shared__ Totals s_warps[33];
+    __shared__ int32_t s_n[1024];
+    __shared__ bool s_last;
+    pdl_enter();
+    const int t0 = blockIdx.x * tb;
+    count_tiles(t0, tb, ntiles, nsub, bin, s_n);
     __syncthreads();
     const int n = (int)threadIdx.x < tb ? s_n[threadIdx.x] : 0;
     if ((int)threadIdx.x < tb && t0 + (int)threadIdx.x < ntiles)
@@ -255,7 +266,9 @@ __device__ __forceinline__ void list_full(WorkItem *__restrict__ out, int tile0,
     }
 }
 
-// Pass 2: every bin's count replaced by its first slot; items and units.
+// Pass 2: every bin's count replaced by its first slot; items and units.  ONE:
+// the only block, which counts its tiles itself (no pass 1b).
+template <bool ONE>
 __global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
     int32_t ntiles, int32_t tb, int32_t nsub, Cut cut,
     const int32_t *__restrict__ tile_count, const Totals *__restrict__ blocks,
@@ -264,15 +277,27 @@ __global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
 {
     __shared__ Totals s_warps[33];
     __shared__ int32_t s_n[1024], s_at[1024], s_items[1024], s_units[1024];
+    pdl_enter();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int t0 = blockIdx.x * tb, t = t0 + threadIdx.x;
-    const int n = (int)threadIdx.x < tb && t < ntiles ? tile_count[t] : 0;
+    int n = 0;
+    if constexpr (ONE) {
+        count_tiles(0, tb, ntiles, nsub, bin, s_n);
+        __syncthreads();
+        n = (int)threadIdx.x < tb ? s_n[threadIdx.x] : 0;
+    } else if ((int)threadIdx.x < tb && t < ntiles) {
+        n = tile_count[t];
+    }
     const Totals mine = tile_totals(n, cut);
     const int chunk = cut.chunk, unit = cut.unit_of(n);
     Totals sum;
-    const Totals before = blocks[blockIdx.x];  // exclusive prefix of the block
-    const Totals in = block_scan(mine, s_warps, sum) - mine, at = before + in;
-    const Totals all = blocks[gridDim.x];
+    const Totals in = block_scan(mine, s_warps, sum) - mine;
+    Totals before{0, 0, 0, 0, 0}, all = sum;  // exclusive prefix of the block, all blocks
+    if constexpr (!ONE) {
+        before = blocks[blockIdx.x];
+        all = blocks[gridDim.x];
+    }
+    const Totals at = before + in;
     if (t == 0) {
         *nitems = all.full_items + all.part_items;
         if (units)
@@ -339,6 +364,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(
     const uint64_t *__restrict__ rec0, const int32_t *__restrict__ bin_first,
     int32_t *__restrict__ perm, uint64_t *__restrict__ rec)
 {
+    pdl_enter();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nvis)
         return;
@@ -382,6 +408,7 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
     __shared__ uint64_t s_rec[kChunk];
     __shared__ int32_t s_perm[kChunk];
     __shared__ int32_t s_wsum[32];
+    pdl_enter(p);
     // blocks stride over the plan's items (sparse plans have far fewer items
     // than their capacity, so the grid is sized by the SM count, not by it)
     const int n_items = *nitems;
@@ -478,12 +505,19 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
     }
 }
 
-// Degridding writes 0 for every dropped visibility of the plan.
+// Degridding writes 0 for every dropped visibility of the plan.  Also clears
+// the degridder's work counter.
 __global__ void zero_dropped_kernel(const int32_t *__restrict__ drop_list,
                                     const unsigned long long *__restrict__ ndrop,
-                                    float2 *__restrict__ vis)
+                                    float2 *__restrict__ vis, int32_t *counter, int64_t *dropped)
 {
+    pdl_enter();
     const unsigned long long n = *ndrop;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *counter = 0;
+        if (dropped)
+            *dropped = (int64_t)n;
+    }
     for (unsigned long long k = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
          k < n; k += (unsigned long long)gridDim.x * blockDim.x)
         vis[drop_list[k]] = make_float2(0.f, 0.f);
@@ -491,8 +525,8 @@ __global__ void zero_dropped_kernel(const int32_t *__restrict__ drop_list,
 
 cudaError_t launch_zero_dropped(const Plan &plan, float2 *vis, cudaStream_t s)
 {
-    zero_dropped_kernel<<<64, 256, 0, s>>>(plan.d_drop_list, plan.d_dropped, vis);
-    return cudaGetLastError();
+    return launch_pdl(zero_dropped_kernel, 64, 256, 0, s, plan.d_drop_list, plan.d_dropped, vis,
+                      plan.d_item_counter + 1, plan.dropped_out);
 }
 
 // The units of the tiled gridders: 32 to 256 visibilities, about two for each
@@ -561,30 +595,33 @@ cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
     if (e != cudaSuccess)
         return e;
     int32_t *const bin = (int32_t *)(plan.d_bin_base + kBinHeader);
-    if (nvis > 0) {
-        locate_bin_kernel<<<(unsigned)((nvis + 255) / 256), 256, 0, s>>>(
-            p, nvis, u, v, w, plan.d_tile, plan.d_rank, plan.d_rec0, bin,
-            plan.d_dropped, plan.d_drop_list, plan.ngrids, plan.d_offsets);
-        if ((e = cudaGetLastError()) != cudaSuccess)
-            return e;
-    }
-    const int tb = plan_block(plan.ntiles, p.nsub), nblk = (plan.ntiles + tb - 1) / tb;
-    Totals *const blocks = (Totals *)plan.d_blocks;
+    if (nvis > 0 &&
+        (e = launch_pdl(locate_bin_kernel, (nvis + 255) / 256, 256, 0, s, p, nvis, u, v, w,
+                        plan.d_tile, plan.d_rank, plan.d_rec0, bin, plan.d_dropped,
+                        plan.d_drop_list, plan.ngrids, plan.d_offsets)) != cudaSuccess)
+        return e;
     const Cut cut{p.chunk, plan.unit, plan.unit_parts};
-    tile_count_kernel<<<nblk, kPlanThreads, 0, s>>>(
-        plan.ntiles, tb, p.nsub, cut, bin, plan.d_tile_count, blocks,
-        (unsigned *)(plan.d_bin_base + kBinTicket));
-    if ((e = cudaGetLastError()) != cudaSuccess)
-        return e;
-    tile_items_kernel<<<nblk, kPlanThreads, 0, s>>>(
-        plan.ntiles, tb, p.nsub, cut, plan.d_tile_count, blocks, bin, plan.d_items, plan.d_nitems,
-        plan.d_units, plan.d_nunits);
-    if ((e = cudaGetLastError()) != cudaSuccess)
+    Totals *const blocks = (Totals *)plan.d_blocks;
+    if (plan.ntiles <= kOneBlockTiles) {
+        e = launch_pdl(tile_items_kernel<true>, 1, kPlanThreads, 0, s, plan.ntiles,
+                       kOneBlockTiles, p.nsub, cut, plan.d_tile_count, blocks, bin, plan.d_items,
+                       plan.d_nitems, plan.d_units, plan.d_nunits);
+    } else {
+        const int tb = plan_block(plan.ntiles, p.nsub), nblk = (plan.ntiles + tb - 1) / tb;
+        e = launch_pdl(tile_count_kernel, nblk, kPlanThreads, 0, s, plan.ntiles, tb, p.nsub, cut,
+                       bin, plan.d_tile_count, blocks,
+                       (unsigned *)(plan.d_bin_base + kBinTicket));
+        if (e == cudaSuccess)
+            e = launch_pdl(tile_items_kernel<false>, nblk, kPlanThreads, 0, s, plan.ntiles, tb,
+                           p.nsub, cut, plan.d_tile_count, blocks, bin, plan.d_items,
+                           plan.d_nitems, plan.d_units, plan.d_nunits);
+    }
+    if (e != cudaSuccess)
         return e;
     if (nvis > 0) {
-        scatter_kernel<<<(unsigned)((nvis + 255) / 256), 256, 0, s>>>(
-            nvis, plan.d_tile, plan.d_rank, plan.d_rec0, bin, plan.d_perm, plan.d_rec);
-        if ((e = cudaGetLastError()) != cudaSuccess)
+        e = launch_pdl(scatter_kernel, (nvis + 255) / 256, 256, 0, s, nvis, plan.d_tile,
+                       plan.d_rank, plan.d_rec0, bin, plan.d_perm, plan.d_rec);
+        if (e != cudaSuccess)
             return e;
         if (plan.sorted)
             return launch_item_sort(p, plan, num_sms, s);
@@ -604,9 +641,8 @@ cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, 
     if (e != cudaSuccess)
         return e;
     const int nblk = std::max(1, std::min(plan.items_capacity, 16 * num_sms));
-    item_sort_kernel<<<nblk, kSortThreads, shm, s>>>(p, plan.d_items, plan.d_nitems, plan.d_perm,
-                                                     plan.d_rec);
-    return cudaGetLastError();
+    return launch_pdl(item_sort_kernel, nblk, kSortThreads, shm, s, p, plan.d_items, plan.d_nitems,
+                      plan.d_perm, plan.d_rec);
 }
 
 }  // namespace sepw

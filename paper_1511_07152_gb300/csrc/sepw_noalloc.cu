@@ -180,11 +180,13 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     pl.window = wbytes > 0 && wbytes <= kTablesBytes && plan_window(dp, nvis, 1);
     pl.sorted = !pl.window;
     set_units(dp, num_sms, pl);
+    dp.early = 1;
     set_bins(dp, pl.window ? kBinsWindow : kBinsSorted);
     float *tables = (float *)(b + kOffTables);
     if (!pl.window && sizeof(float2) * dp.P * dp.OS * (size_t)dp.S > kTablesBytes)
         tables = nullptr;
 
+    pl.dropped_out = n_dropped;
     cudaStream_t s = (cudaStream_t)stream;
     if (launch_plan(dp, nvis, u, v, w, pl, num_sms, s) != cudaSuccess) {
         cudaGetLastError();
@@ -196,8 +198,10 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
         cudaGetLastError();
         return SEPW_ECUDA;
     }
-    if (n_dropped && cudaMemcpyAsync(n_dropped, pl.d_dropped, sizeof(int64_t),
-                                     cudaMemcpyDeviceToDevice, s) != cudaSuccess) {
+    // with visibilities the gridder's launches have written it
+    if (n_dropped && nvis == 0 &&
+        cudaMemcpyAsync(n_dropped, pl.d_dropped, sizeof(int64_t), cudaMemcpyDeviceToDevice, s) !=
+            cudaSuccess) {
         cudaGetLastError();
         return SEPW_ECUDA;
     }

@@ -40,6 +40,7 @@
 // sum_r F1_v(r) X(r, c) per column and then the sum over its columns with
 // F1_u(c); the partial sums of several visibilities are reduced over the
 // lanes together (reduce-scatter), conjugated back as needed and scaled by W.
+#include <algorithm>
 #include <type_traits>
 
 #include "sepw_internal.cuh"
@@ -126,6 +127,7 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) grid_tiled_k
     const float2 *__restrict__ vis, const float *__restrict__ weight,
     const float2 *__restrict__ taps, float2 *grid)
 {
+    pdl_enter(p);
     constexpr int RG = Layout<S>::RG, RPL = Layout<S>::RPL;
     __shared__ int4 s_meta[kTiledWarps * 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -250,6 +252,7 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled
     const float *__restrict__ weight, const float2 *__restrict__ taps,
     float2 *__restrict__ vis_out)
 {
+    pdl_enter(p);
     constexpr int RG = Layout<S>::RG, RPL = Layout<S>::RPL;
     extern __shared__ float4 smem4[];
     __shared__ int s_item;
@@ -438,6 +441,7 @@ __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block
     const float *__restrict__ weight, const float2 *__restrict__ taps,
     float2 *__restrict__ vis_out)
 {
+    pdl_enter(p);
     constexpr int B = Blk<S>::B, K = Blk<S>::K, MS = Blk<S>::MS;
     extern __shared__ float4 smem4[];
     __shared__ int s_item;
@@ -625,6 +629,7 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
     const float2 *__restrict__ vis, const float *__restrict__ weight,
     const float2 *__restrict__ taps, const float *__restrict__ planar, float2 *grid)
 {
+    pdl_enter(p);
     constexpr int RB = Blk2<S>::RB, RP = Blk2<S>::RP, CB = Blk2<S>::CB;
     constexpr bool FULL = Blk2<S>::FULL;
     static_assert(RB % 2 == 0, "rows come in pairs");
@@ -824,9 +829,17 @@ static size_t tiled_smem(int W, int WP)
 // order), with tap k at position (k mod 4) S/4 + floor(k / 4) when 4 divides
 // S.  A lane of the block gridder owns rows g, g + 4, g + 8, ... (g = k mod 4),
 // whose taps are then adjacent: one vector load gives its FP32 pairs.
+// Also clears the gridder's work counter.
 __global__ void planar_taps_kernel(const float2 *__restrict__ taps, float *__restrict__ out,
-                                   int64_t n, int S)
+                                   int64_t n, int S, int32_t *counter,
+                                   const unsigned long long *ndrop, int64_t *dropped)
 {
+    pdl_enter();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *counter = 0;
+        if (dropped)
+            *dropped = (int64_t)*ndrop;
+    }
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
          e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t row = e / S;
@@ -838,44 +851,41 @@ __global__ void planar_taps_kernel(const float2 *__restrict__ taps, float *__res
     }
 }
 
-static cudaError_t launch_planar_taps(const float2 *taps, float *out, int64_t n, int S,
-                               cudaStream_t s)
-{
-    if (n <= 0)
-        return cudaSuccess;
-    const int64_t blocks = (n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096;
-    planar_taps_kernel<<<(unsigned)blocks, 256, 0, s>>>(taps, out, n, S);
-    return cudaGetLastError();
-}
-
 template <int S>
 static cudaError_t launch_grid_S(const DevParams &p, const Plan &plan, const float2 *vis,
                                  const float *weight, const float2 *taps, float *planar,
                                  float2 *grid, int num_sms, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(plan.d_item_counter, 0, sizeof(int32_t), s);
-    if (e != cudaSuccess)
-        return e;
     if constexpr (Blk2<S>::OK) {
-        const unsigned nb = (unsigned)(num_sms * kGridBlkPerSM);
+        const int nb = num_sms * kGridBlkPerSM;
         if (planar) {  // rebuilt per call: the caller's table may have changed
             const int64_t n = (p.facet ? 2 : 1) * (int64_t)p.P * p.OS * S;
-            if ((e = launch_planar_taps(taps, planar, n, S, s)) != cudaSuccess)
+            const cudaError_t e = launch_pdl(planar_taps_kernel,
+                                             std::min<int64_t>((n + 255) / 256, 4096), 256, 0, s,
+                                             taps, planar, n, S, plan.d_item_counter,
+                                             plan.d_dropped, plan.dropped_out);
+            if (e != cudaSuccess)
                 return e;
+            return launch_pdl(grid_tiled_block_kernel<S, true>, nb, kTiledThreads, 0, s, p,
+                              plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec,
+                              plan.d_perm, vis, weight, taps, planar, grid);
         }
-        if (planar)
-            grid_tiled_block_kernel<S, true><<<nb, kTiledThreads, 0, s>>>(
-                p, plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm,
-                vis, weight, taps, planar, grid);
-        else
-            grid_tiled_block_kernel<S, false><<<nb, kTiledThreads, 0, s>>>(
-                p, plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm,
-                vis, weight, taps, nullptr, grid);
-    } else
-        grid_tiled_kernel<S><<<num_sms * kTiledBlocksPerSM, kTiledThreads, 0, s>>>(
-            p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec, plan.d_perm, vis,
-            weight, taps, grid);
-    return cudaGetLastError();
+    }
+    cudaError_t e = cudaMemsetAsync(plan.d_item_counter, 0, sizeof(int32_t), s);
+    if (e == cudaSuccess && plan.dropped_out)
+        e = cudaMemcpyAsync(plan.dropped_out, plan.d_dropped, sizeof(int64_t),
+                            cudaMemcpyDeviceToDevice, s);
+    if (e != cudaSuccess)
+        return e;
+    if constexpr (Blk2<S>::OK)
+        return launch_pdl(grid_tiled_block_kernel<S, false>, num_sms * kGridBlkPerSM,
+                          kTiledThreads, 0, s, p, plan.d_units, plan.d_nunits,
+                          plan.d_item_counter, plan.d_rec, plan.d_perm, vis, weight, taps, nullptr,
+                          grid);
+    else
+        return launch_pdl(grid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, 0, s,
+                          p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec,
+                          plan.d_perm, vis, weight, taps, grid);
 }
 
 template <int S>
@@ -885,26 +895,22 @@ static cudaError_t launch_degrid_S(const DevParams &p, const Plan &plan,
                                    cudaStream_t s)
 {
     const int W = p.T + S - 1;
-    cudaError_t e = cudaMemsetAsync(plan.d_item_counter + 1, 0, sizeof(int32_t), s);
-    if (e != cudaSuccess)
-        return e;
     if constexpr (Blk<S>::OK) {
         // float2 window rows with stride = 4 (mod 8): the 4 x 4 patch read by a
         // virtual warp covers all 32 banks
         const int WP = W + ((4 - W % 8) + 8) % 8;
         const size_t shm = sizeof(float4) * (size_t)((W * WP + 1) / 2) +
                            (size_t)kTiledWarps * 2 * Blk<S>::MS * (sizeof(int4) + sizeof(int));
-        degrid_tiled_block_kernel<S><<<num_sms * Blk<S>::BPS, kTiledThreads, shm, s>>>(
-            p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec,
+        return launch_pdl(
+            degrid_tiled_block_kernel<S>, num_sms * Blk<S>::BPS, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec,
             plan.d_perm, grid, weight, taps, vis);
     } else {
         const int WP = window_stride(W, S);
         const size_t shm = tiled_smem(W, WP);
-        degrid_tiled_kernel<S><<<num_sms * kTiledBlocksPerSM, kTiledThreads, shm, s>>>(
-            p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec,
+        return launch_pdl(
+            degrid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec,
             plan.d_perm, grid, weight, taps, vis);
     }
-    return cudaGetLastError();
 }
 
 #define SEPW_FOR_EACH_S(X) \

@@ -71,12 +71,16 @@ template <int S>
 __global__ void __launch_bounds__(256) window_tables_kernel(
     const float2 *__restrict__ utaps, const float2 *__restrict__ vtaps, int64_t rows,
     float *__restrict__ utab, float *__restrict__ vtab, int32_t *__restrict__ flags,
-    int32_t *counter)
+    int32_t *counter, const unsigned long long *ndrop, int64_t *dropped)
 {
+    pdl_enter();
     using W = Win<S>;
     constexpr int UE = W::UROW / 2, E = UE + 7 * W::RPL;
-    if (blockIdx.x == 0 && threadIdx.x == 0)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         *counter = 0;
+        if (dropped)
+            *dropped = (int64_t)*ndrop;
+    }
     int big = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows * E;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -150,6 +154,7 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
     const float2 *__restrict__ taps, const float *__restrict__ utab,
     const float *__restrict__ vtab, const int32_t *__restrict__ flags, float2 *grid)
 {
+    pdl_enter(p);
     using W = Win<S>;
     constexpr int RPL = W::RPL, CPL = W::CPL, RP = W::RP;
     constexpr bool ODD = W::ODD;
@@ -327,15 +332,14 @@ static cudaError_t launch_S(const DevParams &p, const Plan &plan, const float2 *
     float *const utab = tables;
     float *const vtab = tables + W::UROW * rows;
     int32_t *const flags = reinterpret_cast<int32_t *>(vtab + W::VROW * rows);
-    window_tables_kernel<S><<<kWinTabBlocks, 256, 0, s>>>(taps, taps + p.voff, rows, utab, vtab,
-                                                          flags, plan.d_item_counter);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e =
+        launch_pdl(window_tables_kernel<S>, kWinTabBlocks, 256, 0, s, taps, taps + p.voff, rows,
+                   utab, vtab, flags, plan.d_item_counter, plan.d_dropped, plan.dropped_out);
     if (e != cudaSuccess)
         return e;
-    grid_window_kernel<S><<<num_sms * W::BPS, kWinThreads, 0, s>>>(
-        p, plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm, vis, weight,
-        taps, utab, vtab, flags, grid);
-    return cudaGetLastError();
+    return launch_pdl(grid_window_kernel<S>, num_sms * W::BPS, kWinThreads, 0, s, p, plan.d_units,
+                      plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm, vis, weight,
+                      taps, utab, vtab, flags, grid);
 }
 
 #define SEPW_FOR_EACH_WIN_S(X) \
