@@ -704,8 +704,8 @@ int sepw_degrid_planned(sepw_ctx *ctx, const float *taps, const float *grid,
             DevParams dp = ctx->dp;
             dp.chk_status = ctx->d_status;  // the checked build's bounds failures
             SEPW_CUDA(ctx, launch_degrid_tiled(dp, pl, (const float2 *)grid, weight,
-                                               (const float2 *)taps, (float2 *)vis_out,
-                                               ctx->num_sms, s));
+                                               (const float2 *)taps, ctx->d_planar,
+                                               (float2 *)vis_out, ctx->num_sms, s));
         }
     }
     return SEPW_OK;

@@ -522,7 +522,7 @@ cudaError_t launch_grid_tiled(const DevParams &p, const Plan &plan, const float2
                               float2 *grid, int num_sms, cudaStream_t s);
 cudaError_t launch_degrid_tiled(const DevParams &p, const Plan &plan,
                                 const float2 *grid, const float *weight,
-                                const float2 *taps, float2 *vis, int num_sms,
+                                const float2 *taps, float *tables, float2 *vis, int num_sms,
                                 cudaStream_t s);
 
 // sepw_window.cu: gridder of the tiled form for the supports the block gridder
@@ -532,6 +532,12 @@ size_t window_tables_bytes(const DevParams &p);
 cudaError_t launch_grid_window(const DevParams &p, const Plan &plan, const float2 *vis,
                                const float *weight, const float2 *taps, float *tables,
                                float2 *grid, int num_sms, cudaStream_t s);
+
+// degridder of the same plans for some supports (degrid_window_takes)
+bool degrid_window_takes(const DevParams &p, const Plan &plan);
+cudaError_t launch_degrid_window(const DevParams &p, const Plan &plan, const float2 *grid,
+                                 const float *weight, const float2 *taps, float *tables,
+                                 float2 *vis, int num_sms, cudaStream_t s);
 
 // Control of the tensor-core kernels: the limit of every bounded mbarrier
 // wait, and a test hook (stall != 0: the MMA thread issues and commits

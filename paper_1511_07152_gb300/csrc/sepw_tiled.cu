@@ -944,10 +944,12 @@ cudaError_t launch_grid_tiled(const DevParams &p0, const Plan &plan, const float
 
 cudaError_t launch_degrid_tiled(const DevParams &p0, const Plan &plan,
                                 const float2 *grid, const float *weight,
-                                const float2 *taps, float2 *vis, int num_sms,
+                                const float2 *taps, float *tables, float2 *vis, int num_sms,
                                 cudaStream_t s)
 {
     const DevParams p = with_plan_bounds(p0, plan);
+    if (degrid_window_takes(p, plan))
+        return launch_degrid_window(p, plan, grid, weight, taps, tables, vis, num_sms, s);
     switch (p.S) {
 #define X(SS) \
     case SS: return launch_degrid_S<SS>(p, plan, grid, weight, taps, vis, num_sms, s);

@@ -322,24 +322,305 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
     }
 }
 
+// ---------------------------------------------------------------------------
+// Degridding with the same windows: the warp keeps the window's cells in
+// registers (read once per block of origins, a row at a time as it steps
+// down), sums a visibility's taps against them with paired FMAs over the
+// lane's rows, and leaves a partial sum per lane in shared memory, which is
+// added up for 16 visibilities at a time.  For supports without a block
+// degridder, whose column kernel keeps the tile's window in shared memory and
+// a CTA on every item, with the lanes of one column each: 333k visibilities at
+// S = 10 took it 68 us, this kernel 58 us (bound by the latency of its short
+// units); a step of 2M at S = 20 1090 us, now 734.  S = 2, 6 and 14 keep the
+// column kernel (S = 14, whose window is three lanes' columns wide for 17
+// cells: a step of 4M 1222 us with it, 1323 with this one).
+//
+// As in gridding, zero taps must not meet non-finite values: from the first
+// cell of a unit that is not below 1e30 on, its visibilities go through
+// degrid_footprint.
+// ---------------------------------------------------------------------------
+template <int S>
+__device__ __noinline__ float2 degrid_footprint(const float2 *__restrict__ tu,
+                                                const float2 *__restrict__ tv, float sg,
+                                                const float2 *__restrict__ g, int N, int lane)
+{
+    float2 acc = make_float2(0.f, 0.f);
+    for (int c = lane; c < S * S; c += 32) {
+        const int k = c / S, j = c % S;
+        const float2 a = __ldg(tu + j), b = __ldg(tv + k), x = __ldg(g + (int64_t)k * N + j);
+        const float ay = sg * a.y, by = sg * b.y;  // conjugated taps
+        const float kr = a.x * b.x - ay * by, ki = a.x * by + ay * b.x;
+        acc.x += kr * x.x - ki * x.y;
+        acc.y += kr * x.y + ki * x.x;
+    }
+    return acc;
+}
+
+template <int S>
+__global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) degrid_window_kernel(
+    DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
+    int32_t *counter, const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
+    const float2 *__restrict__ grid, const float *__restrict__ weight,
+    const float2 *__restrict__ taps, const float *__restrict__ utab,
+    const float *__restrict__ vtab, const int32_t *__restrict__ flags, float2 *__restrict__ vis_out)
+{
+    pdl_enter(p);
+    using W = Win<S>;
+    constexpr int RPL = W::RPL, CPL = W::CPL, RP = W::RP;
+    constexpr bool ODD = W::ODD;
+    __shared__ int2 s_meta[kWinWarps * 32];
+    __shared__ float2 s_part[kWinWarps][16 * 33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rg = lane >> 3, cg = lane & 7;
+    int2 *const meta = s_meta + warp * 32;
+    float2 *const part = s_part[warp];
+    const float *const ulane = utab + 2 * cg;
+    const float *const vlane = vtab + rg * W::VG;
+    const bool last_col = cg + 8 * (CPL - 1) < S + 3;
+    const int n_units = *nunits;
+    bool big = false;
+    for (int b = lane; b < kWinTabBlocks; b += 32)
+        big |= flags[b] != 0;
+    big = __any_sync(0xffffffffu, big);
+
+    const int n_warps = gridDim.x * kWinWarps;
+    auto next_unit = [&]() {
+        const int k = lane == 0 ? atomicAdd(counter, 1) : 0;
+        return n_warps + __shfl_sync(0xffffffffu, k, 0);
+    };
+    for (int unit = warp * gridDim.x + blockIdx.x; unit < n_units; unit = next_unit()) {
+        const WorkItem it = units[unit];
+        if (!work_item_ok(p, it))
+            continue;  // checked build only
+        const TileOrigin o = tile_origin(p, it.tile);
+        const int b1 = it.start + it.count;
+        const float2 *const g0 = grid + o.base + (o.gy0 + rg) * p.N + o.gx0 + cg;
+
+        float2 xr[RP][CPL], xi[RP][CPL], xe[CPL];
+#pragma unroll
+        for (int c = 0; c < CPL; ++c) {
+#pragma unroll
+            for (int q = 0; q < RP; ++q)
+                xr[q][c] = xi[q][c] = dup(0.f);
+            xe[c] = dup(0.f);
+        }
+        int cur = -1;  // block: column << 8 | row
+        bool bad = big;
+        // the lane's cells of window row rg + 4 r at block blk
+        auto load_row = [&](int blk, int r, float2(&v)[CPL]) {
+            const int y = 4 * ((blk & 255) + r), x = 4 * (blk >> 8);
+            bool off = false;
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+                v[c] = dup(0.f);
+                if ((c < CPL - 1 || last_col) && o.gy0 + y + rg < p.N &&
+                    o.gx0 + x + cg + 8 * c < p.N)
+                    v[c] = __ldg(g0 + (int64_t)y * p.N + x + 8 * c);
+                off |= !(fabsf(v[c].x) < 1e30f && fabsf(v[c].y) < 1e30f);
+            }
+            bad |= __any_sync(0xffffffffu, off);
+        };
+        auto step = [&]() {  // one block down: the first row leaves, a new last one comes
+            float2 v[CPL];
+            ++cur;
+            load_row(cur, RPL - 1, v);
+#pragma unroll
+            for (int c = 0; c < CPL; ++c) {
+#pragma unroll
+                for (int q = 0; q < RP; ++q) {
+                    const bool more = q + 1 < RP;
+                    const int n = more ? q + 1 : q;
+                    xr[q][c] = make_float2(xr[q][c].y, more ? xr[n][c].x : ODD ? xe[c].x : v[c].x);
+                    xi[q][c] = make_float2(xi[q][c].y, more ? xi[n][c].x : ODD ? xe[c].y : v[c].y);
+                }
+                if constexpr (ODD)
+                    xe[c] = v[c];
+            }
+        };
+        auto move_to = [&](int blk) {
+            const int d = blk - cur;
+            if (cur >= 0 && d > 0 && d < RPL) {
+#pragma unroll 1
+                for (int k = 0; k < d; ++k)
+                    step();
+            } else {
+#pragma unroll
+                for (int r = 0; r < RPL; ++r) {
+                    float2 v[CPL];
+                    load_row(blk, r, v);
+#pragma unroll
+                    for (int c = 0; c < CPL; ++c) {
+                        if (r >= 2 * RP) {
+                            xe[c] = v[c];
+                        } else if (r & 1) {
+                            xr[r >> 1][c].y = v[c].x;
+                            xi[r >> 1][c].y = v[c].y;
+                        } else {
+                            xr[r >> 1][c].x = v[c].x;
+                            xi[r >> 1][c].x = v[c].y;
+                        }
+                    }
+                }
+                cur = blk;
+            }
+        };
+
+        for (int base = it.start; base < b1; base += 32) {
+            const int s = base + lane;
+            int blk = -1, i = -1;
+            bool cj = false;
+            float wt = 0.f;
+            uint64_t r = 0;
+            if (s < b1) {
+                r = rec[s];
+                i = perm[s];
+                if (record_ok(p, r, i, o.gy0, o.gx0)) {
+                    wt = weight ? __ldg(weight + i) : 1.0f;
+                    cj = rec_conj(r);
+                } else {
+                    r = 0;  // checked build: no output
+                    i = -1;
+                }
+                const int row = rec_plane(r) * p.OS;
+                blk = (rec_lx(r) >> 2) << 8 | (rec_ly(r) >> 2);
+                meta[lane] = make_int2((row + rec_ou(r)) * W::UROW + 2 * (3 - (rec_lx(r) & 3)),
+                                       (row + rec_ov(r)) * W::VROW +
+                                           (3 - (rec_ly(r) & 3)) * W::VG);
+            }
+            __syncwarp();
+            const int n = min(32, b1 - base);
+            const int prev = __shfl_up_sync(0xffffffffu, blk, 1);
+            unsigned starts = __ballot_sync(0xffffffffu, lane < n && (lane == 0 || blk != prev));
+            // a half of 16 starts a run of its own, so that runs end with it
+            if (n > 16)
+                starts |= 1u << 16;
+            const unsigned cjs = __ballot_sync(0xffffffffu, cj);
+            for (int q = 0; q < n;) {
+                starts &= starts - 1;  // now the next run's start, if any
+                const int q1 = starts ? __ffs(starts) - 1 : n;
+                const int bq = __shfl_sync(0xffffffffu, blk, q);
+                if (bq != cur)
+                    move_to(bq);
+                if (bad) {
+                    for (; q < q1; ++q) {
+                        const uint64_t rq = __shfl_sync(0xffffffffu, r, q);
+                        const float2 *t = taps + (int64_t)rec_plane(rq) * p.OS * S;
+                        part[(q & 15) * 33 + lane] = degrid_footprint<S>(
+                            t + rec_ou(rq) * S, t + p.voff + rec_ov(rq) * S,
+                            rec_conj(rq) ? 1.f : -1.f,
+                            grid + o.base + (o.gy0 + rec_ly(rq)) * p.N + o.gx0 + rec_lx(rq), p.N,
+                            lane);
+                    }
+                }
+                for (; q < q1; ++q) {
+                    const int2 m = meta[q];
+                    // plain kernels take conjugated taps: sign + 1, conj ones - 1
+                    const float sg = __uint_as_float(0x3f800000u | (cjs >> q) << 31);
+                    const float *tu = ulane + m.x;
+                    float2 vr[RP], vi[RP], ve;
+                    window_vtaps<S>(vlane + m.y, vr, vi, ve);
+#pragma unroll
+                    for (int k = 0; k < RP; ++k)
+                        vi[k] = __fmul2_rn(vi[k], dup(sg));
+                    if constexpr (ODD)
+                        ve.y *= sg;
+                    float sr = 0.f, si = 0.f;
+#pragma unroll
+                    for (int c = 0; c < CPL; ++c) {
+                        float2 a = dup(0.f), b = dup(0.f);  // sum conj(v) x over the rows
+#pragma unroll
+                        for (int k = 0; k < RP; ++k) {
+                            a = __ffma2_rn(vr[k], xr[k][c], a);
+                            a = __ffma2_rn(vi[k], xi[k][c], a);
+                            b = __ffma2_rn(vr[k], xi[k][c], b);
+                            b = __ffma2_rn(make_float2(-vi[k].x, -vi[k].y), xr[k][c], b);
+                        }
+                        float tr = a.x + a.y, ti = b.x + b.y;
+                        if constexpr (ODD) {
+                            tr = fmaf(ve.x, xe[c].x, tr);
+                            tr = fmaf(ve.y, xe[c].y, tr);
+                            ti = fmaf(ve.x, xe[c].y, ti);
+                            ti = fmaf(-ve.y, xe[c].x, ti);
+                        }
+                        const float2 t = __ldg(reinterpret_cast<const float2 *>(tu + 16 * c));
+                        const float uy = sg * t.y;
+                        sr = fmaf(tr, t.x, sr);
+                        sr = fmaf(ti, uy, sr);
+                        si = fmaf(ti, t.x, si);
+                        si = fmaf(-tr, uy, si);
+                    }
+                    part[(q & 15) * 33 + lane] = make_float2(sr, si);
+                }
+                if (q == 16 || q == n) {  // 16 partial sums of each lane's 32, two lanes a sum
+                    __syncwarp();
+                    const int h = (q - 1) & 16, e = h + (lane & 15);
+                    float re = 0.f, im = 0.f;
+#pragma unroll
+                    for (int l = 0; l < 16; ++l) {
+                        const float2 t = part[(lane & 15) * 33 + (lane & 16) + l];
+                        re += t.x;
+                        im += t.y;
+                    }
+                    re += __shfl_xor_sync(0xffffffffu, re, 16);
+                    im += __shfl_xor_sync(0xffffffffu, im, 16);
+                    const int ie = __shfl_sync(0xffffffffu, i, e);
+                    const float we = __shfl_sync(0xffffffffu, wt, e);
+                    if (lane < 16 && e < n && ie >= 0)
+                        vis_out[ie] = make_float2(we * re, we * im);
+                    __syncwarp();
+                }
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// the tables of this call, from the caller's
+template <int S>
+struct Tables {
+    float *u, *v;
+    int32_t *flags;
+    Tables(const DevParams &p, float *at)
+    {
+        const int64_t rows = (int64_t)p.P * p.OS;
+        u = at;
+        v = u + Win<S>::UROW * rows;
+        flags = reinterpret_cast<int32_t *>(v + Win<S>::VROW * rows);
+    }
+    cudaError_t build(const DevParams &p, const float2 *taps, int32_t *counter, const Plan &plan,
+                      int64_t *dropped, cudaStream_t s) const
+    {
+        return launch_pdl(window_tables_kernel<S>, kWinTabBlocks, 256, 0, s, taps, taps + p.voff,
+                          (int64_t)p.P * p.OS, u, v, flags, counter, plan.d_dropped, dropped);
+    }
+};
+
 template <int S>
 static cudaError_t launch_S(const DevParams &p, const Plan &plan, const float2 *vis,
                             const float *weight, const float2 *taps, float *tables, float2 *grid,
                             int num_sms, cudaStream_t s)
 {
-    using W = Win<S>;
-    const int64_t rows = (int64_t)p.P * p.OS;
-    float *const utab = tables;
-    float *const vtab = tables + W::UROW * rows;
-    int32_t *const flags = reinterpret_cast<int32_t *>(vtab + W::VROW * rows);
-    const cudaError_t e =
-        launch_pdl(window_tables_kernel<S>, kWinTabBlocks, 256, 0, s, taps, taps + p.voff, rows,
-                   utab, vtab, flags, plan.d_item_counter, plan.d_dropped, plan.dropped_out);
+    const Tables<S> t(p, tables);
+    const cudaError_t e = t.build(p, taps, plan.d_item_counter, plan, plan.dropped_out, s);
     if (e != cudaSuccess)
         return e;
-    return launch_pdl(grid_window_kernel<S>, num_sms * W::BPS, kWinThreads, 0, s, p, plan.d_units,
-                      plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm, vis, weight,
-                      taps, utab, vtab, flags, grid);
+    return launch_pdl(grid_window_kernel<S>, num_sms * Win<S>::BPS, kWinThreads, 0, s, p,
+                      plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm,
+                      vis, weight, taps, t.u, t.v, t.flags, grid);
+}
+
+template <int S>
+static cudaError_t launch_degrid_S(const DevParams &p, const Plan &plan, const float2 *grid,
+                                   const float *weight, const float2 *taps, float *tables,
+                                   float2 *vis, int num_sms, cudaStream_t s)
+{
+    const Tables<S> t(p, tables);
+    const cudaError_t e = t.build(p, taps, plan.d_item_counter + 1, plan, nullptr, s);
+    if (e != cudaSuccess)
+        return e;
+    return launch_pdl(degrid_window_kernel<S>, num_sms * Win<S>::BPS, kWinThreads, 0, s, p,
+                      plan.d_units, plan.d_nunits, plan.d_item_counter + 1, plan.d_rec, plan.d_perm,
+                      grid, weight, taps, t.u, t.v, t.flags, vis);
 }
 
 #define SEPW_FOR_EACH_WIN_S(X) \
@@ -373,6 +654,35 @@ cudaError_t launch_grid_window(const DevParams &p, const Plan &plan, const float
 #define X(SS) \
     case SS: return launch_S<SS>(p, plan, vis, weight, taps, tables, grid, num_sms, s);
         SEPW_FOR_EACH_WIN_S(X)
+#undef X
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+// supports without a block degridder, but for 2, 6 and 14 (see the kernel)
+#define SEPW_FOR_EACH_DEGRID_S(X) X(10) X(18) X(20) X(22) X(24) X(26) X(28) X(30) X(32)
+
+bool degrid_window_takes(const DevParams &p, const Plan &plan)
+{
+    if (!plan.window)
+        return false;
+    switch (p.S) {
+#define X(SS) case SS:
+        SEPW_FOR_EACH_DEGRID_S(X)
+#undef X
+        return true;
+    default: return false;
+    }
+}
+
+cudaError_t launch_degrid_window(const DevParams &p, const Plan &plan, const float2 *grid,
+                                 const float *weight, const float2 *taps, float *tables,
+                                 float2 *vis, int num_sms, cudaStream_t s)
+{
+    switch (p.S) {
+#define X(SS) \
+    case SS: return launch_degrid_S<SS>(p, plan, grid, weight, taps, tables, vis, num_sms, s);
+        SEPW_FOR_EACH_DEGRID_S(X)
 #undef X
     default: return cudaErrorInvalidValue;
     }

@@ -124,6 +124,25 @@ def test_non_finite_values_stay_in_their_footprints(env, support):
     want = O.grid_separable(p, dict(loc, keep=keep), wl.vis, wl.weight, T)
     rest = ~hit & ~huge
     assert rel_l2(grid[rest], want[rest]) <= TOL
+    # the same for prediction: a cell that is not finite reaches the footprints
+    # that hold it, and no others
+    model = np.random.default_rng(9).standard_normal((p.N, p.N, 2)).astype(np.float32)
+    model = model.view(np.complex64)[:, :, 0]
+    y0, x0 = loc["cv"][bad[0]] + 1, loc["cu"][bad[0]] - 1
+    model[y0, x0] = complex(np.inf, 0)
+    ctx = S.sepw_create(S.make_params(**wl.params(), form=S.FORM_TILED))
+    t0 = S.sepw_make_taps(ctx)
+    dd = _dev(torch, wl)
+    out = torch.empty(wl.nvis, dtype=torch.complex64, device="cuda")
+    S.sepw_degrid(ctx, t0, dd["u"], dd["v"], dd["w"], torch.from_numpy(model).cuda(),
+                  dd["weight"], out)
+    got = out.cpu().numpy()
+    fy, fx = loc["cv"] - p.S // 2 + 1, loc["cu"] - p.S // 2 + 1
+    holds = loc["keep"] & (fy <= y0) & (y0 < fy + p.S) & (fx <= x0) & (x0 < fx + p.S)
+    assert holds.any() and np.array_equal(~np.isfinite(got), holds)
+    clean = np.where(np.isfinite(model), model, 0)
+    pw = O.degrid_separable(p, loc, clean.astype(np.complex128), wl.weight, T)
+    assert rel_l2(got[~holds], pw[~holds]) <= TOL
     # a NaN tap: the same cells as the plain form, which reads no padded rows
     ctxs = [S.sepw_create(S.make_params(**wl.params(), form=f))
             for f in (S.FORM_PLAIN, S.FORM_TILED)]
