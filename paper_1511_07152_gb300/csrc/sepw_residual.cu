@@ -20,12 +20,13 @@
 //   B(x)    = sum_{beta = 0}^{N/2 - 1} C(x, beta) h(N/2, beta),
 //   C(x, beta) = (beta ? 2 : 1) cos(2 pi x beta / N)  (real).
 // The offsets are the multiples of 1/OSr from -Sr/2 + 1/OSr to Sr/2, so |d|
-// takes R/2 + 1 values for R = OSr Sr.  That leaves a sixteenth of the direct
-// sum's multiply-adds (half the alphas, betas and offsets, real by complex),
-// and one thread accumulates all rows of its alpha, so that a screen value is
-// computed once per (plane, alpha, beta) up to 33 rows.  N = 1024, 32 planes,
-// 8 x 8 cells, 8 x 8 offsets: the direct sum took 62.1 ms, this takes 2.4
-// (rows 2.21, columns 0.12, edge 0.06, table 0.01).
+// takes R/2 + 1 values for R = OSr Sr; and A(x, y) = M(x, y) + M(y, x) with M
+// summed over beta <= alpha alone (the diagonal by half).  That leaves a
+// thirty-second of the direct sum's multiply-adds (real by complex, too) and an
+// eighth of its screen values, since one thread accumulates all rows of its
+// alpha (up to 33).  N = 1024, 32 planes, 8 x 8 cells, 8 x 8 offsets: the
+// direct sum took 62.1 ms, all alpha and beta 2.4 ms (rows 2.21, columns 0.12,
+// edge 0.06, table 0.01), this 1.66 (rows 1.46).
 //
 // Pass: each warp takes work items of the plan; per visibility the lanes
 // cover the Sr^2 cells.  Gridding adds W V R (conj(R) for w < 0) with float2
@@ -80,9 +81,10 @@ __device__ __forceinline__ double plane_w(const DevParams &p, int plane)
     return p.P > 1 ? (double)plane * p.w_max / (double)(p.P - 1) : 0.0;
 }
 
-// Rows: Y[p][z][x][alpha] = sum over the z-th part of beta of C(x, beta)
-// h(alpha, beta), for G values of x from x0 (x >= R2: not written).
-// grid (ceil(N/2 / 64), P, parts * groups); block 64
+// Rows: Y[p][z][x][alpha] = sum over the z-th part of beta <= alpha of C(x, beta)
+// h(alpha, beta) (beta = alpha by half), for G values of x from x0 (x >= R2: not
+// written).  grid (ceil(N/2 / 64), P, parts * groups), the long sums first;
+// block 64
 constexpr int kResRowThreads = 64;
 
 template <int G>
@@ -91,13 +93,13 @@ __global__ void __launch_bounds__(kResRowThreads) residual_rows_kernel(
     const double *__restrict__ C, double2 *__restrict__ Y)
 {
     const int H = p.N / 2;
-    const int alpha = blockIdx.x * kResRowThreads + threadIdx.x;
+    const int alpha = (gridDim.x - 1 - blockIdx.x) * kResRowThreads + threadIdx.x;
     const int plane = blockIdx.y;
     const int z = blockIdx.z % parts, x0 = (blockIdx.z / parts) * G;
     if (alpha >= H)
         return;
     const int len = (H + parts - 1) / parts;
-    const int b0 = z * len, b1 = min(H, b0 + len);
+    const int b0 = z * len, b1 = min(alpha + 1, b0 + len);
     const double wp = plane_w(p, plane);
     const double l = (double)alpha / (double)p.N * p.fov;
     const double ca = taper64[H + alpha];
@@ -107,7 +109,7 @@ __global__ void __launch_bounds__(kResRowThreads) residual_rows_kernel(
         acc[q] = make_double2(0.0, 0.0);
     for (int beta = b0; beta < b1; ++beta) {
         const double2 e = screen(wp, l, (double)beta / (double)p.N * p.fov);
-        const double t = ca * taper64[H + beta];
+        const double t = ca * taper64[H + beta] * (beta == alpha ? 0.5 : 1.0);
         const double hr = t * e.x, hi = t * e.y;
         const double *c = C + (int64_t)beta * R2 + x0;
 #pragma unroll
@@ -163,14 +165,14 @@ __global__ void __launch_bounds__(256) residual_edge_kernel(DevParams p, int R2,
     }
 }
 
-// Columns: A[p][x][y] = sum_alpha Y[p][.][x][alpha] C(y, alpha).  A block
+// Columns: M[p][x][y] = sum_alpha Y[p][.][x][alpha] C(y, alpha).  A block
 // takes one (plane, x): the parts of Y are summed into shared memory, then
 // thread (g, y) sums its quarter of each chunk of alphas.
 // grid (R2, P); block (64, 4)
 __global__ void __launch_bounds__(256) residual_cols_kernel(DevParams p, int R2, int parts,
                                                             const double *__restrict__ C,
                                                             const double2 *__restrict__ Y,
-                                                            double2 *__restrict__ A)
+                                                            double2 *__restrict__ M)
 {
     constexpr int kCh = 512;
     __shared__ double2 ys[kCh];
@@ -208,16 +210,16 @@ __global__ void __launch_bounds__(256) residual_cols_kernel(DevParams p, int R2,
                 acc.x += red[q][threadIdx.x].x;
                 acc.y += red[q][threadIdx.x].y;
             }
-            A[((int64_t)plane * R2 + x) * R2 + y] = acc;
+            M[((int64_t)plane * R2 + x) * R2 + y] = acc;
         }
     }
 }
 
-// F_w from A and B, minus the separable product; writes the table.
+// F_w from M and B, minus the separable product; writes the table.
 // grid (ceil(R*R / 256), P); block 256
 __global__ void __launch_bounds__(256) residual_table_kernel(
     DevParams p, int Sr, int OSr, int R2, const double2 *__restrict__ tw,
-    const double2 *__restrict__ A, const double2 *__restrict__ B,
+    const double2 *__restrict__ M2, const double2 *__restrict__ B,
     const double2 *__restrict__ taps64, double2 *out64, float2 *out32)
 {
     const int R = OSr * Sr;
@@ -233,7 +235,9 @@ __global__ void __launch_bounds__(256) residual_table_kernel(
     const double2 ev = dft_tw(tw, M, dv, 0, p.N), eu = dft_tw(tw, M, du, 0, p.N);
     const double2 *b = B + (int64_t)plane * (R2 + 1);
     const double2 bu = b[xu], bv = b[xv], h = b[R2];
-    const double2 a = A[((int64_t)plane * R2 + xv) * R2 + xu];
+    const double2 *m2 = M2 + (int64_t)plane * R2 * R2;
+    const double2 a0 = m2[(int64_t)xv * R2 + xu], a1 = m2[(int64_t)xu * R2 + xv];
+    const double2 a = make_double2(a0.x + a1.x, a0.y + a1.y);
     // e(dv) (B(du) + e(du) h) + e(du) B(dv) + A
     const double tr = bu.x + (eu.x * h.x - eu.y * h.y), ti = bu.y + (eu.x * h.y + eu.y * h.x);
     double kr = a.x + (ev.x * tr - ev.y * ti) + (eu.x * bv.x - eu.y * bv.y);
