@@ -26,7 +26,7 @@
 // eighth of its screen values, since one thread accumulates all rows of its
 // alpha (up to 33).  N = 1024, 32 planes, 8 x 8 cells, 8 x 8 offsets: the
 // direct sum took 62.1 ms, all alpha and beta 2.4 ms (rows 2.21, columns 0.12,
-// edge 0.06, table 0.01), this 1.66 (rows 1.46).
+// edge 0.06, table 0.01), this 1.3 ms in all.
 //
 // Pass: each warp takes work items of the plan; per visibility the lanes
 // cover the Sr^2 cells.  Gridding adds W V R (conj(R) for w < 0) with float2
@@ -67,13 +67,30 @@ __global__ void __launch_bounds__(256) residual_cos_kernel(DevParams p, int OSr,
     C[e] = (beta ? 2.0 : 1.0) * tw[m].x;
 }
 
-__device__ __forceinline__ double2 screen(double wp, double l, double m)
+__device__ __forceinline__ double n_minus_1(double l, double m)
 {
     const double r2 = l * l + m * m;
-    const double nm1 = -r2 / (1.0 + sqrt(1.0 - r2));
+    return -r2 / (1.0 + sqrt(1.0 - r2));
+}
+
+__device__ __forceinline__ double2 screen(double wp, double nm1)
+{
     double s, c;
     sincospi(2.0 * (wp * nm1), &s, &c);
     return make_double2(c, s);
+}
+
+// The pixels' n - 1 once for all planes (its square root and division are a
+// fifth of the rows' FP64 operations): nm1[beta][alpha], beta <= alpha < N/2,
+// for N up to kNm1MaxN (2 N^2 bytes); beyond, the rows compute it.
+constexpr int kNm1MaxN = 8192;
+
+__global__ void __launch_bounds__(256) residual_nm1_kernel(DevParams p, double *nm1)
+{
+    const int H = p.N / 2, alpha = blockIdx.x * blockDim.x + threadIdx.x, beta = blockIdx.y;
+    if (alpha < H && beta <= alpha)
+        nm1[(int64_t)beta * H + alpha] = n_minus_1((double)alpha / (double)p.N * p.fov,
+                                                   (double)beta / (double)p.N * p.fov);
 }
 
 __device__ __forceinline__ double plane_w(const DevParams &p, int plane)
@@ -90,7 +107,7 @@ constexpr int kResRowThreads = 64;
 template <int G>
 __global__ void __launch_bounds__(kResRowThreads) residual_rows_kernel(
     DevParams p, int R2, int parts, const double *__restrict__ taper64,
-    const double *__restrict__ C, double2 *__restrict__ Y)
+    const double *__restrict__ C, const double *__restrict__ nm1, double2 *__restrict__ Y)
 {
     const int H = p.N / 2;
     const int alpha = (gridDim.x - 1 - blockIdx.x) * kResRowThreads + threadIdx.x;
@@ -108,7 +125,9 @@ __global__ void __launch_bounds__(kResRowThreads) residual_rows_kernel(
     for (int q = 0; q < G; ++q)
         acc[q] = make_double2(0.0, 0.0);
     for (int beta = b0; beta < b1; ++beta) {
-        const double2 e = screen(wp, l, (double)beta / (double)p.N * p.fov);
+        const double x = nm1 ? __ldg(nm1 + (int64_t)beta * H + alpha)
+                             : n_minus_1(l, (double)beta / (double)p.N * p.fov);
+        const double2 e = screen(wp, x);
         const double t = ca * taper64[H + beta] * (beta == alpha ? 0.5 : 1.0);
         const double hr = t * e.x, hi = t * e.y;
         const double *c = C + (int64_t)beta * R2 + x0;
@@ -143,7 +162,7 @@ __global__ void __launch_bounds__(256) residual_edge_kernel(DevParams p, int R2,
         for (int c0 = 0; c0 < H; c0 += 1024) {
             __syncthreads();
             for (int i = threadIdx.x; i < 1024 && c0 + i < H; i += blockDim.x) {
-                const double2 e = screen(wp, l, (double)(c0 + i) / (double)p.N * p.fov);
+                const double2 e = screen(wp, n_minus_1(l, (double)(c0 + i) / (double)p.N * p.fov));
                 const double t = ca * taper64[H + c0 + i];
                 h[i] = make_double2(t * e.x, t * e.y);
             }
@@ -160,7 +179,7 @@ __global__ void __launch_bounds__(256) residual_edge_kernel(DevParams p, int R2,
             B[(int64_t)plane * (R2 + 1) + x] = acc;
     }
     if (threadIdx.x == 0) {
-        const double2 e = screen(wp, l, l);
+        const double2 e = screen(wp, n_minus_1(l, l));
         B[(int64_t)plane * (R2 + 1) + R2] = make_double2(ca * ca * e.x, ca * ca * e.y);
     }
 }
@@ -258,11 +277,11 @@ __global__ void __launch_bounds__(256) residual_table_kernel(
         out32[idx] = make_float2((float)kr, (float)ki);
 }
 
-// workspace: C, then Y, A and B (double2)
+// workspace: Y, M and B (double2), then C and n - 1 (double)
 struct ResidualWork {
     int R2, parts;
-    size_t nC, nY, nA, nB;
-    size_t bytes() const { return sizeof(double2) * ((nC + 1) / 2 + nY + nA + nB); }
+    size_t nC, nY, nA, nB, nNm1;
+    size_t bytes() const { return sizeof(double2) * (nY + nA + nB) + sizeof(double) * (nC + nNm1); }
 };
 
 static ResidualWork residual_work(const DevParams &p, int Sr, int OSr)
@@ -278,6 +297,7 @@ static ResidualWork residual_work(const DevParams &p, int Sr, int OSr)
     w.nY = (size_t)p.P * w.parts * w.R2 * H;
     w.nA = (size_t)p.P * w.R2 * w.R2;
     w.nB = (size_t)p.P * (w.R2 + 1);
+    w.nNm1 = p.N <= kNm1MaxN ? H * H : 0;
     return w;
 }
 
@@ -299,16 +319,23 @@ cudaError_t launch_residual_table(const DevParams &p, int Sr, int OSr, const dou
                                                                                 C);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
+    double *nm1 = nullptr;
+    if (w.nNm1) {
+        nm1 = C + w.nC;
+        residual_nm1_kernel<<<dim3((H + 255) / 256, H), 256, 0, s>>>(p, nm1);
+        if ((e = cudaGetLastError()) != cudaSuccess)
+            return e;
+    }
     const unsigned gx = (H + kResRowThreads - 1) / kResRowThreads;
     if (R2 <= 9)
         residual_rows_kernel<9><<<dim3(gx, p.P, w.parts), kResRowThreads, 0, s>>>(
-            p, R2, w.parts, taper64, C, Y);
+            p, R2, w.parts, taper64, C, nm1, Y);
     else if (R2 <= 17)
         residual_rows_kernel<17><<<dim3(gx, p.P, w.parts), kResRowThreads, 0, s>>>(
-            p, R2, w.parts, taper64, C, Y);
+            p, R2, w.parts, taper64, C, nm1, Y);
     else
         residual_rows_kernel<33><<<dim3(gx, p.P, w.parts * ((R2 + 32) / 33)), kResRowThreads, 0,
-                                   s>>>(p, R2, w.parts, taper64, C, Y);
+                                   s>>>(p, R2, w.parts, taper64, C, nm1, Y);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return e;
     residual_edge_kernel<<<p.P, 256, 0, s>>>(p, R2, taper64, C, B);
@@ -374,8 +401,7 @@ __device__ __forceinline__ uint32_t res_entry(uint64_t r, int OSr, int step)
 template <int PPL, bool VEC>
 __global__ void __launch_bounds__(kResWarps * 32) grid_residual_kernel(
     DevParams p, int Sr, int OSr, const WorkItem *__restrict__ items,
-    const int32_t *__restrict__ nitems, int32_t *counter, const uint64_t *__restrict__ rec,
-    const int32_t *__restrict__ perm, const float2 *__restrict__ vis,
+    const int32_t *__restrict__ nitems, int32_t *counter, const Slot *__restrict__ slots, const float2 *__restrict__ vis,
     const float *__restrict__ weight, const float2 *__restrict__ res, float2 *grid)
 {
     __shared__ float4 s_meta[kResWarps * 32];  // entry, key, W V
@@ -429,8 +455,9 @@ __global__ void __launch_bounds__(kResWarps * 32) grid_residual_kernel(
             const int s = base + lane;
             int kq = -1;
             if (s < b1) {
-                const uint64_t r = rec[s];
-                const int i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                const uint64_t r = slot.rec;
+                const int i = slot.vis;
                 const float wt = weight ? __ldg(weight + i) : 1.0f;
                 const float2 x = __ldg(vis + i);
                 const bool cj = rec_conj(r);
@@ -498,8 +525,7 @@ __device__ __forceinline__ void res_reduce8(float (&v)[8], int lane)
 template <int PPL, bool VEC>
 __global__ void __launch_bounds__(kResWarps * 32) degrid_residual_kernel(
     DevParams p, int Sr, int OSr, const WorkItem *__restrict__ items,
-    const int32_t *__restrict__ nitems, int32_t *counter, const uint64_t *__restrict__ rec,
-    const int32_t *__restrict__ perm, const float2 *__restrict__ grid,
+    const int32_t *__restrict__ nitems, int32_t *counter, const Slot *__restrict__ slots, const float2 *__restrict__ grid,
     const float *__restrict__ weight, const float2 *__restrict__ res, float2 *vis_out)
 {
     constexpr int G = PPL == 1 ? 8 : PPL == 2 ? 4 : PPL <= 4 ? 2 : 1;  // entries in flight
@@ -541,8 +567,9 @@ __global__ void __launch_bounds__(kResWarps * 32) degrid_residual_kernel(
             float wt = 0.f;
             float2 old = make_float2(0.f, 0.f);
             if (s < b1) {
-                const uint64_t r = rec[s];
-                i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                const uint64_t r = slot.rec;
+                i = slot.vis;
                 wt = weight ? __ldg(weight + i) : 1.0f;
                 old = vis_out[i];
                 meta[lane] = make_uint2(res_entry(r, OSr, step),
@@ -637,8 +664,7 @@ cudaError_t launch_grid_residual(const DevParams &p, int Sr, int OSr, const Plan
     if (ppl <= PPL) {                                                                       \
         (vec ? grid_residual_kernel<PPL, true> : grid_residual_kernel<PPL, false>)          \
             <<<num_sms * kResBlocksPerSM, kResWarps * 32, 0, s>>>(                          \
-                p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec,   \
-                plan.d_perm, vis, weight, res, grid);                                       \
+                p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_slots, vis, weight, res, grid);                                       \
         return cudaGetLastError();                                                          \
     }
     SEPW_FOR_EACH_PPL(X)
@@ -659,8 +685,7 @@ cudaError_t launch_degrid_residual(const DevParams &p, int Sr, int OSr, const Pl
     if (ppl <= PPL) {                                                                       \
         (vec ? degrid_residual_kernel<PPL, true> : degrid_residual_kernel<PPL, false>)      \
             <<<num_sms * kResBlocksPerSM, kResWarps * 32, 0, s>>>(                          \
-                p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec, \
-                plan.d_perm, grid, weight, res, vis_out);                                   \
+                p, Sr, OSr, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_slots, grid, weight, res, vis_out);                                   \
         return cudaGetLastError();                                                          \
     }
     SEPW_FOR_EACH_PPL(X)
