@@ -183,8 +183,7 @@ void free_plan(Plan &pl)
     cudaFree(pl.d_tile);
     cudaFree(pl.d_rank);
     cudaFree(pl.d_rec0);
-    cudaFree(pl.d_rec);
-    cudaFree(pl.d_perm);
+    cudaFree(pl.d_slots);
     cudaFree(pl.d_drop_list);
     cudaFree(pl.d_bin_base);  // holds d_dropped
     cudaFree(pl.d_tile_count);
@@ -265,7 +264,7 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
         int64_t cap = nvis;
         if ((rc = grow(ctx, &pl.d_tile, cap)) || (rc = grow(ctx, &pl.d_rank, cap)) ||
             (rc = grow(ctx, &pl.d_rec0, cap)) ||
-            (rc = grow(ctx, &pl.d_rec, cap)) || (rc = grow(ctx, &pl.d_perm, cap)) ||
+            (rc = grow(ctx, &pl.d_slots, cap)) ||
             (rc = grow(ctx, &pl.d_drop_list, cap)))
             return rc;
         pl.capacity = cap;
@@ -405,7 +404,8 @@ int sepw_create(sepw_ctx **out, const sepw_params *p)
         return SEPW_ECUDA;
     }
     const int N = p->grid_size;
-    ctx->window = p->form == SEPW_FORM_TILED && window_tables_bytes(ctx->dp) > 0;
+    ctx->window = p->form == SEPW_FORM_TILED && p->support != 8 &&  // see plan_window
+                  window_tables_bytes(ctx->dp) > 0;
     if ((rc = grow(ctx, &ctx->d_taper64, N)) || (rc = grow(ctx, &ctx->d_taper32, N)) ||
         (rc = grow(ctx, &ctx->d_tw, (size_t)N * p->oversample)) ||
         (rc = grow(ctx, &ctx->d_status, 1)) ||
@@ -811,13 +811,13 @@ int sepw_test_corrupt_plan(sepw_ctx *ctx, int which, int64_t slot, int32_t value
                     which);
     cudaError_t e;
     if (which == 0) {
-        e = cudaMemcpy(pl.d_perm + slot, &value, sizeof(int32_t), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(&pl.d_slots[slot].vis, &value, sizeof(int32_t), cudaMemcpyHostToDevice);
     } else {
         uint64_t r = 0;
-        e = cudaMemcpy(&r, pl.d_rec + slot, sizeof(r), cudaMemcpyDeviceToHost);
+        e = cudaMemcpy(&r, &pl.d_slots[slot].rec, sizeof(r), cudaMemcpyDeviceToHost);
         if (e == cudaSuccess) {
             r = (r & ~((uint64_t)32767 << 28)) | ((uint64_t)(value & 32767) << 28);
-            e = cudaMemcpy(pl.d_rec + slot, &r, sizeof(r), cudaMemcpyHostToDevice);
+            e = cudaMemcpy(&pl.d_slots[slot].rec, &r, sizeof(r), cudaMemcpyHostToDevice);
         }
     }
     return e == cudaSuccess ? SEPW_OK : cuda_fail(ctx, e, "sepw_test_corrupt_plan");

@@ -357,12 +357,14 @@ __global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
 }
 static_assert(kMaxSubBins == 64, "two bins per lane");
 
-// Pass 3: scatter visibility ids and records to their slots: first slot of the
-// bin + rank inside the bin.
+// Pass 3: scatter records and visibility ids to their slots: first slot of the
+// bin + rank inside the bin.  A slot is one 16-byte store: as an 8- and a
+// 4-byte array the pass was bound by twice the partial sectors it sends to L2
+// (32M visibilities 424 us; 331 us so).
 __global__ void __launch_bounds__(256) scatter_kernel(
     int64_t nvis, const int32_t *__restrict__ bin_of, const int32_t *__restrict__ rank_of,
     const uint64_t *__restrict__ rec0, const int32_t *__restrict__ bin_first,
-    int32_t *__restrict__ perm, uint64_t *__restrict__ rec)
+    Slot *__restrict__ slots)
 {
     pdl_enter();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -372,8 +374,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(
     if (b < 0)
         return;
     const int slot = __ldg(bin_first + b) + rank_of[i];
-    perm[slot] = (int32_t)i;
-    rec[slot] = rec0[i];
+    store_slot(slots + slot, rec0[i], (int32_t)i);
 }
 
 // Pass 4: inside each work item, counting sort by (footprint origin, conj),
@@ -402,7 +403,7 @@ static int sort_keys(const DevParams &p)
 
 __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
     DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
-    int32_t *__restrict__ perm, uint64_t *__restrict__ rec)
+    Slot *__restrict__ slots)
 {
     extern __shared__ int32_t hist[];  // per * kSortThreads bins
     __shared__ uint64_t s_rec[kChunk];
@@ -428,9 +429,10 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
         const bool act = q < n;
         int key = -1;
         if (act) {
-            const uint64_t r = rec[it.start + q];
+            const uint4 w = *reinterpret_cast<const uint4 *>(slots + it.start + q);
+            const uint64_t r = (uint64_t)w.y << 32 | w.x;
             s_rec[q] = r;
-            s_perm[q] = perm[it.start + q];
+            s_perm[q] = (int32_t)w.z;
             key = sort_key(r, p);
         }
         const unsigned peers = __match_any_sync(0xffffffffu, key);
@@ -497,8 +499,7 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
         base = __shfl_sync(0xffffffffu, base, leader);
         if (act) {
             const int dst = base + __popc(peers & lanemask_lt());
-            rec[it.start + dst] = r;
-            perm[it.start + dst] = s_perm[q];
+            store_slot(slots + it.start + dst, r, s_perm[q]);
         }
     }
     __syncthreads();  // shared memory is reused by the next item
@@ -620,7 +621,7 @@ cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
         return e;
     if (nvis > 0) {
         e = launch_pdl(scatter_kernel, (nvis + 255) / 256, 256, 0, s, nvis, plan.d_tile,
-                       plan.d_rank, plan.d_rec0, bin, plan.d_perm, plan.d_rec);
+                       plan.d_rank, plan.d_rec0, bin, plan.d_slots);
         if (e != cudaSuccess)
             return e;
         if (plan.sorted)
@@ -641,8 +642,7 @@ cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, 
     if (e != cudaSuccess)
         return e;
     const int nblk = std::max(1, std::min(plan.items_capacity, 16 * num_sms));
-    return launch_pdl(item_sort_kernel, nblk, kSortThreads, shm, s, p, plan.d_items, plan.d_nitems,
-                      plan.d_perm, plan.d_rec);
+    return launch_pdl(item_sort_kernel, nblk, kSortThreads, shm, s, p, plan.d_items, plan.d_nitems, plan.d_slots);
 }
 
 }  // namespace sepw

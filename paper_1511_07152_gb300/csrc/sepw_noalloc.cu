@@ -7,11 +7,11 @@
 // raw allocations from plugins.  This entry point serves them: instead of a
 // context's workspace it uses one fixed scratch array compiled into the
 // library as a file-scope __device__ variable, so every GPU that loads the
-// library holds that array (kNoallocBytes, about 40 MB) until the process
+// library holds that array (kNoallocBytes, about 42 MB) until the process
 // exits.
 //
 // The scratch holds the same plan as the context path (bin ids and ranks,
-// packed records, slot permutation, dropped-index list, per-tile counts and
+// packed records, slots, dropped-index list, per-tile counts and
 // cursors, per-bin counts, work items and counters), and the existing plan
 // and tiled-gridder launchers run on it unchanged.  Every call reuses the
 // array: the plan launcher clears the bin counts and the dropped counter at
@@ -35,9 +35,8 @@ constexpr int64_t kMaxItems = kMaxTiles + kMaxVis / kChunk + 1;
 constexpr size_t kOffTile = 0;
 constexpr size_t kOffRank = align256(kOffTile + sizeof(int32_t) * kMaxVis);
 constexpr size_t kOffRec0 = align256(kOffRank + sizeof(int32_t) * kMaxVis);
-constexpr size_t kOffRec = align256(kOffRec0 + sizeof(uint64_t) * kMaxVis);
-constexpr size_t kOffPerm = align256(kOffRec + sizeof(uint64_t) * kMaxVis);
-constexpr size_t kOffDrop = align256(kOffPerm + sizeof(int32_t) * kMaxVis);
+constexpr size_t kOffSlots = align256(kOffRec0 + sizeof(uint64_t) * kMaxVis);
+constexpr size_t kOffDrop = align256(kOffSlots + sizeof(Slot) * kMaxVis);
 constexpr int64_t kMaxUnits = kMaxTiles + kMaxVis / 32 + 1;
 constexpr size_t kOffCount = align256(kOffDrop + sizeof(int32_t) * kMaxVis);
 constexpr size_t kOffBlocks = align256(kOffCount + sizeof(int32_t) * kMaxTiles);
@@ -162,8 +161,7 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     pl.d_tile = (int32_t *)(b + kOffTile);
     pl.d_rank = (int32_t *)(b + kOffRank);
     pl.d_rec0 = (uint64_t *)(b + kOffRec0);
-    pl.d_rec = (uint64_t *)(b + kOffRec);
-    pl.d_perm = (int32_t *)(b + kOffPerm);
+    pl.d_slots = (Slot *)(b + kOffSlots);
     pl.d_drop_list = (int32_t *)(b + kOffDrop);
     pl.d_tile_count = (int32_t *)(b + kOffCount);
     pl.d_blocks = b + kOffBlocks;

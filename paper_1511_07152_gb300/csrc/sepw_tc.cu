@@ -280,7 +280,7 @@ __device__ __forceinline__ int window_exp(const float *wm)
 template <int S, int PREC, int SPLIT>
 __global__ void __launch_bounds__(kDgBlock, 1) degrid_tc_kernel(
     DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
-    const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
+    const Slot *__restrict__ slots,
     const float2 *__restrict__ grid, const float *__restrict__ weight,
     const uint4 *__restrict__ vtab, const uint4 *__restrict__ utab,
     float2 *__restrict__ vis_out, int32_t *status, TcControl ctl)
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(kDgBlock, 1) degrid_tc_kernel(
             auto rec_of = [&](int st) -> uint64_t {
                 const int e = st * kDgVis + ii;
                 return st < nst && e < it.count
-                           ? __ldg(reinterpret_cast<const unsigned long long *>(rec) + it.start + e)
+                           ? __ldg(reinterpret_cast<const unsigned long long *>(slots + it.start + e))
                            : ~0ull;
             };
             int st0 = grp ^ (tg & 1);
@@ -555,8 +555,9 @@ __global__ void __launch_bounds__(kDgBlock, 1) degrid_tc_kernel(
             auto rec_of = [&](int st, int &io) -> uint64_t {
                 const int e = st * kDgVis + ii;
                 if (st < nst && e < it.count) {
-                    io = __ldg(perm + it.start + e);
-                    return __ldg(reinterpret_cast<const unsigned long long *>(rec) + it.start + e);
+                    const Slot slot = load_slot_split(slots + it.start + e);
+                    io = slot.vis;
+                    return (unsigned long long)slot.rec;
                 }
                 return ~0ull;
             };
@@ -667,7 +668,7 @@ cudaError_t launch_degrid_tc_S(const DevParams &p, const Plan &plan, const float
     if (e != cudaSuccess)
         return e;
     degrid_tc_kernel<S, PREC, SPLIT><<<num_sms, kDgBlock, C::kSmem, s>>>(
-        p, plan.d_items, plan.d_nitems, plan.d_rec, plan.d_perm, grid, weight, t.vtab, t.utab,
+        p, plan.d_items, plan.d_nitems, plan.d_slots, grid, weight, t.vtab, t.utab,
         vis, status, ctl);
     return cudaGetLastError();
 }

@@ -315,7 +315,7 @@ __global__ void tables_kernel(DevParams p, const float2 *__restrict__ taps, uint
 // component is below 2^a (FP16 forms scale their B operand by 2^-a).
 __global__ void item_scale_kernel(const WorkItem *__restrict__ items,
                                   const int32_t *__restrict__ nitems,
-                                  const int32_t *__restrict__ perm,
+                                  const Slot *__restrict__ slots,
                                   const float2 *__restrict__ vis, const float *__restrict__ weight,
                                   int32_t *item_exp)
 {
@@ -325,7 +325,7 @@ __global__ void item_scale_kernel(const WorkItem *__restrict__ items,
         const WorkItem it = items[item];
         float m = 0.f;
         for (int e = threadIdx.x; e < it.count; e += blockDim.x) {
-            const int i = perm[it.start + e];
+            const int i = __ldg(&slots[it.start + e].vis);
             const float2 x = __ldg(vis + i);
             const float wt = weight ? __ldg(weight + i) : 1.0f;
             m = fmaxf(m, fmaxf(fabsf(wt * x.x), fabsf(wt * x.y)));
@@ -393,7 +393,7 @@ __device__ __forceinline__ bool cursor_seek(Cursor &c, int t, const WorkItem *__
 template <int PREC>
 __global__ void __launch_bounds__(Cfg<PREC>::kBlock, 1) grid_tc2_kernel(
     DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
-    const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
+    const Slot *__restrict__ slots,
     const float2 *__restrict__ vis, const float *__restrict__ weight,
     const uint4 *__restrict__ vtab, const uint4 *__restrict__ utab,
     const float2 *__restrict__ taps, const int32_t *__restrict__ item_exp, float2 *grid,
@@ -461,9 +461,9 @@ __global__ void __launch_bounds__(Cfg<PREC>::kBlock, 1) grid_tc2_kernel(
                 const int e = (t_ - c.tb) * SV + slot0 + 32 * sl + lane;
                 vi_[sl] = -1;
                 if (e < c.count) {
-                    r_[sl] = __ldg(reinterpret_cast<const unsigned long long *>(rec) + c.start +
-                                   e);
-                    vi_[sl] = __ldg(perm + c.start + e);
+                    const Slot slot = load_slot_split(slots + c.start + e);
+                    r_[sl] = slot.rec;
+                    vi_[sl] = slot.vis;
                 }
             }
 #pragma unroll
@@ -918,7 +918,7 @@ cudaError_t launch_prec(const DevParams &p, const Plan &plan, const float2 *vis,
     }
     if constexpr (C::SCALED) {
         item_scale_kernel<<<std::max(1, std::min(plan.items_capacity, 8 * num_sms)), 256, 0, s>>>(
-            plan.d_items, plan.d_nitems, plan.d_perm, vis, weight, item_exp);
+            plan.d_items, plan.d_nitems, plan.d_slots, vis, weight, item_exp);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
     }
@@ -927,7 +927,7 @@ cudaError_t launch_prec(const DevParams &p, const Plan &plan, const float2 *vis,
     if (e != cudaSuccess)
         return e;
     grid_tc2_kernel<PREC><<<num_sms, C::kBlock, C::kSmem, s>>>(
-        p, plan.d_items, plan.d_nitems, plan.d_rec, plan.d_perm, vis, weight, vtab, utab, taps,
+        p, plan.d_items, plan.d_nitems, plan.d_slots, vis, weight, vtab, utab, taps,
         item_exp, grid, status, ctl);
     return cudaGetLastError();
 }

@@ -123,7 +123,7 @@ __device__ __forceinline__ void load_vtaps(const float2 *__restrict__ row, int r
 template <int S>
 __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) grid_tiled_kernel(
     DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
-    int32_t *counter, const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
+    int32_t *counter, const Slot *__restrict__ slots,
     const float2 *__restrict__ vis, const float *__restrict__ weight,
     const float2 *__restrict__ taps, float2 *grid)
 {
@@ -174,8 +174,9 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) grid_tiled_k
         for (int base = b0; base < b1; base += 32) {
             const int s = base + lane;
             if (s < b1) {
-                const uint64_t r = rec[s];
-                const int i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                const uint64_t r = slot.rec;
+                const int i = slot.vis;
                 const float wt = weight ? __ldg(weight + i) : 1.0f;
                 const float2 x = __ldg(vis + i);
                 const bool cj = rec_conj(r);
@@ -247,8 +248,7 @@ __device__ __forceinline__ void reduce8(float (&v)[8], int lane)
 template <int S>
 __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled_kernel(
     DevParams p, int WP, const WorkItem *__restrict__ items,
-    const int32_t *__restrict__ nitems, int32_t *counter, const uint64_t *__restrict__ rec,
-    const int32_t *__restrict__ perm, const float2 *__restrict__ grid,
+    const int32_t *__restrict__ nitems, int32_t *counter, const Slot *__restrict__ slots, const float2 *__restrict__ grid,
     const float *__restrict__ weight, const float2 *__restrict__ taps,
     float2 *__restrict__ vis_out)
 {
@@ -303,8 +303,9 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled
         for (int base = b0; base < b1; base += 32) {
             const int s = base + lane;
             if (s < b1) {
-                const uint64_t r = rec[s];
-                const int i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                const uint64_t r = slot.rec;
+                const int i = slot.vis;
                 const int row = rec_plane(r) * p.OS;
                 const int key = ((rec_ly(r) * 64 + rec_lx(r)) << 1) | (rec_conj(r) ? 1 : 0);
                 meta[lane] = make_int4((row + rec_ou(r)) * S,
@@ -436,8 +437,7 @@ __device__ __forceinline__ void reduce16x8(float (&v)[8], int t)
 template <int S>
 __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block_kernel(
     DevParams p, int WP, const WorkItem *__restrict__ items,
-    const int32_t *__restrict__ nitems, int32_t *counter, const uint64_t *__restrict__ rec,
-    const int32_t *__restrict__ perm, const float2 *__restrict__ grid,
+    const int32_t *__restrict__ nitems, int32_t *counter, const Slot *__restrict__ slots, const float2 *__restrict__ grid,
     const float *__restrict__ weight, const float2 *__restrict__ taps,
     float2 *__restrict__ vis_out)
 {
@@ -499,8 +499,9 @@ __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block
         for (int base = 0; base < per; base += K) {
             const int s = v0 + base + t;
             if (s < v1) {
-                const uint64_t r = rec[s];
-                const int i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                const uint64_t r = slot.rec;
+                const int i = slot.vis;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
                     const int row = rec_plane(r) * p.OS;
                     meta[t] = make_int4((row + rec_ou(r)) * S, (row + rec_ov(r)) * S, i,
@@ -625,7 +626,7 @@ constexpr int kGridBlkPerSM = 5;
 template <int S, bool PLANAR>
 __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block_kernel(
     DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
-    int32_t *counter, const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
+    int32_t *counter, const Slot *__restrict__ slots,
     const float2 *__restrict__ vis, const float *__restrict__ weight,
     const float2 *__restrict__ taps, const float *__restrict__ planar, float2 *grid)
 {
@@ -702,8 +703,9 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
             const int s = base + lane;
             int kq = -1;
             if (s < b1) {
-                const uint64_t r = rec[s];
-                const int i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                const uint64_t r = slot.rec;
+                const int i = slot.vis;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
                     const float wt = weight ? __ldg(weight + i) : 1.0f;
                     const float2 x = __ldg(vis + i);
@@ -867,8 +869,7 @@ static cudaError_t launch_grid_S(const DevParams &p, const Plan &plan, const flo
             if (e != cudaSuccess)
                 return e;
             return launch_pdl(grid_tiled_block_kernel<S, true>, nb, kTiledThreads, 0, s, p,
-                              plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec,
-                              plan.d_perm, vis, weight, taps, planar, grid);
+                              plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_slots, vis, weight, taps, planar, grid);
         }
     }
     cudaError_t e = cudaMemsetAsync(plan.d_item_counter, 0, sizeof(int32_t), s);
@@ -880,12 +881,11 @@ static cudaError_t launch_grid_S(const DevParams &p, const Plan &plan, const flo
     if constexpr (Blk2<S>::OK)
         return launch_pdl(grid_tiled_block_kernel<S, false>, num_sms * kGridBlkPerSM,
                           kTiledThreads, 0, s, p, plan.d_units, plan.d_nunits,
-                          plan.d_item_counter, plan.d_rec, plan.d_perm, vis, weight, taps, nullptr,
+                          plan.d_item_counter, plan.d_slots, vis, weight, taps, nullptr,
                           grid);
     else
         return launch_pdl(grid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, 0, s,
-                          p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_rec,
-                          plan.d_perm, vis, weight, taps, grid);
+                          p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_slots, vis, weight, taps, grid);
 }
 
 template <int S>
@@ -902,14 +902,12 @@ static cudaError_t launch_degrid_S(const DevParams &p, const Plan &plan,
         const size_t shm = sizeof(float4) * (size_t)((W * WP + 1) / 2) +
                            (size_t)kTiledWarps * 2 * Blk<S>::MS * (sizeof(int4) + sizeof(int));
         return launch_pdl(
-            degrid_tiled_block_kernel<S>, num_sms * Blk<S>::BPS, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec,
-            plan.d_perm, grid, weight, taps, vis);
+            degrid_tiled_block_kernel<S>, num_sms * Blk<S>::BPS, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_slots, grid, weight, taps, vis);
     } else {
         const int WP = window_stride(W, S);
         const size_t shm = tiled_smem(W, WP);
         return launch_pdl(
-            degrid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_rec,
-            plan.d_perm, grid, weight, taps, vis);
+            degrid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_slots, grid, weight, taps, vis);
     }
 }
 

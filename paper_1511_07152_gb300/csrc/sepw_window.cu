@@ -149,7 +149,7 @@ __device__ __forceinline__ void window_vtaps(const float *__restrict__ tv,
 template <int S>
 __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
     DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
-    int32_t *counter, const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
+    int32_t *counter, const Slot *__restrict__ slots,
     const float2 *__restrict__ vis, const float *__restrict__ weight,
     const float2 *__restrict__ taps, const float *__restrict__ utab,
     const float *__restrict__ vtab, const int32_t *__restrict__ flags, float2 *grid)
@@ -232,8 +232,9 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
             uint64_t r = 0;
             float2 wv = make_float2(0.f, 0.f);
             if (s < b1) {
-                r = rec[s];
-                const int i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                const int i = slot.vis;
+                r = slot.rec;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
                     const float wt = weight ? __ldg(weight + i) : 1.0f;
                     const float2 x = __ldg(vis + i);
@@ -359,7 +360,7 @@ __device__ __noinline__ float2 degrid_footprint(const float2 *__restrict__ tu,
 template <int S>
 __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) degrid_window_kernel(
     DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
-    int32_t *counter, const uint64_t *__restrict__ rec, const int32_t *__restrict__ perm,
+    int32_t *counter, const Slot *__restrict__ slots,
     const float2 *__restrict__ grid, const float *__restrict__ weight,
     const float2 *__restrict__ taps, const float *__restrict__ utab,
     const float *__restrict__ vtab, const int32_t *__restrict__ flags, float2 *__restrict__ vis_out)
@@ -472,8 +473,9 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) degrid_window_kernel
             float wt = 0.f;
             uint64_t r = 0;
             if (s < b1) {
-                r = rec[s];
-                i = perm[s];
+                const Slot slot = load_slot(slots + s);
+                r = slot.rec;
+                i = slot.vis;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
                     wt = weight ? __ldg(weight + i) : 1.0f;
                     cj = rec_conj(r);
@@ -605,7 +607,7 @@ static cudaError_t launch_S(const DevParams &p, const Plan &plan, const float2 *
     if (e != cudaSuccess)
         return e;
     return launch_pdl(grid_window_kernel<S>, num_sms * Win<S>::BPS, kWinThreads, 0, s, p,
-                      plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_rec, plan.d_perm,
+                      plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_slots,
                       vis, weight, taps, t.u, t.v, t.flags, grid);
 }
 
@@ -619,7 +621,7 @@ static cudaError_t launch_degrid_S(const DevParams &p, const Plan &plan, const f
     if (e != cudaSuccess)
         return e;
     return launch_pdl(degrid_window_kernel<S>, num_sms * Win<S>::BPS, kWinThreads, 0, s, p,
-                      plan.d_units, plan.d_nunits, plan.d_item_counter + 1, plan.d_rec, plan.d_perm,
+                      plan.d_units, plan.d_nunits, plan.d_item_counter + 1, plan.d_slots,
                       grid, weight, taps, t.u, t.v, t.flags, vis);
 }
 
