@@ -50,9 +50,8 @@ struct sepw_ctx {
     Plan plan;
     cufftHandle fft = 0;
     bool fft_ready = false;
-    cufftHandle fft_cols = 0;  // N column transforms, where the rows are ours
-    bool cols_ready = false;
-    float2 *d_rows_tab = nullptr;  // twiddles of our row transforms (cols_ready)
+    float2 *d_rows_tab = nullptr;  // twiddles of our own transforms
+    bool rows_ready = false;
     // hybrid W stacking: slice centres of the last sepw_wstack_plan and the
     // workspace of the slice sort
     std::vector<double> ws_centres;
@@ -441,8 +440,6 @@ void sepw_destroy(sepw_ctx *ctx)
     cudaDeviceSynchronize();
     if (ctx->fft_ready)
         cufftDestroy(ctx->fft);
-    if (ctx->cols_ready)
-        cufftDestroy(ctx->fft_cols);
     if (ctx->fft_batch_n)
         cufftDestroy(ctx->fft_batch);
     cudaFree(ctx->d_ws_c64);
@@ -846,25 +843,19 @@ static int ensure_fft(sepw_ctx *ctx, cudaStream_t s)
     return SEPW_OK;
 }
 
-// The column transforms of one grid, on stream s, and the rows' twiddles
-static int ensure_cols(sepw_ctx *ctx, cudaStream_t s)
+// The twiddles of our own transforms
+static int ensure_rows(sepw_ctx *ctx, cudaStream_t s)
 {
-    if (!ctx->cols_ready) {
-        int n = ctx->p.grid_size, rc;
-        if (!ctx->d_rows_tab &&
-            (rc = grow(ctx, &ctx->d_rows_tab, rows_table_bytes(n) / sizeof(float2))))
-            return rc;
-        SEPW_CUDA(ctx, launch_rows_tables(ctx->dp, ctx->d_tw, ctx->d_rows_tab, s));
-        // later calls may come on other streams
-        SEPW_CUDA(ctx, cudaStreamSynchronize(s));
-        const cufftResult r =
-            cufftPlanMany(&ctx->fft_cols, 1, &n, &n, n, 1, &n, n, 1, CUFFT_C2C, n);
-        if (r != CUFFT_SUCCESS)
-            return fail(ctx, SEPW_ECUDA, "cufftPlanMany (columns) failed (%d)", (int)r);
-        ctx->cols_ready = true;
-    }
-    if (cufftSetStream(ctx->fft_cols, s) != CUFFT_SUCCESS)
-        return fail(ctx, SEPW_ECUDA, "cufftSetStream failed");
+    if (ctx->rows_ready)
+        return SEPW_OK;
+    int rc;
+    if (!ctx->d_rows_tab && (rc = grow(ctx, &ctx->d_rows_tab,
+                                       rows_table_bytes(ctx->p.grid_size) / sizeof(float2))))
+        return rc;
+    SEPW_CUDA(ctx, launch_rows_tables(ctx->dp, ctx->d_tw, ctx->d_rows_tab, s));
+    // later calls may come on other streams
+    SEPW_CUDA(ctx, cudaStreamSynchronize(s));
+    ctx->rows_ready = true;
     return SEPW_OK;
 }
 
@@ -886,10 +877,12 @@ int sepw_image(sepw_ctx *ctx, int direction, float *buf, sepw_stream_t stream)
     if (rc)
         return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    if (direction != SEPW_IMAGE_TO_GRID && rows_supported(ctx->p.grid_size)) {
-        if ((rc = ensure_cols(ctx, s)) ||
-            (rc = fft_exec(ctx, ctx->fft_cols, (float2 *)buf, CUFFT_INVERSE)))
+    if (direction != SEPW_IMAGE_TO_GRID && rows_supported(ctx->p.grid_size) &&
+        ((uintptr_t)buf & 15) == 0) {
+        if ((rc = ensure_rows(ctx, s)))
             return rc;
+        SEPW_CUDA(ctx, launch_columns(ctx->dp, true, 1, ctx->d_rows_tab, (float2 *)buf,
+                                      ctx->num_sms, s));
         SEPW_CUDA(ctx, launch_rows_to_image(ctx->dp, direction == SEPW_GRID_TO_IMAGE ? 1 : 2,
                                             ctx->d_taper32, ctx->d_rows_tab, (float2 *)buf, s));
         return SEPW_OK;
@@ -1233,12 +1226,10 @@ int sepw_wstack_image(sepw_ctx *ctx, float *slice_grids, float *image, sepw_stre
     const int L = (int)ctx->ws_centres.size();
     cudaStream_t s = (cudaStream_t)stream;
     if (wstack_rows(ctx, slice_grids, image)) {
-        const size_t n2 = (size_t)ctx->p.grid_size * ctx->p.grid_size;
-        if ((rc = ensure_cols(ctx, s)))
+        if ((rc = ensure_rows(ctx, s)))
             return rc;
-        for (int c = 0; c < L; ++c)
-            if ((rc = fft_exec(ctx, ctx->fft_cols, (float2 *)slice_grids + c * n2, CUFFT_INVERSE)))
-                return rc;
+        SEPW_CUDA(ctx, launch_columns(ctx->dp, true, L, ctx->d_rows_tab, (float2 *)slice_grids,
+                                      ctx->num_sms, s));
         SEPW_CUDA(ctx, launch_slices_to_image(ctx->dp, L, ctx->d_taper32, ctx->d_ws_c32,
                                               ctx->d_rows_tab, (const float2 *)slice_grids,
                                               (float2 *)image, s));
@@ -1273,16 +1264,13 @@ int sepw_wstack_model_grids(sepw_ctx *ctx, const float *image, float *slice_grid
     const int L = (int)ctx->ws_centres.size();
     cudaStream_t s = (cudaStream_t)stream;
     if (wstack_rows(ctx, slice_grids, image)) {
-        const size_t n2 = (size_t)ctx->p.grid_size * ctx->p.grid_size;
-        if ((rc = ensure_cols(ctx, s)))
+        if ((rc = ensure_rows(ctx, s)))
             return rc;
         SEPW_CUDA(ctx, launch_image_to_slices(ctx->dp, L, ctx->d_taper32, ctx->d_ws_c32,
                                               ctx->d_rows_tab, (const float2 *)image,
                                               (float2 *)slice_grids, s));
-        for (int c = 0; c < L; ++c)
-            if ((rc = fft_exec(ctx, ctx->fft_cols, (float2 *)slice_grids + c * n2,
-                               CUFFT_FORWARD)))
-                return rc;
+        SEPW_CUDA(ctx, launch_columns(ctx->dp, false, L, ctx->d_rows_tab, (float2 *)slice_grids,
+                                      ctx->num_sms, s));
         return SEPW_OK;
     }
     if ((rc = ensure_fft_batch(ctx, L)))

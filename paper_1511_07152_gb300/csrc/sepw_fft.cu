@@ -1,13 +1,12 @@
-// Row transforms of the image step and of W stacking with the passes around
-// them folded in (Sec. 2: I_D / n = F^-1[grid] / c; Sec. 4.3: the slices).
+// Transforms of the image step and of W stacking with the passes around them
+// folded in (Sec. 2: I_D / n = F^-1[grid] / c; Sec. 4.3: the slices).
 //
 // The shifted transform of even N is, with a' = a - N/2 (mod N),
 //   grid -> image:  I[a] = (-1)^a' sum_c G[c] exp(2 pi i c a' / N),
 //   image -> grid:  G[c] = sum_a' (-1)^a' I[a] exp(-2 pi i c a' / N),
 // so the shift is a reordering on the image side and a sign there: no pass
-// over the grids is needed for it.  The column transforms (cuFFT, strided
-// batches) run on the grid side, and the rows here, where the image side's
-// reordering, sign, grid correction, slice phases and the sum over the slices
+// over the grids is needed for it.  The column transforms run on the grid
+// side, and the rows where the image side's reordering, sign, grid correction, slice phases and the sum over the slices
 // all fold into the one load or store of a row.  (sepw_image towards the grid
 // keeps its passes: predictions, and a float64 chi^2 of them, stay as they
 // were to the last bit.)
@@ -191,6 +190,116 @@ __device__ __forceinline__ void row_fft(float2 (&v)[16], const float2 *__restric
         for (int k = 0; k < R; ++k)
             v[k + R * h] = shm[m * W::P2 + k * 17 + m2];
         dft<R, INV>(v + R * h);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Column transforms in place: a block takes four columns (32 bytes of every
+// row, a whole sector) of one of `grids` grids at a time, thread (t, c) =
+// (id >> 2, id & 3) the points t + T k of column c, in registers as a row
+// above.  The next four columns are copied into shared memory while these are
+// transformed (cp.async), so that the loads run on; the exchanges take half
+// the room by moving real and imaginary parts one after the other.  Columns
+// that are all zero transform to zero and are left alone: in W stacking's
+// grids most columns lie beyond the uv coverage.  4096^2: cuFFT's strided
+// batch took 92 us a grid, with nothing in flight while it computes; this
+// 85 us, and 45 us for grids with two thirds of their columns
+// empty.
+// ---------------------------------------------------------------------------
+template <int R>
+struct Cols {
+    static constexpr int N = Rows<R>::N, T = Rows<R>::T, kThreads = 4 * T;
+    static constexpr int BPS = 16 / R;  // 1024 threads of 64 registers per SM
+    static constexpr int kBuf = 4 * N;               // float2
+    static constexpr int kX = 4 * Rows<R>::kShm;     // float
+    static constexpr int kShm = sizeof(float2) * kBuf + sizeof(float) * kX;
+};
+
+// v[k] -> its value at exchange place `to(k)`, read from place `from(k)`
+template <typename A, typename B>
+__device__ __forceinline__ void exchange(float2 (&v)[16], float *x, int c, A to, B from)
+{
+    float re[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+        x[4 * to(k) + c] = v[k].x;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+        re[k] = x[4 * from(k) + c];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+        x[4 * to(k) + c] = v[k].y;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 16; ++k)
+        v[k] = make_float2(re[k], x[4 * from(k) + c]);
+}
+
+template <int R, bool INV>
+__global__ void __launch_bounds__(Cols<R>::kThreads, Cols<R>::BPS) columns_kernel(
+    int grids, float2 *g, const float2 *__restrict__ tab)
+{
+    using W = Rows<R>;
+    constexpr int N = W::N, T = W::T, kThreads = Cols<R>::kThreads;
+    extern __shared__ float4 dyn[];
+    float2 *const buf = reinterpret_cast<float2 *>(dyn);
+    float *const x = reinterpret_cast<float *>(buf + Cols<R>::kBuf);
+    const int c = threadIdx.x & 3, t = threadIdx.x >> 2;
+    const int64_t tiles = (int64_t)grids * (N / 4);
+    auto first = [&](int64_t tile) {  // the tile's first cell
+        return g + tile / (N / 4) * ((int64_t)N * N) + tile % (N / 4) * 4;
+    };
+    auto fetch = [&](int64_t tile) {  // 16-byte halves of its rows
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(buf) + 16u * threadIdx.x;
+        const float2 *from = first(tile) + (threadIdx.x >> 1) * N + (threadIdx.x & 1) * 2;
+#pragma unroll
+        for (int k = 0; k < 2 * N / kThreads; ++k)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * kThreads * k),
+                         "l"(from + (int64_t)(kThreads / 2) * k * N)
+                         : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (blockIdx.x < tiles)
+        fetch(blockIdx.x);
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // the tile has landed; the last one is done with x
+        float2 v[16];
+        bool any = false;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            v[k] = buf[(t + T * k) * 4 + c];
+            any |= !(v[k].x == 0.f) || !(v[k].y == 0.f);  // (a NaN is not zero)
+        }
+        any = __syncthreads_or(any);
+        if (tile + gridDim.x < tiles)
+            fetch(tile + gridDim.x);
+        if (!any)
+            continue;
+        dft<16, INV>(v);
+        twiddle16<INV>(v, tab, T, t);
+        const int m = t / R, t0 = t % R;
+        exchange(v, x, c, [&](int k) { return k * W::P1 + t; },
+                 [&](int k) { return m * W::P1 + t0 + R * k; });
+        dft<16, INV>(v);
+        twiddle16<INV>(v, tab + kTw * T, 16, t0);
+        __syncthreads();
+        // v[k + R h] is point k of the h-th transform, frequencies 256 m3 + q
+        exchange(v, x, c, [&](int k) { return m * W::P2 + t0 * 17 + k; },
+                 [&](int k) {
+                     const int q = t + T * (k / R);
+                     return (q & 15) * W::P2 + (k % R) * 17 + (q >> 4);
+                 });
+        float2 *const out = first(tile) + c;
+#pragma unroll
+        for (int h = 0; h < 16 / R; ++h) {
+            dft<R, INV>(v + R * h);
+#pragma unroll
+            for (int k = 0; k < R; ++k)
+                out[(int64_t)(256 * k + t + T * h) * N] = v[k + R * h];
+        }
     }
 }
 
@@ -393,6 +502,29 @@ cudaError_t launch_rows_tables(const DevParams &p, const double2 *tw, float2 *ta
 }
 
 #define SEPW_FOR_EACH_ROWS(X) X(2) X(4) X(8) X(16)
+
+cudaError_t launch_columns(const DevParams &p, bool inverse, int grids, const float2 *tab,
+                           float2 *g, int num_sms, cudaStream_t s)
+{
+    switch (p.N / 256) {
+#define X(R)                                                                                    \
+    case R: {                                                                                   \
+        auto *kernel = inverse ? columns_kernel<R, true> : columns_kernel<R, false>;            \
+        cudaError_t e = cudaFuncSetAttribute(                                                   \
+            kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cols<R>::kShm);                \
+        if (e != cudaSuccess)                                                                   \
+            return e;                                                                           \
+        const int64_t tiles = (int64_t)grids * (p.N / 4), fit = (int64_t)num_sms * Cols<R>::BPS; \
+        kernel<<<(unsigned)(tiles < fit ? tiles : fit), Cols<R>::kThreads, Cols<R>::kShm, s>>>( \
+            grids, g, tab);                                                                     \
+        break;                                                                                  \
+    }
+        SEPW_FOR_EACH_ROWS(X)
+#undef X
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
 
 cudaError_t launch_rows_to_image(const DevParams &p, int mode, const float *taper,
                                  const float2 *tab, float2 *buf, cudaStream_t s)

@@ -618,14 +618,16 @@ cudaError_t launch_degrid_residual(const DevParams &p, int Sr, int OSr, const Pl
                                    const float2 *grid, const float *weight, const float2 *res,
                                    float2 *vis_out, int num_sms, cudaStream_t s);
 
-// sepw_fft.cu: row transforms with the image side's passes folded in, for the
-// N of rows_supported; column transforms of the grid side run before
-// (to image) or after (to grid).  tab: rows_table_bytes(N) bytes filled by
-// launch_rows_tables.  mode 1: n / (c c), 2: 1 / (n c c).  launch_slices_to_image
-// wants g 16-byte aligned.
+// sepw_fft.cu: transforms of N x N grids for the N of rows_supported: columns
+// in place on the grid side, before (to image) or after (to grid) the rows,
+// which have the image side's passes folded in.  tab: rows_table_bytes(N) bytes
+// filled by launch_rows_tables.  mode 1: n / (c c), 2: 1 / (n c c).  The column
+// transforms and launch_slices_to_image want g 16-byte aligned.
 bool rows_supported(int N);
 size_t rows_table_bytes(int N);
 cudaError_t launch_rows_tables(const DevParams &p, const double2 *tw, float2 *tab, cudaStream_t s);
+cudaError_t launch_columns(const DevParams &p, bool inverse, int grids, const float2 *tab,
+                           float2 *g, int num_sms, cudaStream_t s);
 cudaError_t launch_rows_to_image(const DevParams &p, int mode, const float *taper,
                                  const float2 *tab, float2 *buf, cudaStream_t s);
 cudaError_t launch_slices_to_image(const DevParams &p, int L, const float *taper, const float *wc,
