@@ -179,8 +179,8 @@ SEPW_API int sepw_locate(sepw_ctx *ctx, int64_t nvis, const double *u, const dou
                 sepw_stream_t stream);
 
 /* Locate and bin nvis visibilities into the context's plan (tiled forms:
- * counting sort by tile and by 4 x 4 sub-block of the footprint origin
- * inside the tile, cut into work items, each sorted by origin).  The
+ * counting sort by tile and by block of footprint origins inside the tile,
+ * cut into work items, each sorted by origin where the kernels need it).  The
  * plan is reused by sepw_grid_planned / sepw_degrid_planned until the next
  * sepw_plan; u, v, w need not stay alive.  Binning is amortisable over the
  * gridding/degridding calls of a major cycle (Sec. 6).  For the plain form
@@ -324,7 +324,9 @@ SEPW_API int sepw_test_stall_mma(sepw_ctx *ctx, int enable);
  *       I[b][a] = 1 / (n_ab c1(nu_a) c1(nu_b)) *
  *       sum_{cu,cv} grid[cv][cu] exp(2 pi i ((cu-N/2) nu_a + (cv-N/2) nu_b))
  *       = GRID_TO_IMAGE / n_ab^2.
- * Uses cuFFT (FP32 C2C); the plan is created on first use. */
+ * FP32.  The directions towards the image run the library's own transforms at
+ * N = 512, 1024, 2048 and 4096 (buf 16-byte aligned), everything else cuFFT C2C;
+ * twiddles and the cuFFT plan are made on first use. */
 SEPW_API int sepw_image(sepw_ctx *ctx, int direction, float *buf, sepw_stream_t stream);
 
 /* Taper of the grid correction: taper[a] = c1(nu_a), nu_a = (a - N/2)/N, the
@@ -426,7 +428,9 @@ SEPW_API int sepw_wstack_plan(sepw_ctx *ctx, int32_t nslices, const double *w_ce
  * complex64, device; transformed IN PLACE, their contents are destroyed):
  *   image[b][a] = sum_c exp(2 pi i w_c (n_ab - 1)) GRID_TO_IMAGE(grid_c)[b][a]
  * (GRID_TO_IMAGE as in sepw_image).  image (N x N complex64) is overwritten.
- * One batched cuFFT over the slices; FP32. */
+ * FP32.  The library's own transforms at N = 512, 1024, 2048 and 4096 with a
+ * 16-byte aligned image apart from the grids, else one batched cuFFT over the
+ * slices. */
 SEPW_API int sepw_wstack_image(sepw_ctx *ctx, float *slice_grids, float *image,
                                sepw_stream_t stream);
 

@@ -6,7 +6,7 @@ representative set of visibilities, every candidate (form, T) is timed on the
 GPU through the C ABI (plan + grid, CUDA events, median of a few runs) and the
 fastest one that meets the caller's accuracy class is kept; then, for that
 (form, T), the schedule of the plan (visibilities per work item, and for the
-FP32 block gridder the parts of an item a warp takes at a time) is tuned the
+FP32 tiled gridders the parts of an item a warp takes at a time) is tuned the
 same way.  Results are cached in a JSON file keyed by the GPU name and the
 geometry, so a pipeline tunes once and reuses the choice.
 
@@ -44,7 +44,7 @@ def candidate_tiles(support: int, form: str) -> list[int]:
 def candidate_schedules(form: str) -> list[tuple[int, int]]:
     """(chunk, grid_parts) candidates for a form: work items of 512 .. 2048
     visibilities; the FP32 tiled form also tries whole items (1) and eighths
-    (8) per warp unit besides the density rule (0).  The plain form has no
+    (8) per warp unit besides units by the plan's size (0).  The plain form has no
     plan schedule."""
     if form == "plain":
         return [(0, 0)]

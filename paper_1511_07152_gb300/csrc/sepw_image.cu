@@ -1,5 +1,6 @@
 // Image step with grid correction (Sec. 2: I_D / n = F^-1[grid] / c), around
-// an in-place cuFFT C2C transform of the N x N buffer.
+// an in-place cuFFT C2C transform of the N x N buffer.  The directions
+// towards the image run in sepw_fft.cu at the sizes it takes.
 //
 // With the u = 0 column at N/2, the shifted transform
 //   sum_c G[c] exp(2 pi i (c - N/2)(a - N/2) / N)

@@ -1,9 +1,10 @@
 // Tiled FP32 gridder and degridder (the separable update of Sec. 5, binned).
 //
 // Work items are <= kChunk visibilities of one T x T tile, sorted by
-// (footprint origin, conj) ("key"), taken from an atomic counter: by a whole
-// warp in the gridder, by a whole CTA in the degridder, which keeps the
-// tile's window of (T + S - 1)^2 cells in shared memory.  Per batch of
+// (footprint origin, conj) ("key").  A warp of a gridder takes units of 32 to
+// 256 of a tile's visibilities from an atomic counter; a CTA of a degridder takes
+// parts of an item and keeps the tile's window of (T + S - 1)^2 cells in shared
+// memory.  Per batch of
 // visibilities a warp first decodes the records once (one per lane: tap-row
 // offsets, W V or the output index and weight, key) into shared memory; the
 // inner loop reads them as broadcasts.
@@ -19,7 +20,8 @@
 //   * degridding, S = 4 .. 16, S % 4 = 0: two virtual warps of 16 lanes take
 //     two visibilities per step; lane (rg, cg) = (t >> 2, t & 3) owns rows
 //     rg + 4 r and columns cg + 4 c (2 S / 4 taps per lane per visibility);
-//   * other supports: lane (rg, j) owns footprint column j and S / RG rows.
+//   * other supports, where the window kernels (sepw_window.cu) are not taken:
+//     lane (rg, j) owns footprint column j and S / RG rows.
 // The interleaved cell assignment makes the lanes of one atomic or window
 // read cover a compact patch (few sectors per atomic, no bank conflicts).
 //

@@ -9,9 +9,10 @@
 // plan's slot -> visibility map is then composed with the sort, so gridding
 // and degridding read V, W and write predictions in the caller's order.
 //
-// Image step: one batched inverse FFT of all slice grids between a sign pass
-// and a combine pass that applies the grid correction n / (c c), the slice
-// phase and the sum over slices; the prediction direction mirrors it.
+// Image step here: one batched inverse FFT of all slice grids between a sign
+// pass and a combine pass that applies the grid correction n / (c c), the slice
+// phase and the sum over slices; the prediction direction mirrors it.  It serves
+// the sizes and buffers that the fused transforms (sepw_fft.cu) do not take.
 #include "sepw_internal.cuh"
 
 namespace sepw {

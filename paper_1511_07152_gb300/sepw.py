@@ -393,7 +393,7 @@ def sepw_set_wait_limit(ctx: Context, limit_ns: int):
 
 
 def sepw_set_schedule(ctx: Context, chunk: int = 0, grid_parts: int = 0):
-    """Work-item size and block-gridder parts of the next plans (0: defaults)."""
+    """Work-item size and FP32 gridder parts of the next plans (0: defaults)."""
     ctx.check(LIB.sepw_set_schedule(ctx.handle, int(chunk), int(grid_parts)))
     ctx.plan_nvis = 0
 
