@@ -295,17 +295,44 @@ struct alignas(16) Slot {
     int32_t vis;
     int32_t pad;
 };
+// Loads of what a kernel reads once, kept out of L1 so that the tap rows, which
+// are read again and again, stay there: window gridder at S = 12, 63M
+// visibilities, 6076 -> 5959 us; TF32 gridder, 32M, 3335 -> 3252 us; BF16 and
+// BF16 hi + lo gridders 0.1% and 0.2%, their degridders 0.5% by the slots alone.  The
+// hi + lo gridder (values loaded where they are used: 2504 -> 2578 us) and the
+// degridders' weights (neighbours share a sector: BF16 1597 -> 2026 us) keep
+// __ldg for theirs.
+__device__ __forceinline__ float2 ldg_once(const float2 *p)
+{
+    float2 x;
+    asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y)
+                 : "l"(p));
+    return x;
+}
+__device__ __forceinline__ float ldg_once(const float *p)
+{
+    float x;
+    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(x) : "l"(p));
+    return x;
+}
 __device__ __forceinline__ Slot load_slot(const Slot *p)
 {
-    const uint4 w = __ldg(reinterpret_cast<const uint4 *>(p));
+    uint4 w;
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w)
+                 : "l"(p));
     return {(uint64_t)w.y << 32 | w.x, (int32_t)w.z, 0};
 }
 // The same as two loads, for the tensor-core kernels, whose L1 data path is
 // their limit and does not carry the unused word so (8M visibilities in the
-// BF16 form: 1094 us with one load, 1070 with two).
+// BF16 form: 1094 us with one load, 1062 with two).
 __device__ __forceinline__ Slot load_slot_split(const Slot *p)
 {
-    return {__ldg(reinterpret_cast<const unsigned long long *>(&p->rec)), __ldg(&p->vis), 0};
+    unsigned long long rec;
+    int32_t vis;
+    asm volatile("ld.global.nc.L1::no_allocate.u64 %0, [%1];" : "=l"(rec) : "l"(&p->rec));
+    asm volatile("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(vis) : "l"(&p->vis));
+    return {rec, vis, 0};
 }
 __device__ __forceinline__ void store_slot(Slot *p, uint64_t rec, int32_t vis)
 {

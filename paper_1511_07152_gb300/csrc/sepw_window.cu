@@ -236,8 +236,8 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
                 const int i = slot.vis;
                 r = slot.rec;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
-                    const float wt = weight ? __ldg(weight + i) : 1.0f;
-                    const float2 x = __ldg(vis + i);
+                    const float wt = weight ? ldg_once(weight + i) : 1.0f;
+                    const float2 x = ldg_once(vis + i);
                     cj = rec_conj(r);
                     wv = make_float2(wt * x.x, wt * x.y);
                     slow = big || !(fabsf(wv.x) < 1e30f && fabsf(wv.y) < 1e30f);
