@@ -265,7 +265,7 @@ SEPW_API int sepw_set_wait_limit(sepw_ctx *ctx, uint64_t limit_ns);
  * Sec. 4.3): `chunk` visibilities per work item (64 .. 2048, a multiple of
  * 32; 0 = 2048, the default) and the number of parts the FP32 tiled
  * gridders cut an item into, one per warp at a time (1 .. 16; 0 = parts of 32
- * to 256 visibilities by the plan's size, the default).  Takes
+ * to 1024 visibilities by the plan's size, the default).  Takes
  * effect at the next sepw_plan (the current plan is invalidated); results
  * do not depend on it beyond FP32 rounding order.  Host only. */
 SEPW_API int sepw_set_schedule(sepw_ctx *ctx, int32_t chunk, int32_t grid_parts);

@@ -530,15 +530,19 @@ cudaError_t launch_zero_dropped(const Plan &plan, float2 *vis, cudaStream_t s)
                       plan.d_item_counter + 1, plan.dropped_out);
 }
 
-// The units of the tiled gridders: 32 to 256 visibilities, about two for each
+// The units of the tiled gridders: 32 to 256 (1024) visibilities, about two for each
 // of the ~40 warps an SM holds; for the block gridders also an eighth of their
 // tile, as long as that does not make more units than those warps can use
 // (sparse tiles then weigh as little as dense ones at the end of the launch,
 // and dense ones keep their runs).  Whole items of 2048 gave 524,288
 // visibilities to 400 warps (S = 16, 758 us; 155 us so).  Above 256 the last
 // warps work alone on 32M visibilities (2.13 ms for 256, 2.16 for 512, 2.24
-// for 1024, 2.38 for 2048); the window gridder adds whole windows at the ends
-// of a unit (128 grids at S = 12: 8.97 ms for 256, 9.55 for 128).
+// for 1024, 2.38 for 2048).  The window gridder adds whole windows at the ends
+// of a unit: up to 1024 below one visibility per cell (63M visibilities over
+// 128 grids of 2048^2 at S = 12: 5.96 ms for 256, 5.70 for 512, 5.58 for 1024
+// and 2048; 20M over 40: 1.95 -> 1.82 ms), where no tile holds a large part of
+// them; in dense data longer units only leave the end to few warps (32M on
+// 4096^2: 2.14 ms for 256, 2.18 for 1024).
 void set_units(const DevParams &p, int num_sms, Plan &plan)
 {
     plan.unit_parts = 1;
@@ -548,7 +552,8 @@ void set_units(const DevParams &p, int num_sms, Plan &plan)
     }
     const int64_t per = plan.window ? 320 : 80;
     const int64_t u = (plan.nvis / std::max<int64_t>(1, per * num_sms) + 31) & ~31ll;
-    plan.unit = (int32_t)std::min<int64_t>(256, std::max<int64_t>(32, u));
+    const bool sparse = plan.window && plan.nvis < (int64_t)plan.ntiles * p.T * p.T;
+    plan.unit = (int32_t)std::min<int64_t>(sparse ? 1024 : 256, std::max<int64_t>(32, u));
     if (!plan.window)
         plan.unit_parts = (int32_t)std::min<int64_t>(
             8, std::max<int64_t>(1, 640ll * num_sms / std::max(1, plan.ntiles)));

@@ -16,7 +16,7 @@
 // visibilities with one origin, and in sparse data nearly every visibility
 // has its own (63M visibilities over 128 grids of 2048^2 at S = 12: 144
 // atomics each, 0.83e12 a second, 10.97 ms, after a 2.5 ms sort by origin that
-// this kernel does not need; now 6.2 ms, 70% of the issue slots).  The window
+// this kernel does not need; now 5.57 ms, 70% of the issue slots).  The window
 // adds 4 (S + 3) cells per block of 16 origins and a whole window per column
 // of blocks instead.  The price is the zero taps: (S + 3)^2 cells rounded up
 // to the lanes' 4 RPL x 8 CPL, 256 for the 144 of S = 12.
@@ -28,7 +28,7 @@
 // row pairs (re, re, im, im): paired FP32 FMAs take them as loaded.
 // Pairs along columns (no register moves as the window steps down, a copy of
 // the loop for each place of its first row) and scalar FMAs were slower: 7.4
-// and 7.1 ms against 6.2 ms, as was a fifth CTA per SM (48 registers, 7.9 ms).
+// and 7.1 ms against 6.2 ms then, as was a fifth CTA per SM (48 registers, 7.9 ms).
 //
 // Zero taps must not meet non-finite values (Inf * 0 would spread to cells
 // outside the footprint): visibilities whose W V is not below 1e30, and all

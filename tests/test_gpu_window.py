@@ -78,7 +78,7 @@ def test_tile_sizes(env, tile):
 
 
 @pytest.mark.parametrize("nvis", [1, 31, 32, 33, 2047, 2048, 2049])
-@pytest.mark.parametrize("schedule", [None, (64, 1), (2048, 16)])
+@pytest.mark.parametrize("schedule", [None, (64, 1), (2048, 1), (2048, 16)])
 def test_unit_edges(env, nvis, schedule):
     """Units and items at their edges, all visibilities in one or two tiles."""
     _check(env, synth.random_case(341, nvis, 96, 12, 8, 5, radius_cells=3.0), schedule=schedule)
