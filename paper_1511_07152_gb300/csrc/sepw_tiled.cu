@@ -1,7 +1,7 @@
 // Tiled FP32 gridder and degridder (the separable update of Sec. 5, binned).
 //
 // Work items are <= kChunk visibilities of one T x T tile, sorted by
-// (footprint origin, conj) ("key").  A warp of a gridder takes units of 32 to
+// (footprint origin, conj) ("key").  A warp of a block gridder takes units of 32 to
 // 256 of a tile's visibilities from an atomic counter; a CTA of a degridder takes
 // parts of an item and keeps the tile's window of (T + S - 1)^2 cells in shared
 // memory.  Per batch of
