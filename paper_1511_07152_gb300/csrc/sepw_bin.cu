@@ -24,11 +24,11 @@ __device__ __forceinline__ unsigned lanemask_lt()
 // Pass 1: locate, record, bin histogram with each visibility's rank inside
 // its bin (the order of arrival at the bin's counter), dropped count.
 __global__ void __launch_bounds__(256) locate_bin_kernel(
-    DevParams p, int64_t nvis, const double *__restrict__ u, const double *__restrict__ v,
-    const double *__restrict__ w, int32_t *__restrict__ bin_of,
+    DevParams p, int64_t nvis, const double *u, const double *v,
+    const double *w, int32_t *__restrict__ bin_of,
     int32_t *__restrict__ rank_of, uint64_t *__restrict__ rec0, int32_t *bin_count,
     unsigned long long *dropped, int32_t *__restrict__ drop_list, int ngrids,
-    const int64_t *__restrict__ offsets)
+    const int64_t *offsets)
 {
     pdl_enter();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -204,7 +204,7 @@ __device__ __forceinline__ void count_tiles(int t0, int tb, int ntiles, int nsub
 
 __global__ void __launch_bounds__(kPlanThreads) tile_count_kernel(
     int32_t ntiles, int32_t tb, int32_t nsub, Cut cut,
-    const int32_t *__restrict__ bin, int32_t *__restrict__ tile_count,
+    const int32_t *bin, int32_t *__restrict__ tile_count,
     Totals *__restrict__ blocks, unsigned *ticket)
 {
     __shared__ Totals s_warps[33];
@@ -271,7 +271,7 @@ __device__ __forceinline__ void list_full(WorkItem *__restrict__ out, int tile0,
 template <bool ONE>
 __global__ void __launch_bounds__(kPlanThreads) tile_items_kernel(
     int32_t ntiles, int32_t tb, int32_t nsub, Cut cut,
-    const int32_t *__restrict__ tile_count, const Totals *__restrict__ blocks,
+    const int32_t *tile_count, const Totals *blocks,
     int32_t *__restrict__ bin, WorkItem *__restrict__ items, int32_t *nitems,
     WorkItem *__restrict__ units, int32_t *nunits)
 {
@@ -362,8 +362,8 @@ static_assert(kMaxSubBins == 64, "two bins per lane");
 // 4-byte array the pass was bound by twice the partial sectors it sends to L2
 // (32M visibilities 424 us; 331 us so).
 __global__ void __launch_bounds__(256) scatter_kernel(
-    int64_t nvis, const int32_t *__restrict__ bin_of, const int32_t *__restrict__ rank_of,
-    const uint64_t *__restrict__ rec0, const int32_t *__restrict__ bin_first,
+    int64_t nvis, const int32_t *bin_of, const int32_t *rank_of,
+    const uint64_t *rec0, const int32_t *bin_first,
     Slot *__restrict__ slots)
 {
     pdl_enter();
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(
     const int b = bin_of[i];
     if (b < 0)
         return;
-    const int slot = __ldg(bin_first + b) + rank_of[i];
+    const int slot = bin_first[b] + rank_of[i];
     store_slot(slots + slot, rec0[i], (int32_t)i);
 }
 
@@ -402,7 +402,7 @@ static int sort_keys(const DevParams &p)
 }
 
 __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
-    DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
+    DevParams p, const WorkItem *items, const int32_t *nitems,
     Slot *__restrict__ slots)
 {
     extern __shared__ int32_t hist[];  // per * kSortThreads bins
@@ -508,8 +508,8 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
 
 // Degridding writes 0 for every dropped visibility of the plan.  Also clears
 // the degridder's work counter.
-__global__ void zero_dropped_kernel(const int32_t *__restrict__ drop_list,
-                                    const unsigned long long *__restrict__ ndrop,
+__global__ void zero_dropped_kernel(const int32_t *drop_list,
+                                    const unsigned long long *ndrop,
                                     float2 *__restrict__ vis, int32_t *counter, int64_t *dropped)
 {
     pdl_enter();

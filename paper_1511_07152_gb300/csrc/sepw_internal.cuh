@@ -64,6 +64,13 @@ struct DevParams {
 // waits, so a kernel completes after all kernels before it; a launch without
 // the attribute makes both calls no-ops.  pdl_trigger lets the next kernel's
 // blocks take free places from here on.
+//
+// Such a kernel can be resident while the ones before it still write, and the
+// non-coherent load path (ld.global.nc: __ldg, const __restrict__ arguments)
+// is only defined for data that nobody writes during the reading kernel's
+// life.  So the kernels launched by launch_pdl read memory with ordinary loads
+// alone, also what only the caller writes (the kernel before the first of a
+// chain may be the caller's and may trigger early, too).
 __device__ __forceinline__ void pdl_wait()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -302,23 +309,23 @@ struct alignas(16) Slot {
 // hi + lo gridder (values loaded where they are used: 2504 -> 2578 us) and the
 // degridders' weights (neighbours share a sector: BF16 1597 -> 2026 us) keep
 // __ldg for theirs.
-__device__ __forceinline__ float2 ldg_once(const float2 *p)
+__device__ __forceinline__ float2 load_once(const float2 *p)
 {
     float2 x;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y)
+    asm volatile("ld.global.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(x.x), "=f"(x.y)
                  : "l"(p));
     return x;
 }
-__device__ __forceinline__ float ldg_once(const float *p)
+__device__ __forceinline__ float load_once(const float *p)
 {
     float x;
-    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(x) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.f32 %0, [%1];" : "=f"(x) : "l"(p));
     return x;
 }
 __device__ __forceinline__ Slot load_slot(const Slot *p)
 {
     uint4 w;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w)
                  : "l"(p));
     return {(uint64_t)w.y << 32 | w.x, (int32_t)w.z, 0};
@@ -330,8 +337,8 @@ __device__ __forceinline__ Slot load_slot_split(const Slot *p)
 {
     unsigned long long rec;
     int32_t vis;
-    asm volatile("ld.global.nc.L1::no_allocate.u64 %0, [%1];" : "=l"(rec) : "l"(&p->rec));
-    asm volatile("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(vis) : "l"(&p->vis));
+    asm volatile("ld.global.L1::no_allocate.u64 %0, [%1];" : "=l"(rec) : "l"(&p->rec));
+    asm volatile("ld.global.L1::no_allocate.s32 %0, [%1];" : "=r"(vis) : "l"(&p->vis));
     return {rec, vis, 0};
 }
 __device__ __forceinline__ void store_slot(Slot *p, uint64_t rec, int32_t vis)

@@ -471,8 +471,8 @@ __global__ void __launch_bounds__(Cfg<PREC>::kBlock, 1) grid_tc2_kernel(
                 x_[sl] = make_float2(0.f, 0.f);
                 w_[sl] = 0.f;
                 if (C::PRE && vi_[sl] >= 0) {
-                    x_[sl] = ldg_once(vis + vi_[sl]);
-                    w_[sl] = weight ? ldg_once(weight + vi_[sl]) : 1.0f;
+                    x_[sl] = load_once(vis + vi_[sl]);
+                    w_[sl] = weight ? load_once(weight + vi_[sl]) : 1.0f;
                 }
             }
         };

@@ -92,7 +92,7 @@ __device__ __forceinline__ int key_lx(int key) { return (key >> 1) & 63; }
 
 // Loads the RPL v-taps of this lane's rows (rows >= S give zero).
 template <int S>
-__device__ __forceinline__ void load_vtaps(const float2 *__restrict__ row, int rg,
+__device__ __forceinline__ void load_vtaps(const float2 *row, int rg,
                                            float (&tr)[Layout<S>::RPL],
                                            float (&ti)[Layout<S>::RPL])
 {
@@ -104,7 +104,7 @@ __device__ __forceinline__ void load_vtaps(const float2 *__restrict__ row, int r
         for (int q = 0; q < RPL / 2; ++q) {
             float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
             if (Layout<S>::FULL_ROWS || k0 + 2 * q < S)
-                t = __ldg(r4 + q);
+                t = r4[q];
             tr[2 * q] = t.x;
             ti[2 * q] = t.y;
             tr[2 * q + 1] = t.z;
@@ -115,7 +115,7 @@ __device__ __forceinline__ void load_vtaps(const float2 *__restrict__ row, int r
         for (int q = 0; q < RPL; ++q) {
             float2 t = make_float2(0.f, 0.f);
             if (Layout<S>::FULL_ROWS || k0 + q < S)
-                t = __ldg(row + k0 + q);
+                t = row[k0 + q];
             tr[q] = t.x;
             ti[q] = t.y;
         }
@@ -124,10 +124,10 @@ __device__ __forceinline__ void load_vtaps(const float2 *__restrict__ row, int r
 
 template <int S>
 __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) grid_tiled_kernel(
-    DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
-    int32_t *counter, const Slot *__restrict__ slots,
-    const float2 *__restrict__ vis, const float *__restrict__ weight,
-    const float2 *__restrict__ taps, float2 *grid)
+    DevParams p, const WorkItem *items, const int32_t *nitems,
+    int32_t *counter, const Slot *slots,
+    const float2 *vis, const float *weight,
+    const float2 *taps, float2 *grid)
 {
     pdl_enter(p);
     constexpr int RG = Layout<S>::RG, RPL = Layout<S>::RPL;
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) grid_tiled_k
                 const Slot slot = load_slot(slots + s);
                 const uint64_t r = slot.rec;
                 const int i = slot.vis;
-                const float wt = weight ? __ldg(weight + i) : 1.0f;
-                const float2 x = __ldg(vis + i);
+                const float wt = weight ? weight[i] : 1.0f;
+                const float2 x = vis[i];
                 const bool cj = rec_conj(r);
                 const int row = rec_plane(r) * p.OS;
                 const int key = ((rec_ly(r) * 64 + rec_lx(r)) << 1) | (cj ? 1 : 0);
@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) grid_tiled_k
                 if (lane_ok) {
                     const float wx = __int_as_float(m.z), wy = __int_as_float(m.w);
                     const float2 *tu = taps + m.x;
-                    const float2 a = __ldg(tu + j);
+                    const float2 a = tu[j];
                     const float pr = wx * a.x - wy * a.y;
                     const float pi = wx * a.y + wy * a.x;
                     float tr[RPL], ti[RPL];
@@ -249,9 +249,9 @@ __device__ __forceinline__ void reduce8(float (&v)[8], int lane)
 
 template <int S>
 __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled_kernel(
-    DevParams p, int WP, const WorkItem *__restrict__ items,
-    const int32_t *__restrict__ nitems, int32_t *counter, const Slot *__restrict__ slots, const float2 *__restrict__ grid,
-    const float *__restrict__ weight, const float2 *__restrict__ taps,
+    DevParams p, int WP, const WorkItem *items,
+    const int32_t *nitems, int32_t *counter, const Slot *slots, const float2 *grid,
+    const float *weight, const float2 *taps,
     float2 *__restrict__ vis_out)
 {
     pdl_enter(p);
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled
             for (int cc = lane; cc < W; cc += 32) {
                 float2 g = make_float2(0.f, 0.f);
                 if (gy < p.N && o.gx0 + cc < p.N)
-                    g = __ldg(grow + cc);
+                    g = grow[cc];
                 wre[rr * WP + cc] = g.x;
                 wim[rr * WP + cc] = g.y;
             }
@@ -312,7 +312,7 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled
                 const int key = ((rec_ly(r) * 64 + rec_lx(r)) << 1) | (rec_conj(r) ? 1 : 0);
                 meta[lane] = make_int4((row + rec_ou(r)) * S,
                                        key | ((rec_ov(r) - rec_ou(r)) * S) * 8192, i,
-                                       __float_as_int(weight ? __ldg(weight + i) : 1.0f));
+                                       __float_as_int(weight ? weight[i] : 1.0f));
             }
             __syncwarp();
             const int n = min(32, b1 - base);
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kTiledThreads, kTiledBlocksPerSM) degrid_tiled
                                 si = fmaf(tr[k], xi[k], si);
                                 si = fmaf(ti[k], xr[k], si);
                             }
-                            const float2 a = __ldg(tu + j);
+                            const float2 a = tu[j];
                             vr[e] = sr * a.x - si * a.y;
                             vi[e] = sr * a.y + si * a.x;
                         }
@@ -398,12 +398,12 @@ struct Blk {
 
 // Loads the B taps k0, k0 + 4, ... of one table row.
 template <int B>
-__device__ __forceinline__ void load_taps4(const float2 *__restrict__ row, int k0,
+__device__ __forceinline__ void load_taps4(const float2 *row, int k0,
                                            float (&re)[B], float (&im)[B])
 {
 #pragma unroll
     for (int c = 0; c < B; ++c) {
-        const float2 t = __ldg(row + k0 + 4 * c);
+        const float2 t = row[k0 + 4 * c];
         re[c] = t.x;
         im[c] = t.y;
     }
@@ -438,9 +438,9 @@ __device__ __forceinline__ void reduce16x8(float (&v)[8], int t)
 
 template <int S>
 __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block_kernel(
-    DevParams p, int WP, const WorkItem *__restrict__ items,
-    const int32_t *__restrict__ nitems, int32_t *counter, const Slot *__restrict__ slots, const float2 *__restrict__ grid,
-    const float *__restrict__ weight, const float2 *__restrict__ taps,
+    DevParams p, int WP, const WorkItem *items,
+    const int32_t *nitems, int32_t *counter, const Slot *slots, const float2 *grid,
+    const float *weight, const float2 *taps,
     float2 *__restrict__ vis_out)
 {
     pdl_enter(p);
@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block
             for (int cc = lane; cc < W; cc += 32) {
                 float2 g = make_float2(0.f, 0.f);
                 if (gy < p.N && o.gx0 + cc < p.N)
-                    g = __ldg(grow + cc);
+                    g = grow[cc];
                 win[rr * WP + cc] = g;
             }
         }
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(kTiledThreads, Blk<S>::BPS) degrid_tiled_block
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
                     const int row = rec_plane(r) * p.OS;
                     meta[t] = make_int4((row + rec_ou(r)) * S, (row + rec_ov(r)) * S, i,
-                                        __float_as_int(weight ? __ldg(weight + i) : 1.0f));
+                                        __float_as_int(weight ? weight[i] : 1.0f));
                     keys[t] = ((rec_ly(r) * 64 + rec_lx(r)) << 1) | (rec_conj(r) ? 1 : 0);
                 } else {
                     // checked build: taps of row 0 at window origin 0, no output
@@ -627,10 +627,10 @@ constexpr int kGridBlkPerSM = 5;
 
 template <int S, bool PLANAR>
 __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block_kernel(
-    DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
-    int32_t *counter, const Slot *__restrict__ slots,
-    const float2 *__restrict__ vis, const float *__restrict__ weight,
-    const float2 *__restrict__ taps, const float *__restrict__ planar, float2 *grid)
+    DevParams p, const WorkItem *units, const int32_t *nunits,
+    int32_t *counter, const Slot *slots,
+    const float2 *vis, const float *weight,
+    const float2 *taps, const float *planar, float2 *grid)
 {
     pdl_enter(p);
     constexpr int RB = Blk2<S>::RB, RP = Blk2<S>::RP, CB = Blk2<S>::CB;
@@ -709,8 +709,8 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
                 const uint64_t r = slot.rec;
                 const int i = slot.vis;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
-                    const float wt = weight ? __ldg(weight + i) : 1.0f;
-                    const float2 x = __ldg(vis + i);
+                    const float wt = weight ? weight[i] : 1.0f;
+                    const float2 x = vis[i];
                     const bool cj = rec_conj(r);
                     const int row = rec_plane(r) * p.OS;
                     kq = ((rec_ly(r) * 64 + rec_lx(r)) << 1) | (cj ? 1 : 0);
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
                     for (int c = 0; c < CB; ++c) {
                         float2 a = make_float2(0.f, 0.f);
                         if (FULL || cg + 8 * c < S)
-                            a = __ldg(tu + 8 * c);
+                            a = tu[8 * c];
                         // partial product W V F1(u), Sec. 5
                         pr[c] = wx * a.x - wy * a.y;
                         pi[c] = wx * a.y + wy * a.x;
@@ -756,8 +756,8 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
                     if constexpr (PLANAR) {
                         const float *pv = prow + 2 * m.y;
                         if constexpr (RP == 2) {
-                            const float4 re = __ldg(reinterpret_cast<const float4 *>(pv));
-                            const float4 im = __ldg(reinterpret_cast<const float4 *>(pv + S));
+                            const float4 re = *reinterpret_cast<const float4 *>(pv);
+                            const float4 im = *reinterpret_cast<const float4 *>(pv + S);
                             vr[0] = make_float2(re.x, re.y);
                             vr[1] = make_float2(re.z, re.w);
                             vi[0] = make_float2(im.x, im.y);
@@ -765,15 +765,15 @@ __global__ void __launch_bounds__(kTiledThreads, kGridBlkPerSM) grid_tiled_block
                         } else {
 #pragma unroll
                             for (int q2 = 0; q2 < RP; ++q2) {
-                                vr[q2] = __ldg(reinterpret_cast<const float2 *>(pv) + q2);
-                                vi[q2] = __ldg(reinterpret_cast<const float2 *>(pv + S) + q2);
+                                vr[q2] = reinterpret_cast<const float2 *>(pv)[q2];
+                                vi[q2] = reinterpret_cast<const float2 *>(pv + S)[q2];
                             }
                         }
                     } else {
                         const float2 *tv = trow + m.y;
 #pragma unroll
                         for (int q2 = 0; q2 < RP; ++q2) {
-                            const float2 t0 = __ldg(tv + 8 * q2), t1 = __ldg(tv + 8 * q2 + 4);
+                            const float2 t0 = tv[8 * q2], t1 = tv[8 * q2 + 4];
                             vr[q2] = make_float2(t0.x, t1.x);
                             vi[q2] = make_float2(t0.y, t1.y);
                         }
@@ -834,7 +834,7 @@ static size_t tiled_smem(int W, int WP)
 // S.  A lane of the block gridder owns rows g, g + 4, g + 8, ... (g = k mod 4),
 // whose taps are then adjacent: one vector load gives its FP32 pairs.
 // Also clears the gridder's work counter.
-__global__ void planar_taps_kernel(const float2 *__restrict__ taps, float *__restrict__ out,
+__global__ void planar_taps_kernel(const float2 *taps, float *__restrict__ out,
                                    int64_t n, int S, int32_t *counter,
                                    const unsigned long long *ndrop, int64_t *dropped)
 {

@@ -69,7 +69,7 @@ constexpr size_t win_row_floats()
 // clears the work counter.
 template <int S>
 __global__ void __launch_bounds__(256) window_tables_kernel(
-    const float2 *__restrict__ utaps, const float2 *__restrict__ vtaps, int64_t rows,
+    const float2 *utaps, const float2 *vtaps, int64_t rows,
     float *__restrict__ utab, float *__restrict__ vtab, int32_t *__restrict__ flags,
     int32_t *counter, const unsigned long long *ndrop, int64_t *dropped)
 {
@@ -109,13 +109,13 @@ __global__ void __launch_bounds__(256) window_tables_kernel(
 
 // Adds one visibility's exact S x S footprint (origin cell g) by atomics.
 template <int S>
-__device__ __noinline__ void add_footprint(const float2 *__restrict__ tu,
-                                           const float2 *__restrict__ tv, float2 wv, float sg,
+__device__ __noinline__ void add_footprint(const float2 *tu,
+                                           const float2 *tv, float2 wv, float sg,
                                            float2 *g, int N, int lane)
 {
     for (int c = lane; c < S * S; c += 32) {
         const int k = c / S, j = c % S;
-        const float2 a = __ldg(tu + j), b = __ldg(tv + k);
+        const float2 a = tu[j], b = tv[k];
         const float ay = sg * a.y, by = sg * b.y;
         const float pr = wv.x * a.x - wv.y * ay, pi = wv.x * ay + wv.y * a.x;
         atomicAdd(g + (int64_t)k * N + j, make_float2(pr * b.x - pi * by, pr * by + pi * b.x));
@@ -126,7 +126,7 @@ __device__ __forceinline__ float2 dup(float x) { return make_float2(x, x); }
 
 // A lane's v-taps at an alignment: row pairs and the single last row.
 template <int S>
-__device__ __forceinline__ void window_vtaps(const float *__restrict__ tv,
+__device__ __forceinline__ void window_vtaps(const float *tv,
                                              float2 (&vr)[Win<S>::RP], float2 (&vi)[Win<S>::RP],
                                              float2 &ve)
 {
@@ -134,25 +134,25 @@ __device__ __forceinline__ void window_vtaps(const float *__restrict__ tv,
 #pragma unroll
     for (int k = 0; k < W::RP; ++k) {
         if constexpr (W::VG % 4 == 0) {
-            const float4 t = __ldg(reinterpret_cast<const float4 *>(tv) + k);
+            const float4 t = reinterpret_cast<const float4 *>(tv)[k];
             vr[k] = make_float2(t.x, t.y);
             vi[k] = make_float2(t.z, t.w);
         } else {
-            vr[k] = __ldg(reinterpret_cast<const float2 *>(tv) + 2 * k);
-            vi[k] = __ldg(reinterpret_cast<const float2 *>(tv) + 2 * k + 1);
+            vr[k] = reinterpret_cast<const float2 *>(tv)[2 * k];
+            vi[k] = reinterpret_cast<const float2 *>(tv)[2 * k + 1];
         }
     }
     if constexpr (W::ODD)
-        ve = __ldg(reinterpret_cast<const float2 *>(tv) + 2 * W::RP);
+        ve = reinterpret_cast<const float2 *>(tv)[2 * W::RP];
 }
 
 template <int S>
 __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
-    DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
-    int32_t *counter, const Slot *__restrict__ slots,
-    const float2 *__restrict__ vis, const float *__restrict__ weight,
-    const float2 *__restrict__ taps, const float *__restrict__ utab,
-    const float *__restrict__ vtab, const int32_t *__restrict__ flags, float2 *grid)
+    DevParams p, const WorkItem *units, const int32_t *nunits,
+    int32_t *counter, const Slot *slots,
+    const float2 *vis, const float *weight,
+    const float2 *taps, const float *utab,
+    const float *vtab, const int32_t *flags, float2 *grid)
 {
     pdl_enter(p);
     using W = Win<S>;
@@ -236,8 +236,8 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
                 const int i = slot.vis;
                 r = slot.rec;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
-                    const float wt = weight ? ldg_once(weight + i) : 1.0f;
-                    const float2 x = ldg_once(vis + i);
+                    const float wt = weight ? load_once(weight + i) : 1.0f;
+                    const float2 x = load_once(vis + i);
                     cj = rec_conj(r);
                     wv = make_float2(wt * x.x, wt * x.y);
                     slow = big || !(fabsf(wv.x) < 1e30f && fabsf(wv.y) < 1e30f);
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
                     window_vtaps<S>(vlane + m.y, vr, vi, ve);
 #pragma unroll
                     for (int c = 0; c < CPL; ++c) {
-                        const float2 t = __ldg(reinterpret_cast<const float2 *>(tu + 16 * c));
+                        const float2 t = *reinterpret_cast<const float2 *>(tu + 16 * c);
                         // W V F1(u), Sec. 5
                         const float pr = wx * t.x - wy * t.y, pi = wx * t.y + wy * t.x;
                         const float spr = sg * pr, spi = sg * pi;
@@ -341,14 +341,14 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
 // degrid_footprint.
 // ---------------------------------------------------------------------------
 template <int S>
-__device__ __noinline__ float2 degrid_footprint(const float2 *__restrict__ tu,
-                                                const float2 *__restrict__ tv, float sg,
-                                                const float2 *__restrict__ g, int N, int lane)
+__device__ __noinline__ float2 degrid_footprint(const float2 *tu,
+                                                const float2 *tv, float sg,
+                                                const float2 *g, int N, int lane)
 {
     float2 acc = make_float2(0.f, 0.f);
     for (int c = lane; c < S * S; c += 32) {
         const int k = c / S, j = c % S;
-        const float2 a = __ldg(tu + j), b = __ldg(tv + k), x = __ldg(g + (int64_t)k * N + j);
+        const float2 a = tu[j], b = tv[k], x = g[(int64_t)k * N + j];
         const float ay = sg * a.y, by = sg * b.y;  // conjugated taps
         const float kr = a.x * b.x - ay * by, ki = a.x * by + ay * b.x;
         acc.x += kr * x.x - ki * x.y;
@@ -359,11 +359,11 @@ __device__ __noinline__ float2 degrid_footprint(const float2 *__restrict__ tu,
 
 template <int S>
 __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) degrid_window_kernel(
-    DevParams p, const WorkItem *__restrict__ units, const int32_t *__restrict__ nunits,
-    int32_t *counter, const Slot *__restrict__ slots,
-    const float2 *__restrict__ grid, const float *__restrict__ weight,
-    const float2 *__restrict__ taps, const float *__restrict__ utab,
-    const float *__restrict__ vtab, const int32_t *__restrict__ flags, float2 *__restrict__ vis_out)
+    DevParams p, const WorkItem *units, const int32_t *nunits,
+    int32_t *counter, const Slot *slots,
+    const float2 *grid, const float *weight,
+    const float2 *taps, const float *utab,
+    const float *vtab, const int32_t *flags, float2 *__restrict__ vis_out)
 {
     pdl_enter(p);
     using W = Win<S>;
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) degrid_window_kernel
                 v[c] = dup(0.f);
                 if ((c < CPL - 1 || last_col) && o.gy0 + y + rg < p.N &&
                     o.gx0 + x + cg + 8 * c < p.N)
-                    v[c] = __ldg(g0 + (int64_t)y * p.N + x + 8 * c);
+                    v[c] = g0[(int64_t)y * p.N + x + 8 * c];
                 off |= !(fabsf(v[c].x) < 1e30f && fabsf(v[c].y) < 1e30f);
             }
             bad |= __any_sync(0xffffffffu, off);
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) degrid_window_kernel
                 r = slot.rec;
                 i = slot.vis;
                 if (record_ok(p, r, i, o.gy0, o.gx0)) {
-                    wt = weight ? __ldg(weight + i) : 1.0f;
+                    wt = weight ? weight[i] : 1.0f;
                     cj = rec_conj(r);
                 } else {
                     r = 0;  // checked build: no output
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) degrid_window_kernel
                             ti = fmaf(ve.x, xe[c].y, ti);
                             ti = fmaf(-ve.y, xe[c].x, ti);
                         }
-                        const float2 t = __ldg(reinterpret_cast<const float2 *>(tu + 16 * c));
+                        const float2 t = *reinterpret_cast<const float2 *>(tu + 16 * c);
                         const float uy = sg * t.y;
                         sr = fmaf(tr, t.x, sr);
                         sr = fmaf(ti, uy, sr);
