@@ -312,6 +312,11 @@ SEPW_API int sepw_test_corrupt_plan(sepw_ctx *ctx, int which, int64_t slot, int3
  * restores normal operation.  Host only. */
 SEPW_API int sepw_test_stall_mma(sepw_ctx *ctx, int enable);
 
+/* Test hook for the out-of-memory path (no counterpart in the paper): the k-th
+ * workspace allocation of this context from now on (k >= 1; 0: none) fails,
+ * and the call that makes it returns SEPW_ENOMEM.  Host only. */
+SEPW_API int sepw_test_fail_alloc(sepw_ctx *ctx, int32_t k);
+
 /* Image step with grid correction, Sec. 2 (I_D / n = F^-1[grid] / c), in
  * place on an N x N complex64 buffer:
  *   SEPW_GRID_TO_IMAGE:  I[b][a] = n_ab / (c1(nu_a) c1(nu_b)) *

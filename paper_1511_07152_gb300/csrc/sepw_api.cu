@@ -65,6 +65,7 @@ struct sepw_ctx {
     int64_t ws_cap = 0;
     cufftHandle fft_batch = 0;
     int fft_batch_n = 0;  // slices of fft_batch, 0 = none
+    int32_t fail_alloc = 0;  // sepw_test_fail_alloc
     char err[512] = {0};
 };
 
@@ -159,6 +160,9 @@ namespace {
 
 DevParams make_dev(const sepw_params *p) { return sepw::make_dev_params(p); }
 
+// Replaces *ptr by a new allocation.  The old one is gone also when this fails:
+// the caller sets the capacity that stands for *ptr to 0 before the call and to
+// its new value once all allocations it stands for are there.
 template <typename T>
 int grow(sepw_ctx *ctx, T **ptr, size_t count)
 {
@@ -167,7 +171,9 @@ int grow(sepw_ctx *ctx, T **ptr, size_t count)
     *ptr = nullptr;
     if (count == 0)
         count = 1;
-    cudaError_t e = cudaMalloc((void **)ptr, count * sizeof(T));
+    cudaError_t e = ctx->fail_alloc > 0 && --ctx->fail_alloc == 0
+                        ? cudaErrorMemoryAllocation
+                        : cudaMalloc((void **)ptr, count * sizeof(T));
     if (e != cudaSuccess) {
         *ptr = nullptr;
         cudaGetLastError();
@@ -232,11 +238,11 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
         set_bins(ctx->dp, kBinsSorted);
     if (ntiles64 * ctx->dp.nsub > INT32_MAX)
         return fail(ctx, SEPW_EINVAL, "too many bins (%lld tiles)", (long long)ntiles64);
-    if (!pl.d_nitems) {
-        if ((rc = grow(ctx, &pl.d_nitems, 2)) || (rc = grow(ctx, &pl.d_item_counter, 2)))
-            return rc;
-        pl.d_nunits = pl.d_nitems + 1;
-    }
+    if (!pl.d_nitems && (rc = grow(ctx, &pl.d_nitems, 2)))
+        return rc;
+    if (!pl.d_item_counter && (rc = grow(ctx, &pl.d_item_counter, 2)))
+        return rc;
+    pl.d_nunits = pl.d_nitems + 1;
     if (pl.tiles_capacity < ntiles) {
         pl.tiles_capacity = 0;
         unsigned char *blocks = (unsigned char *)pl.d_blocks;
@@ -261,6 +267,7 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
         return SEPW_OK;  // the plain form keeps no per-visibility state
     if (pl.capacity < nvis) {
         int64_t cap = nvis;
+        pl.capacity = 0;
         if ((rc = grow(ctx, &pl.d_tile, cap)) || (rc = grow(ctx, &pl.d_rank, cap)) ||
             (rc = grow(ctx, &pl.d_rec0, cap)) ||
             (rc = grow(ctx, &pl.d_slots, cap)) ||
@@ -272,6 +279,7 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     if (items > INT32_MAX)
         return fail(ctx, SEPW_EINVAL, "too many work items");
     if (pl.items_capacity < items) {
+        pl.items_capacity = 0;
         if ((rc = grow(ctx, &pl.d_items, (size_t)items)))
             return rc;
         pl.items_capacity = (int32_t)items;
@@ -532,6 +540,7 @@ static int plan_impl(sepw_ctx *ctx, int32_t ngrids, const int64_t *offsets_host,
     pl.h_offsets.assign(offsets_host, offsets_host + ngrids + 1);
     if (ngrids > 1) {
         if (pl.offsets_capacity < ngrids + 1) {
+            pl.offsets_capacity = 0;
             if ((rc = grow(ctx, &pl.d_offsets, (size_t)ngrids + 1)))
                 return rc;
             pl.offsets_capacity = ngrids + 1;
@@ -825,6 +834,14 @@ int sepw_test_stall_mma(sepw_ctx *ctx, int enable)
     if (!ctx)
         return SEPW_EINVAL;
     ctx->tc_ctl.stall = enable ? 1 : 0;
+    return SEPW_OK;
+}
+
+int sepw_test_fail_alloc(sepw_ctx *ctx, int32_t k)
+{
+    if (!ctx)
+        return SEPW_EINVAL;
+    ctx->fail_alloc = k;
     return SEPW_OK;
 }
 
@@ -1136,6 +1153,7 @@ int sepw_wstack_plan(sepw_ctx *ctx, int32_t nslices, const double *w_centres, in
         return rc;
     cudaStream_t s = (cudaStream_t)stream;
     if (nslices > ctx->ws_centres_cap) {
+        ctx->ws_centres_cap = 0;
         if ((rc = grow(ctx, &ctx->d_ws_c64, (size_t)nslices)) ||
             (rc = grow(ctx, &ctx->d_ws_c32, (size_t)nslices)) ||
             (rc = grow(ctx, &ctx->d_ws_count, (size_t)nslices)))
@@ -1144,6 +1162,7 @@ int sepw_wstack_plan(sepw_ctx *ctx, int32_t nslices, const double *w_centres, in
     }
     if (nvis > ctx->ws_cap) {
         const size_t cap = (size_t)nvis + nvis / 8;
+        ctx->ws_cap = 0;
         if ((rc = grow(ctx, &ctx->d_ws_slice, cap)) || (rc = grow(ctx, &ctx->d_ws_part, cap)) ||
             (rc = grow(ctx, &ctx->d_ws_u, cap)) || (rc = grow(ctx, &ctx->d_ws_v, cap)) ||
             (rc = grow(ctx, &ctx->d_ws_w, cap)))

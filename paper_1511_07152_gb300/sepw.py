@@ -85,6 +85,7 @@ _SIG = {
     "sepw_device_status": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int), _P]),
     "sepw_set_wait_limit": (ctypes.c_int, [_P, ctypes.c_uint64]),
     "sepw_test_stall_mma": (ctypes.c_int, [_P, ctypes.c_int]),
+    "sepw_test_fail_alloc": (ctypes.c_int, [_P, ctypes.c_int32]),
     "sepw_fma_probe": (ctypes.c_int, [ctypes.c_int, _I64, _P, _I64, ctypes.POINTER(_I64), _P]),
     "sepw_checked_build": (ctypes.c_int, []),
     "sepw_test_corrupt_plan": (ctypes.c_int, [_P, ctypes.c_int, _I64, ctypes.c_int32]),
@@ -421,6 +422,11 @@ def sepw_fma_probe(paired: bool, iters: int, out, stream=None) -> int:
 def sepw_checked_build() -> bool:
     """True when the loaded library is the bounds-checked build."""
     return LIB.sepw_checked_build() != 0
+
+
+def sepw_test_fail_alloc(ctx: Context, k: int):
+    """Test hook: the k-th workspace allocation from now on fails (0: none)."""
+    ctx.check(LIB.sepw_test_fail_alloc(ctx.handle, int(k)))
 
 
 def sepw_test_corrupt_plan(ctx: Context, which: int, slot: int, value: int):
