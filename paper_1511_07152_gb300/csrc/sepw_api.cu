@@ -230,14 +230,12 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     if (ntiles64 > (1ll << 26))
         return fail(ctx, SEPW_EINVAL, "too many tiles (%lld)", (long long)ntiles64);
     const int ntiles = (int)ntiles64;
-    // the window gridder's bins unless their ids (tile * nsub + bin) leave int32
+    // at most 2^26 tiles of 32 bins: the ids fit int32; with more bins a tile
+    // (the window gridder's, fine ones) the tiles have to be fewer
     const bool sorts = ctx->p.form == SEPW_FORM_TILED || ctx->p.form == SEPW_FORM_TC_TF32;
-    const bool window = ctx->window && plan_window(ctx->dp, nvis, ngrids);
-    set_bins(ctx->dp, window ? kBinsWindow : sorts ? kBinsSorted : kBinsTile);
-    if (ntiles64 * ctx->dp.nsub > INT32_MAX)
-        set_bins(ctx->dp, kBinsSorted);
-    if (ntiles64 * ctx->dp.nsub > INT32_MAX)
-        return fail(ctx, SEPW_EINVAL, "too many bins (%lld tiles)", (long long)ntiles64);
+    pl.window = ctx->window && plan_window(ctx->dp, nvis, ngrids) &&
+                ntiles64 * kMaxSubBins <= (1ll << 31);
+    set_bins(ctx->dp, pl.window ? kBinsWindow : plan_bins(ctx->dp, ctx->p.form, nvis, ntiles64));
     if (!pl.d_nitems && (rc = grow(ctx, &pl.d_nitems, 2)))
         return rc;
     if (!pl.d_item_counter && (rc = grow(ctx, &pl.d_item_counter, 2)))
@@ -286,7 +284,6 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     }
     pl.nvis = nvis;
     ctx->dp.early = nvis <= kEarlyVis ? 1 : 0;
-    pl.window = ctx->dp.sub_log2 == 2;  // kBinsWindow
     set_units(ctx->dp, ctx->num_sms, pl);
     if (ctx->p.form == SEPW_FORM_TILED) {
         const int64_t units = max_units(pl);

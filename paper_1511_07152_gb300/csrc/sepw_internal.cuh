@@ -418,15 +418,54 @@ constexpr int kMaxWindow = 64;    // T + S - 1 <= kMaxWindow
 //     against 438 us: its writes go to four times as many places) and the
 //     runs no longer; without conj apart the S = 8 gridder took 190 us
 //     against 181 us (4M visibilities).
-//   kBinsTile: one bin, for the tensor-core forms, which take any order
-//     (8M visibilities, T = 16: plan 308 -> 178 us with 32 bins -> 1).
-enum PlanBins { kBinsWindow, kBinsSorted, kBinsTile };
+//   kBinsFine: edge 4 (T > 32: as kBinsSorted), conj apart as far as 64 bins
+//     go, for grids of few tiles: locate_bin_kernel sends an atomic per warp
+//     and bin to the counters, and those of few bins lie in few L2 sectors,
+//     where they queue.
+//   kBinsTile: one bin, for the tensor-core forms, which take any order.
+// Which one: plan_bins.
+enum PlanBins { kBinsWindow, kBinsSorted, kBinsFine, kBinsTile };
 inline void set_bins(DevParams &d, PlanBins b)
 {
-    d.sub_log2 = b == kBinsWindow ? 2 : b == kBinsTile ? 6 : d.T <= 32 ? 3 : 4;
+    if (b == kBinsFine && d.T > 32)
+        b = kBinsSorted;
+    d.sub_log2 = b == kBinsWindow || b == kBinsFine ? 2
+               : b == kBinsTile                     ? 6
+               : d.T <= 32                          ? 3
+                                                    : 4;
     d.sub_n = (d.T + (1 << d.sub_log2) - 1) >> d.sub_log2;
-    d.sub_conj = b == kBinsSorted ? 1 : 0;
+    d.sub_conj = b == kBinsSorted || (b == kBinsFine && d.sub_n * d.sub_n <= 32) ? 1 : 0;
     d.nsub = (d.sub_n * d.sub_n) << d.sub_conj;
+}
+
+// Bins of a plan that the window gridder does not take.
+//
+// Few tiles: the finer of the two block edges while the coarser one leaves few
+// counters, at most 32768 for the tiled form, 12288 for the tensor-core forms
+// (T = 26 of S = 6 has the same 32 bins either way, and with edge 4 none for
+// conj).  Steps with edge 8 and edge 4, 4M visibilities in random order (d) or
+// on tracks (t): tiled, S = 8, T = 32: 256^2 d 663 and 555 us, 1024^2 (32768
+// counters) d 626 and 605, t 489 and 461, 2048^2 (131072) d 733 and 740, t 522
+// and 525.  BF16: S = 16 256^2 d 693 and 557, S = 12 512^2 (12168) t 500 and
+// 478, S = 6 512^2 (12800) d 536 and 532, t 459 and 482, S = 16 1024^2 (32768)
+// d 578 and 568, t 469 and 477, S = 6 1024^2 (51200) t 453 and 473.
+//
+// One bin for the 16-bit tensor-core forms (their order within a tile is worth
+// 2% to the kernels) where its counters are many, or the visibilities few
+// enough that the scan of the bins counts for more than the queue at the
+// counters.  Steps with one bin and edge 8, BF16: 16384 tiles 740 and 746 us
+// (random order) and 512 and 516 (tracks), 65536 tiles 1718 and 1764, 579 and
+// 618; but 6241 tiles 630 and 596, and 256 tiles 935 and 693 (557 with edge
+// 4).  600k on 10404 tiles 306 and 314, 30k on 100 tiles 65 and 69 (tracks);
+// 100k on 400 tiles 80 and 73.
+inline PlanBins plan_bins(const DevParams &p, int form, int64_t nvis, int64_t ntiles)
+{
+    const bool sorts = form == SEPW_FORM_TILED || form == SEPW_FORM_TC_TF32;
+    if (!sorts && (ntiles >= 16384 || nvis < 64 * ntiles || nvis <= 32768))
+        return kBinsTile;
+    DevParams d = p;
+    set_bins(d, kBinsSorted);
+    return ntiles * d.nsub <= (form == SEPW_FORM_TILED ? 32768 : 12288) ? kBinsFine : kBinsSorted;
 }
 constexpr int kMaxSubBins = 64;
 

@@ -179,7 +179,7 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     pl.sorted = !pl.window;
     set_units(dp, num_sms, pl);
     dp.early = 1;
-    set_bins(dp, pl.window ? kBinsWindow : kBinsSorted);
+    set_bins(dp, pl.window ? kBinsWindow : plan_bins(dp, SEPW_FORM_TILED, nvis, ntiles));
     float *tables = (float *)(b + kOffTables);
     if (!pl.window && sizeof(float2) * dp.P * dp.OS * (size_t)dp.S > kTablesBytes)
         tables = nullptr;
