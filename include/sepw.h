@@ -330,8 +330,10 @@ SEPW_API int sepw_test_fail_alloc(sepw_ctx *ctx, int32_t k);
  *       sum_{cu,cv} grid[cv][cu] exp(2 pi i ((cu-N/2) nu_a + (cv-N/2) nu_b))
  *       = GRID_TO_IMAGE / n_ab^2.
  * FP32.  The directions towards the image run the library's own transforms at
- * N = 512, 1024, 2048 and 4096 (buf 16-byte aligned), everything else cuFFT C2C;
- * twiddles and the cuFFT plan are made on first use. */
+ * N = 512, 1024, 2048 and 4096 (buf 16-byte aligned), everything else cuFFT C2C.
+ * The cuFFT plan is made by the first call in any direction that is not being
+ * captured; captured calls that use cuFFT need one before them, the library's own
+ * transforms none. */
 SEPW_API int sepw_image(sepw_ctx *ctx, int direction, float *buf, sepw_stream_t stream);
 
 /* Taper of the grid correction: taper[a] = c1(nu_a), nu_a = (a - N/2)/N, the

@@ -50,8 +50,7 @@ struct sepw_ctx {
     Plan plan;
     cufftHandle fft = 0;
     bool fft_ready = false;
-    float2 *d_rows_tab = nullptr;  // twiddles of our own transforms
-    bool rows_ready = false;
+    float2 *d_rows_tab = nullptr;  // twiddles of our own transforms (rows_supported sizes)
     // hybrid W stacking: slice centres of the last sepw_wstack_plan and the
     // workspace of the slice sort
     std::vector<double> ws_centres;
@@ -413,6 +412,8 @@ int sepw_create(sepw_ctx **out, const sepw_params *p)
     if ((rc = grow(ctx, &ctx->d_taper64, N)) || (rc = grow(ctx, &ctx->d_taper32, N)) ||
         (rc = grow(ctx, &ctx->d_tw, (size_t)N * p->oversample)) ||
         (rc = grow(ctx, &ctx->d_status, 1)) ||
+        (rows_supported(N) &&
+         (rc = grow(ctx, &ctx->d_rows_tab, rows_table_bytes(N) / sizeof(float2)))) ||
         (rc = grow(ctx, &ctx->d_planar,
                    std::max(2 * 2 * sepw_taps_count(p),
                             ctx->window ? window_tables_bytes(ctx->dp) / sizeof(float) : 0)))) {
@@ -424,6 +425,9 @@ int sepw_create(sepw_ctx **out, const sepw_params *p)
         e = launch_taper(ctx->dp, ctx->d_taper64, ctx->d_taper32, 0);
     if (e == cudaSuccess)
         e = launch_twiddles(ctx->dp, ctx->d_tw, 0);
+    // (here, so that the first image step of any direction can be captured)
+    if (e == cudaSuccess && ctx->d_rows_tab)
+        e = launch_rows_tables(ctx->dp, ctx->d_tw, ctx->d_rows_tab, 0);
     if (e == cudaSuccess)
         e = cudaStreamSynchronize(0);
     if (e != cudaSuccess) {
@@ -842,6 +846,18 @@ int sepw_test_fail_alloc(sepw_ctx *ctx, int32_t k)
     return SEPW_OK;
 }
 
+// Whether work on s goes into a graph instead of running (also where the legacy
+// stream may not be used because of another stream's capture)
+static bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // The context's 2-D transform, on stream s
 static int ensure_fft(sepw_ctx *ctx, cudaStream_t s)
 {
@@ -854,22 +870,6 @@ static int ensure_fft(sepw_ctx *ctx, cudaStream_t s)
     }
     if (cufftSetStream(ctx->fft, s) != CUFFT_SUCCESS)
         return fail(ctx, SEPW_ECUDA, "cufftSetStream failed");
-    return SEPW_OK;
-}
-
-// The twiddles of our own transforms
-static int ensure_rows(sepw_ctx *ctx, cudaStream_t s)
-{
-    if (ctx->rows_ready)
-        return SEPW_OK;
-    int rc;
-    if (!ctx->d_rows_tab && (rc = grow(ctx, &ctx->d_rows_tab,
-                                       rows_table_bytes(ctx->p.grid_size) / sizeof(float2))))
-        return rc;
-    SEPW_CUDA(ctx, launch_rows_tables(ctx->dp, ctx->d_tw, ctx->d_rows_tab, s));
-    // later calls may come on other streams
-    SEPW_CUDA(ctx, cudaStreamSynchronize(s));
-    ctx->rows_ready = true;
     return SEPW_OK;
 }
 
@@ -893,8 +893,10 @@ int sepw_image(sepw_ctx *ctx, int direction, float *buf, sepw_stream_t stream)
     cudaStream_t s = (cudaStream_t)stream;
     if (direction != SEPW_IMAGE_TO_GRID && rows_supported(ctx->p.grid_size) &&
         ((uintptr_t)buf & 15) == 0) {
-        if ((rc = ensure_rows(ctx, s)))
-            return rc;
+        // one call in any direction prepares them all for a later capture (a
+        // failure is left for the call that needs the plan)
+        if (!ctx->fft_ready && !capturing(s))
+            (void)ensure_fft(ctx, s);
         SEPW_CUDA(ctx, launch_columns(ctx->dp, true, 1, ctx->d_rows_tab, (float2 *)buf,
                                       ctx->num_sms, s));
         SEPW_CUDA(ctx, launch_rows_to_image(ctx->dp, direction == SEPW_GRID_TO_IMAGE ? 1 : 2,
@@ -1242,8 +1244,6 @@ int sepw_wstack_image(sepw_ctx *ctx, float *slice_grids, float *image, sepw_stre
     const int L = (int)ctx->ws_centres.size();
     cudaStream_t s = (cudaStream_t)stream;
     if (wstack_rows(ctx, slice_grids, image)) {
-        if ((rc = ensure_rows(ctx, s)))
-            return rc;
         SEPW_CUDA(ctx, launch_columns(ctx->dp, true, L, ctx->d_rows_tab, (float2 *)slice_grids,
                                       ctx->num_sms, s));
         SEPW_CUDA(ctx, launch_slices_to_image(ctx->dp, L, ctx->d_taper32, ctx->d_ws_c32,
@@ -1280,8 +1280,6 @@ int sepw_wstack_model_grids(sepw_ctx *ctx, const float *image, float *slice_grid
     const int L = (int)ctx->ws_centres.size();
     cudaStream_t s = (cudaStream_t)stream;
     if (wstack_rows(ctx, slice_grids, image)) {
-        if ((rc = ensure_rows(ctx, s)))
-            return rc;
         SEPW_CUDA(ctx, launch_image_to_slices(ctx->dp, L, ctx->d_taper32, ctx->d_ws_c32,
                                               ctx->d_rows_tab, (const float2 *)image,
                                               (float2 *)slice_grids, s));

@@ -102,3 +102,47 @@ def test_wstack_directions(env, N, layout):
     S.sepw_wstack_model_grids(ctx, image, grids)
     want = np.stack([_to_grid(x * np.conj(ph[c]) * corr / n ** 2) for c in range(L)])
     assert rel_l2(grids.cpu().numpy(), want) <= TOL
+
+
+@pytest.mark.parametrize("warm,direction", [
+    (None, "GRID_TO_IMAGE"), ("IMAGE_TO_GRID", "GRID_TO_IMAGE"),
+    ("IMAGE_TO_GRID", "IMAGE_TO_GRID_ADJOINT"), ("GRID_TO_IMAGE", "IMAGE_TO_GRID")])
+def test_first_call_in_a_direction_can_be_captured(env, warm, direction):
+    """One call in any direction (towards the image: none) is all that a capture
+    in another one needs."""
+    torch, S = env
+    N = 512
+    ctx = S.sepw_create(S.make_params(N, math.radians(3.0), 4, 3, 2, 100.0))
+    if warm:
+        S.sepw_image(ctx, getattr(S, warm), torch.zeros((N, N), dtype=torch.complex64,
+                                                        device="cuda"))
+    d = getattr(S, direction)
+    buf = torch.zeros((N, N), dtype=torch.complex64, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        S.sepw_image(ctx, d, buf)
+    x = torch.from_numpy(_random(np.random.default_rng(4), N, N)).cuda()
+    buf.copy_(x)
+    graph.replay()
+    want = x.clone()
+    S.sepw_image(ctx, d, want)
+    assert torch.equal(torch.view_as_real(buf), torch.view_as_real(want))
+
+
+def test_first_wstack_image_can_be_captured(env):
+    torch, S = env
+    N = 512
+    ctx = S.sepw_create(S.make_params(N, math.radians(3.0), 4, 3, 2, 100.0))
+    u = torch.zeros(4, dtype=torch.float64, device="cuda")
+    S.sepw_wstack_plan(ctx, [-50.0, 50.0], u, u, u)
+    g = torch.zeros((2, N, N), dtype=torch.complex64, device="cuda")
+    image = torch.zeros((N, N), dtype=torch.complex64, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        S.sepw_wstack_image(ctx, g, image)
+    x = torch.from_numpy(_random(np.random.default_rng(5), 2, N, N)).cuda()
+    g.copy_(x)
+    graph.replay()
+    got = image.clone()
+    S.sepw_wstack_image(ctx, x, image)
+    assert torch.equal(torch.view_as_real(got), torch.view_as_real(image))
