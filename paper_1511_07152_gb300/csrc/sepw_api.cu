@@ -210,6 +210,18 @@ bool is_device_ptr(const void *ptr)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Whether work on s goes into a graph instead of running (also where the legacy
+// stream may not be used because of another stream's capture)
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 int check_dev(sepw_ctx *ctx, const void *ptr, const char *name, bool allow_null)
 {
     if (!ptr)
@@ -846,18 +858,6 @@ int sepw_test_fail_alloc(sepw_ctx *ctx, int32_t k)
     return SEPW_OK;
 }
 
-// Whether work on s goes into a graph instead of running (also where the legacy
-// stream may not be used because of another stream's capture)
-static bool capturing(cudaStream_t s)
-{
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
-        cudaGetLastError();
-        return true;
-    }
-    return st != cudaStreamCaptureStatusNone;
-}
-
 // The context's 2-D transform, on stream s
 static int ensure_fft(sepw_ctx *ctx, cudaStream_t s)
 {
@@ -1005,20 +1005,27 @@ static int residual_pass_check(sepw_ctx *ctx, int32_t Sr, int32_t OSr, const flo
     return check_dev(ctx, table, "table", false);
 }
 
-// Sorts the items of a plan made without it before the first correction pass,
-// whose kernels walk runs of one origin, if there is a visibility per four
-// cells to make runs (2M visibilities on 1024^2 at S = 12: step 1366 -> 513
-// us).  The order inside a bin is free, so every other kernel can use the plan
-// as before.  (The tiled degridder did not gain by it: 1440 us either way for
-// a step of 8M at S = 12.)
-static int sort_for_runs(sepw_ctx *ctx, cudaStream_t s)
+// Sorts the items of a plan made without it.  The order inside a bin is free,
+// so every other kernel can use the plan as before.
+static int sort_items(sepw_ctx *ctx, cudaStream_t s)
 {
     Plan &pl = ctx->plan;
-    if (pl.sorted || 4 * pl.nvis < (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N)
+    if (pl.sorted)
         return SEPW_OK;
-    SEPW_CUDA(ctx, launch_item_sort(ctx->dp, pl, ctx->num_sms, s));
-    pl.sorted = true;
+    SEPW_CUDA(ctx, launch_item_sort(ctx->dp, pl, ctx->num_sms, true, s));
+    pl.sorted = !capturing(s);  // a captured sort has not run yet
     return SEPW_OK;
+}
+
+// Before a correction pass, whose kernels walk runs of one origin: worth it
+// with a visibility per four cells to make runs (2M visibilities on 1024^2 at
+// S = 12: step 1366 -> 513 us).
+static int sort_for_runs(sepw_ctx *ctx, cudaStream_t s)
+{
+    const Plan &pl = ctx->plan;
+    if (4 * pl.nvis < (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N)
+        return SEPW_OK;
+    return sort_items(ctx, s);
 }
 
 int sepw_grid_residual_planned(sepw_ctx *ctx, int32_t support_r, int32_t oversample_r,

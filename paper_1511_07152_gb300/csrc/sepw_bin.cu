@@ -402,7 +402,7 @@ static int sort_keys(const DevParams &p)
 }
 
 __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
-    DevParams p, const WorkItem *items, const int32_t *nitems,
+    DevParams p, const WorkItem *items, const int32_t *nitems, const int32_t *mark,
     Slot *__restrict__ slots)
 {
     extern __shared__ int32_t hist[];  // per * kSortThreads bins
@@ -410,6 +410,8 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
     __shared__ int32_t s_perm[kChunk];
     __shared__ int32_t s_wsum[32];
     pdl_enter(p);
+    if (mark && *mark)
+        return;
     // blocks stride over the plan's items (sparse plans have far fewer items
     // than their capacity, so the grid is sized by the SM count, not by it)
     const int n_items = *nitems;
@@ -630,15 +632,18 @@ cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
         if (e != cudaSuccess)
             return e;
         if (plan.sorted)
-            return launch_item_sort(p, plan, num_sms, s);
+            return launch_item_sort(p, plan, num_sms, false, s);
     }
     return cudaSuccess;
 }
 
 // The per-item sort serves the kernels that walk runs of one origin; the
 // 16-bit tensor-core forms and the window gridder take any order within a bin
-// and leave it out until a call that gains by it (sort_for_runs).
-cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, cudaStream_t s)
+// and leave it out until a call that gains by it.  That call may be captured
+// into a graph, so whether the sort has run is known on the device alone: the
+// mark makes every later one a launch that returns at once.
+cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, bool marked,
+                             cudaStream_t s)
 {
     const int nb = sort_keys(p);
     const size_t shm = sizeof(int32_t) * kSortThreads * ((nb + kSortThreads - 1) / kSortThreads);
@@ -646,8 +651,13 @@ cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, 
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     if (e != cudaSuccess)
         return e;
+    int32_t *const mark = (int32_t *)(plan.d_bin_base + kBinSortMark);
     const int nblk = std::max(1, std::min(plan.items_capacity, 16 * num_sms));
-    return launch_pdl(item_sort_kernel, nblk, kSortThreads, shm, s, p, plan.d_items, plan.d_nitems, plan.d_slots);
+    e = launch_pdl(item_sort_kernel, nblk, kSortThreads, shm, s, p, plan.d_items, plan.d_nitems,
+                   marked ? mark : nullptr, plan.d_slots);
+    if (e == cudaSuccess && marked)
+        e = cudaMemsetAsync(mark, 1, sizeof(*mark), s);
+    return e;
 }
 
 }  // namespace sepw

@@ -470,8 +470,9 @@ inline PlanBins plan_bins(const DevParams &p, int form, int64_t nvis, int64_t nt
 constexpr int kMaxSubBins = 64;
 
 // the plan's bins follow a header that is cleared with them: the dropped
-// count (8 bytes), then the tile passes' ticket
-constexpr size_t kBinHeader = 64, kBinTicket = 8;
+// count (8 bytes), then the tile passes' ticket and the mark of a plan whose
+// items were sorted after it was made (launch_item_sort)
+constexpr size_t kBinHeader = 64, kBinTicket = 8, kBinSortMark = 12;
 
 // ceil(2^32 / T) for the tile edge T (8 <= T <= 64)
 // Bounds of locate_axis's integer path for grid size N and OS = 2^os_log2
@@ -525,7 +526,7 @@ struct Plan {
     int32_t unit = 256;         // most visibilities per unit
     int32_t unit_parts = 1;     // units are at most this part of their tile
     bool valid = false;
-    bool sorted = true;         // items sorted by (block, origin, conj)
+    bool sorted = true;         // items known to be sorted by (block, origin, conj)
     bool window = false;        // gridding by the window gridder
     int form = 0;
     // tiled forms
@@ -593,7 +594,10 @@ bool plan_window(const DevParams &p, int64_t nvis, int ngrids);
 cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
                         const double *v, const double *w, Plan &plan, int num_sms,
                         cudaStream_t s);
-cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, cudaStream_t s);
+// sorts every item by (block, origin, conj); marked: unless an earlier such
+// launch on the same plan has done it
+cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, bool marked,
+                             cudaStream_t s);
 // batched: plan.ngrids > 1 and plan.d_offsets hold the per-grid ranges
 cudaError_t launch_zero_dropped(const Plan &plan, float2 *vis, cudaStream_t s);
 
