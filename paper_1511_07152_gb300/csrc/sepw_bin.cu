@@ -647,8 +647,11 @@ cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, 
 {
     const int nb = sort_keys(p);
     const size_t shm = sizeof(int32_t) * kSortThreads * ((nb + kSortThreads - 1) / kSortThreads);
+    // the largest size, not this plan's: the limit belongs to the kernel, and
+    // another thread's context may launch it with more in between
     cudaError_t e = cudaFuncSetAttribute(item_sort_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(int32_t) * kMaxSortBins);
     if (e != cudaSuccess)
         return e;
     int32_t *const mark = (int32_t *)(plan.d_bin_base + kBinSortMark);
