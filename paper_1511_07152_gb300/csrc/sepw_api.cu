@@ -310,6 +310,7 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     // for the kernels that walk runs of one origin: the tiled form's block and
     // column gridders, and the tiled degridder of the TF32 form
     pl.sorted = sorts && !pl.window;
+    pl.predictions = 0;
     return SEPW_OK;
 }
 
@@ -677,6 +678,45 @@ int sepw_grid_planned(sepw_ctx *ctx, const float *taps, const float *vis,
     return SEPW_OK;
 }
 
+// Sorts the items of a plan made without it.  The order inside a bin is free,
+// so every other kernel can use the plan as before.
+static int sort_items(sepw_ctx *ctx, cudaStream_t s)
+{
+    Plan &pl = ctx->plan;
+    if (pl.sorted)
+        return SEPW_OK;
+    SEPW_CUDA(ctx, launch_item_sort(ctx->dp, pl, ctx->num_sms, true, s));
+    pl.sorted = !capturing(s);  // a captured sort has not run yet
+    return SEPW_OK;
+}
+
+// Before a correction pass, whose kernels walk runs of one origin: worth it
+// with a visibility per four cells to make runs (2M visibilities on 1024^2 at
+// S = 12: step 1366 -> 513 us).
+static int sort_for_runs(sepw_ctx *ctx, cudaStream_t s)
+{
+    const Plan &pl = ctx->plan;
+    if (4 * pl.nvis < (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N)
+        return SEPW_OK;
+    return sort_items(ctx, s);
+}
+
+// From the second prediction on one plan: a program that keeps its plan gets
+// the order that the column and block degridders gain by, one that does not
+// pays nothing.  6M visibilities on 2048^2 at S = 12: predictions 421 -> 318 us
+// on tracks, 439 -> 420 in random order, for one sort of 56 and 81 us; 1.5M on
+// 4096^2 at S = 14 251 -> 216 and 306 -> 305; 400k at S = 6 on 1000^2 52 -> 44.
+// Above S = 16 the window degridder is the faster one on any order.
+static int sort_for_predictions(sepw_ctx *ctx, cudaStream_t s)
+{
+    Plan &pl = ctx->plan;
+    if (pl.form != SEPW_FORM_TILED || pl.predictions++ == 0 || ctx->dp.S > 16 ||
+        pl.nvis < (1 << 18) ||
+        16 * pl.nvis < (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N)
+        return SEPW_OK;
+    return sort_items(ctx, s);
+}
+
 int sepw_degrid_planned(sepw_ctx *ctx, const float *taps, const float *grid,
                         const float *weight, float *vis_out, sepw_stream_t stream)
 {
@@ -708,6 +748,8 @@ int sepw_degrid_planned(sepw_ctx *ctx, const float *taps, const float *grid,
     } else {
         if (((uintptr_t)taps) & 15)
             return fail(ctx, SEPW_EINVAL, "taps must be 16-byte aligned");
+        if ((rc = sort_for_predictions(ctx, s)))
+            return rc;
         SEPW_CUDA(ctx, launch_zero_dropped(pl, (float2 *)vis_out, s));
         if (pl.form == SEPW_FORM_TC_BF16 || pl.form == SEPW_FORM_TC_FP16 ||
             pl.form == SEPW_FORM_TC_FP16X2 || pl.form == SEPW_FORM_TC_BF16X2) {
@@ -1003,29 +1045,6 @@ static int residual_pass_check(sepw_ctx *ctx, int32_t Sr, int32_t OSr, const flo
         return fail(ctx, SEPW_EINVAL, "need 1 <= support_r <= S, S - support_r even, "
                                       "oversample_r dividing OS");
     return check_dev(ctx, table, "table", false);
-}
-
-// Sorts the items of a plan made without it.  The order inside a bin is free,
-// so every other kernel can use the plan as before.
-static int sort_items(sepw_ctx *ctx, cudaStream_t s)
-{
-    Plan &pl = ctx->plan;
-    if (pl.sorted)
-        return SEPW_OK;
-    SEPW_CUDA(ctx, launch_item_sort(ctx->dp, pl, ctx->num_sms, true, s));
-    pl.sorted = !capturing(s);  // a captured sort has not run yet
-    return SEPW_OK;
-}
-
-// Before a correction pass, whose kernels walk runs of one origin: worth it
-// with a visibility per four cells to make runs (2M visibilities on 1024^2 at
-// S = 12: step 1366 -> 513 us).
-static int sort_for_runs(sepw_ctx *ctx, cudaStream_t s)
-{
-    const Plan &pl = ctx->plan;
-    if (4 * pl.nvis < (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N)
-        return SEPW_OK;
-    return sort_items(ctx, s);
 }
 
 int sepw_grid_residual_planned(sepw_ctx *ctx, int32_t support_r, int32_t oversample_r,

@@ -527,6 +527,7 @@ struct Plan {
     int32_t unit_parts = 1;     // units are at most this part of their tile
     bool valid = false;
     bool sorted = true;         // items known to be sorted by (block, origin, conj)
+    int64_t predictions = 0;    // degridding calls since the plan was made
     bool window = false;        // gridding by the window gridder
     int form = 0;
     // tiled forms

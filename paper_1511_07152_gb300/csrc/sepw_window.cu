@@ -664,9 +664,26 @@ cudaError_t launch_grid_window(const DevParams &p, const Plan &plan, const float
 // supports without a block degridder, but for 2, 6 and 14 (see the kernel)
 #define SEPW_FOR_EACH_DEGRID_S(X) X(10) X(18) X(20) X(22) X(24) X(26) X(28) X(30) X(32)
 
+// Left to the column degridder:
+//   * small plans of medium density: its CTAs take parts of an item, the
+//     window's warps whole units, one visibility after the other.  20k on
+//     1000^2 (21 a tile), random order: S = 10 38 us with the window and 17
+//     with the columns, S = 18 56 and 23; 100k on 2048^2 (24 a tile) S = 10 62
+//     and 42, on tracks 31 and 29, S = 18 98 and 63, 46 and 49; 100k on 1000^2
+//     (104 a tile) S = 10 45 and 31, 31 and 26.  But there S = 24 76 and 79, 47
+//     and 66, and 100k on 4096^2 (6 a tile, and a tile's cells loaded for each)
+//     S = 10 69 and 155;
+//   * sorted plans at S = 10: 6M on 1000^2, tracks 585 and 473 us, random order
+//     640 and 564; 1.5M 165 and 142, 184 and 194.  (S = 18: 1054 and 1108,
+//     1124 and 1300.)
+// Sparse plans in random order are slower with the window from there on (400k
+// on 2048^2, S = 18: 168 and 148 us), tracks faster (114 and 149).
 bool degrid_window_takes(const DevParams &p, const Plan &plan)
 {
-    if (!plan.window)
+    const int64_t tiles = plan.ntiles;
+    if (!plan.window || (p.S == 10 && plan.sorted) ||
+        (plan.nvis <= (128 << 10) && plan.nvis >= 12 * tiles &&
+         plan.nvis <= (p.S == 10 ? 512 : 64) * tiles))
         return false;
     switch (p.S) {
 #define X(SS) case SS:

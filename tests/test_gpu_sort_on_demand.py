@@ -121,3 +121,39 @@ def test_captured_correction_pass_leaves_the_plan_to_the_next(env):
     graph.replay()
     assert rel_l2(st.grid.cpu().numpy(), want.cpu().numpy()) <= TOL
     st.check()
+
+
+@pytest.mark.parametrize("support", [4, 6, 10, 12, 14, 16, 18])
+def test_second_prediction_sorts(env, support):
+    """At the smallest size that sorts: the second prediction does, up to S = 16
+    (S = 16 below a visibility per four cells, where its plan is unsorted), and
+    later ones find the plan sorted; every prediction is the oracle's."""
+    st = Step(env, support, nvis=1 << 18, N=1100 if support == 16 else 600)
+    st.plan()
+    assert _sorts(st.torch, st.degrid) == 0
+    st.check()
+    assert _sorts(st.torch, st.degrid) == 0  # the third: check() was the second
+    st.check()
+    st.plan()
+    st.degrid()
+    assert _sorts(st.torch, st.degrid) == (1 if support <= 16 else 0)
+
+
+@pytest.mark.parametrize("support", [10, 18])
+@pytest.mark.parametrize("nvis,N", [(300, 230), (600, 230), (3_136, 230), (3_137, 230),
+                                    (25_088, 230), (25_089, 230), (131_072, 512),
+                                    (131_073, 512)])
+def test_small_predictions(env, support, nvis, N):
+    """Both sides of the lines between the window and the column degridder (49
+    tiles at S = 10 or 18 on 230^2)."""
+    st = Step(env, support, nvis=nvis, N=N)
+    st.plan()
+    st.check()
+
+
+def test_few_cells_per_visibility_stay_unsorted(env):
+    st = Step(env, 12, nvis=1 << 18, N=2100)
+    st.plan()
+    st.degrid()
+    assert _sorts(st.torch, st.degrid) == 0
+    st.check()
