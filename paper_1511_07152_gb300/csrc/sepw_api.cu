@@ -43,10 +43,12 @@ struct sepw_ctx {
     unsigned char *d_tc2 = nullptr;
     size_t tc2_cap = 0;
     // workspace of the tiled gridders' copies of the caller's tap table(s):
-    // the block gridder's planar copy (two tables in facet mode) or the
-    // window gridder's padded ones
+    // the block gridder's planar copy (two tables in facet mode), and the
+    // window kernels' padded ones (window_bytes, 0: they do not take these
+    // parameters), allocated by the first plan that takes them
     float *d_planar = nullptr;
-    bool window = false;  // the tiled form can grid with the window gridder
+    float *d_window = nullptr;
+    size_t window_bytes = 0;
     Plan plan;
     cufftHandle fft = 0;
     bool fft_ready = false;
@@ -233,7 +235,7 @@ int check_dev(sepw_ctx *ctx, const void *ptr, const char *name, bool allow_null)
     return SEPW_OK;
 }
 
-int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
+int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids, cudaStream_t s)
 {
     Plan &pl = ctx->plan;
     int rc;
@@ -244,8 +246,12 @@ int ensure_plan_capacity(sepw_ctx *ctx, int64_t nvis, int ngrids)
     // at most 2^26 tiles of 32 bins: the ids fit int32; with more bins a tile
     // (the window gridder's, fine ones) the tiles have to be fewer
     const bool sorts = ctx->p.form == SEPW_FORM_TILED || ctx->p.form == SEPW_FORM_TC_TF32;
-    pl.window = ctx->window && plan_window(ctx->dp, nvis, ngrids) &&
+    pl.window = plan_window(ctx->dp, ctx->window_bytes, nvis, ngrids) &&
                 ntiles64 * kMaxSubBins <= (1ll << 31);
+    // (no allocation inside a capture that worked without one)
+    if (pl.window && !ctx->d_window &&
+        (capturing(s) || grow(ctx, &ctx->d_window, ctx->window_bytes / sizeof(float))))
+        pl.window = false;
     set_bins(ctx->dp, pl.window ? kBinsWindow : plan_bins(ctx->dp, ctx->p.form, nvis, ntiles64));
     if (!pl.d_nitems && (rc = grow(ctx, &pl.d_nitems, 2)))
         return rc;
@@ -420,16 +426,13 @@ int sepw_create(sepw_ctx **out, const sepw_params *p)
         return SEPW_ECUDA;
     }
     const int N = p->grid_size;
-    ctx->window = p->form == SEPW_FORM_TILED && p->support != 8 &&  // see plan_window
-                  window_tables_bytes(ctx->dp) > 0;
+    ctx->window_bytes = p->form == SEPW_FORM_TILED ? window_tables_bytes(ctx->dp) : 0;
     if ((rc = grow(ctx, &ctx->d_taper64, N)) || (rc = grow(ctx, &ctx->d_taper32, N)) ||
         (rc = grow(ctx, &ctx->d_tw, (size_t)N * p->oversample)) ||
         (rc = grow(ctx, &ctx->d_status, 1)) ||
         (rows_supported(N) &&
          (rc = grow(ctx, &ctx->d_rows_tab, rows_table_bytes(N) / sizeof(float2)))) ||
-        (rc = grow(ctx, &ctx->d_planar,
-                   std::max(2 * 2 * sepw_taps_count(p),
-                            ctx->window ? window_tables_bytes(ctx->dp) / sizeof(float) : 0)))) {
+        (rc = grow(ctx, &ctx->d_planar, 2 * 2 * sepw_taps_count(p)))) {
         sepw_destroy(ctx);
         return rc;
     }
@@ -477,6 +480,7 @@ void sepw_destroy(sepw_ctx *ctx)
     cudaFree(ctx->d_tw);
     cudaFree(ctx->d_status);
     cudaFree(ctx->d_planar);
+    cudaFree(ctx->d_window);
     cudaFree(ctx->d_rows_tab);
     cudaFree(ctx->d_tc2);
     free_plan(ctx->plan);
@@ -545,7 +549,7 @@ static int plan_impl(sepw_ctx *ctx, int32_t ngrids, const int64_t *offsets_host,
                      (rc = check_dev(ctx, v, "v", false)) ||
                      (rc = check_dev(ctx, w, "w", false))))
         return rc;
-    if ((rc = ensure_plan_capacity(ctx, nvis, ngrids)))
+    if ((rc = ensure_plan_capacity(ctx, nvis, ngrids, s)))
         return rc;
     Plan &pl = ctx->plan;
     pl.form = ctx->p.form;
@@ -672,8 +676,9 @@ int sepw_grid_planned(sepw_ctx *ctx, const float *taps, const float *vis,
         DevParams dp = ctx->dp;
         dp.chk_status = ctx->d_status;  // the checked build's bounds failures
         SEPW_CUDA(ctx, launch_grid_tiled(dp, pl, (const float2 *)vis, weight,
-                                         (const float2 *)taps, ctx->d_planar, (float2 *)grid,
-                                         ctx->num_sms, s));
+                                         (const float2 *)taps,
+                                         pl.window ? ctx->d_window : ctx->d_planar,
+                                         (float2 *)grid, ctx->num_sms, s));
     }
     return SEPW_OK;
 }
@@ -765,7 +770,7 @@ int sepw_degrid_planned(sepw_ctx *ctx, const float *taps, const float *grid,
             DevParams dp = ctx->dp;
             dp.chk_status = ctx->d_status;  // the checked build's bounds failures
             SEPW_CUDA(ctx, launch_degrid_tiled(dp, pl, (const float2 *)grid, weight,
-                                               (const float2 *)taps, ctx->d_planar,
+                                               (const float2 *)taps, ctx->d_window,
                                                (float2 *)vis_out, ctx->num_sms, s));
         }
     }

@@ -570,14 +570,26 @@ int64_t max_units(const Plan &plan)
            plan.ntiles + 1;
 }
 
-// Whether the tiled form grids with the window gridder (where its tables can
-// be had): every support without a block gridder, and S = 16 below a
-// visibility per four cells, where runs of one origin are short (524,288
-// visibilities on 2048^2: 155 us with the block gridder, 86 us with the window
-// gridder; 4M: 355 and 468 us).  At S = 8 the block gridder is the faster one (1M on 1024^2: 62 and
-// 74 us; 8M on 15 x 4096^2: 475 and 556 us).
-bool plan_window(const DevParams &p, int64_t nvis, int ngrids)
+// Whether a plan of the tiled form is for the window gridder (table_bytes: what
+// its tap tables take, 0 if it does not take the parameters): every support
+// without a block gridder, and S = 16 below a visibility per four cells, where
+// runs of one origin are short (524,288 visibilities on 2048^2: 155 us with the
+// block gridder, 86 us with the window gridder; 4M: 355 and 468 us).  At S = 8
+// the block gridder is the faster one (1M on 1024^2: 62 and 74 us; 8M on 15 x
+// 4096^2: 475 and 556 us).
+//
+// The tables are built in every call, about 2.3 us a MB, so calls of few
+// visibilities with large tables are left to the column gridder.  Steps on
+// 1000^2, random order (d) and tracks (t), window and column: 3k visibilities,
+// 14 MB (S = 30) d 145 and 98 us, t 189 and 532, 24 MB (S = 12) d 75 and 57, t
+// 79 and 136, 70 MB (S = 20) d 345 and 70, t 390 and 323; 20k, 24 MB (S = 12) d
+// 95 and 70, t 86 and 599, 48 MB d 133 and 69, t 121 and 601; 100k, 48 MB d 134
+// and 136, t 142 and 695.
+bool plan_window(const DevParams &p, size_t table_bytes, int64_t nvis, int ngrids)
 {
+    if (table_bytes == 0 ||
+        table_bytes > std::max<size_t>((size_t)16 << 20, 2048 * (size_t)nvis))
+        return false;
     if (p.S == 16)
         return 4 * nvis < (int64_t)ngrids * p.N * p.N;
     return p.S != 8;

@@ -591,7 +591,7 @@ size_t plan_bin_bytes(int64_t ntiles, const DevParams &p);
 size_t plan_block_bytes(int64_t ntiles);
 void set_units(const DevParams &p, int num_sms, Plan &plan);  // from nvis, ntiles, window
 int64_t max_units(const Plan &plan);
-bool plan_window(const DevParams &p, int64_t nvis, int ngrids);
+bool plan_window(const DevParams &p, size_t table_bytes, int64_t nvis, int ngrids);
 cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
                         const double *v, const double *w, Plan &plan, int num_sms,
                         cudaStream_t s);

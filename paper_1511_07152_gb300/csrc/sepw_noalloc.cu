@@ -175,7 +175,7 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     if (plan_block_bytes(ntiles) > kBlocksBytes)
         return SEPW_ETOOLARGE;
     const size_t wbytes = window_tables_bytes(dp);
-    pl.window = wbytes > 0 && wbytes <= kTablesBytes && plan_window(dp, nvis, 1);
+    pl.window = wbytes <= kTablesBytes && plan_window(dp, wbytes, nvis, 1);
     pl.sorted = !pl.window;
     set_units(dp, num_sms, pl);
     dp.early = 1;
