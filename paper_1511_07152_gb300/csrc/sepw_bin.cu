@@ -571,12 +571,12 @@ int64_t max_units(const Plan &plan)
 }
 
 // Whether a plan of the tiled form is for the window gridder (table_bytes: what
-// its tap tables take, 0 if it does not take the parameters): every support
-// without a block gridder, and S = 16 below a visibility per four cells, where
-// runs of one origin are short (524,288 visibilities on 2048^2: 155 us with the
-// block gridder, 86 us with the window gridder; 4M: 355 and 468 us).  At S = 8
-// the block gridder is the faster one (1M on 1024^2: 62 and 74 us; 8M on 15 x
-// 4096^2: 475 and 556 us).
+// its tap tables take, 0 if it does not take the parameters, S = 8 among them):
+// every support without a block gridder, and S = 16 below a visibility per four
+// cells, where runs of one origin are short (524,288 visibilities on 2048^2:
+// 155 us with the block gridder, 86 us with the window gridder; 4M: 355 and 468
+// us).  At S = 8 the block gridder is the faster one (1M on 1024^2: 62 and 74
+// us; 8M on 15 x 4096^2: 475 and 556 us).
 //
 // The tables are built in every call, about 2.3 us a MB, so calls of few
 // visibilities with large tables are left to the column gridder.  Steps on
@@ -590,9 +590,7 @@ bool plan_window(const DevParams &p, size_t table_bytes, int64_t nvis, int ngrid
     if (table_bytes == 0 ||
         table_bytes > std::max<size_t>((size_t)16 << 20, 2048 * (size_t)nvis))
         return false;
-    if (p.S == 16)
-        return 4 * nvis < (int64_t)ngrids * p.N * p.N;
-    return p.S != 8;
+    return p.S != 16 || 4 * nvis < (int64_t)ngrids * p.N * p.N;
 }
 
 size_t plan_bin_bytes(int64_t ntiles, const DevParams &p)

@@ -625,8 +625,9 @@ static cudaError_t launch_degrid_S(const DevParams &p, const Plan &plan, const f
                       grid, weight, taps, t.u, t.v, t.flags, vis);
 }
 
+// every support but 8, whose block gridder is the faster one (plan_window)
 #define SEPW_FOR_EACH_WIN_S(X) \
-    X(2) X(4) X(6) X(8) X(10) X(12) X(14) X(16) X(18) X(20) X(22) X(24) X(26) X(28) X(30) X(32)
+    X(2) X(4) X(6) X(10) X(12) X(14) X(16) X(18) X(20) X(22) X(24) X(26) X(28) X(30) X(32)
 
 // Bytes of the tables, 0 if the window gridder does not take these
 // parameters: tiles above 32 (a tile has at most 64 blocks of 4 x 4 origins)
