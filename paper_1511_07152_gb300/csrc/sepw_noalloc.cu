@@ -40,7 +40,7 @@ constexpr size_t kOffDrop = align256(kOffSlots + sizeof(Slot) * kMaxVis);
 constexpr int64_t kMaxUnits = kMaxTiles + kMaxVis / 32 + 1;
 constexpr size_t kOffCount = align256(kOffDrop + sizeof(int32_t) * kMaxVis);
 constexpr size_t kOffBlocks = align256(kOffCount + sizeof(int32_t) * kMaxTiles);
-constexpr size_t kBlocksBytes = 64 * 1024;  // plan_block_bytes(kMaxTiles), checked per call
+constexpr size_t kBlocksBytes = 64 * 1024;  // above plan_block_bytes(kMaxTiles): 1025 x 20 bytes
 constexpr size_t kOffBin = align256(kOffBlocks + kBlocksBytes);
 constexpr size_t kOffItems =
     align256(kOffBin + kBinHeader + sizeof(int32_t) * kMaxSubBins * kMaxTiles);
@@ -172,13 +172,11 @@ extern "C" int sepw_grid_noalloc(const sepw_params *prm, const float *taps, int6
     pl.d_nunits = pl.d_nitems + 1;
     pl.d_item_counter = (int32_t *)(b + kOffCounter);
     pl.d_dropped = (unsigned long long *)pl.d_bin_base;
-    if (plan_block_bytes(ntiles) > kBlocksBytes)
-        return SEPW_ETOOLARGE;
     const size_t wbytes = window_tables_bytes(dp);
     pl.window = wbytes <= kTablesBytes && plan_window(dp, wbytes, nvis, 1);
     pl.sorted = !pl.window;
     set_units(dp, num_sms, pl);
-    dp.early = 1;
+    dp.early = nvis <= kEarlyVis ? 1 : 0;
     set_bins(dp, pl.window ? kBinsWindow : plan_bins(dp, SEPW_FORM_TILED, nvis, ntiles));
     float *tables = (float *)(b + kOffTables);
     if (!pl.window && sizeof(float2) * dp.P * dp.OS * (size_t)dp.S > kTablesBytes)
