@@ -53,6 +53,12 @@ struct Win {
     // single row's (re, im); 16-byte multiples unless that loads more
     static constexpr int VG = RPL == 3 ? 6 : (2 * RPL + 3) & ~3;
     static constexpr int VROW = 7 * VG;
+    // gridding adds a visibility's product to a cell's sum as one number: two
+    // FMAs round the sum twice.  Up to S = 6 few visibilities meet in a cell,
+    // and the grid was less exact than with each of them added to it alone,
+    // whose sums are longer (S = 6, 2 visibilities a cell: 1.65e-7 from the
+    // float64 sum, 1.47e-7 alone; S = 12 2.06e-7 and 2.56e-7).
+    static constexpr bool ONE_SUM = S <= 6;
     // resident CTAs per SM the registers are limited to
     static constexpr int BPS = S <= 12 ? 4 : S <= 20 ? 3 : 2;
 };
@@ -300,12 +306,24 @@ __global__ void __launch_bounds__(kWinThreads, Win<S>::BPS) grid_window_kernel(
                         const float spr = sg * pr, spi = sg * pi;
 #pragma unroll
                         for (int k = 0; k < RP; ++k) {
-                            ar[k][c] = __ffma2_rn(vr[k], dup(pr), ar[k][c]);
-                            ar[k][c] = __ffma2_rn(vi[k], dup(-pi), ar[k][c]);
-                            ai[k][c] = __ffma2_rn(vr[k], dup(spi), ai[k][c]);
-                            ai[k][c] = __ffma2_rn(vi[k], dup(spr), ai[k][c]);
+                            if constexpr (W::ONE_SUM) {
+                                const float2 r = __ffma2_rn(vi[k], dup(-pi),
+                                                            __fmul2_rn(vr[k], dup(pr)));
+                                const float2 i = __ffma2_rn(vi[k], dup(spr),
+                                                            __fmul2_rn(vr[k], dup(spi)));
+                                ar[k][c] = __fadd2_rn(ar[k][c], r);
+                                ai[k][c] = __fadd2_rn(ai[k][c], i);
+                            } else {
+                                ar[k][c] = __ffma2_rn(vr[k], dup(pr), ar[k][c]);
+                                ar[k][c] = __ffma2_rn(vi[k], dup(-pi), ar[k][c]);
+                                ai[k][c] = __ffma2_rn(vr[k], dup(spi), ai[k][c]);
+                                ai[k][c] = __ffma2_rn(vi[k], dup(spr), ai[k][c]);
+                            }
                         }
-                        if constexpr (ODD) {
+                        if constexpr (ODD && W::ONE_SUM) {
+                            ae[c].x = __fadd_rn(ae[c].x, fmaf(-ve.y, pi, __fmul_rn(ve.x, pr)));
+                            ae[c].y = __fadd_rn(ae[c].y, fmaf(ve.y, spr, __fmul_rn(ve.x, spi)));
+                        } else if constexpr (ODD) {
                             ae[c].x = fmaf(ve.x, pr, ae[c].x);
                             ae[c].x = fmaf(-ve.y, pi, ae[c].x);
                             ae[c].y = fmaf(ve.x, spi, ae[c].y);
