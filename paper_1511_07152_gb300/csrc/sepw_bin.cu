@@ -384,7 +384,8 @@ __global__ void __launch_bounds__(256) scatter_kernel(
 // never mixes conjugated and plain kernels; the bins stay contiguous inside an
 // item, so a run of slots that starts and ends in one bin lies inside it.  One
 // block of threads per item; the item's slots are rewritten in place.  The
-// order among equal keys is arbitrary.
+// order among equal keys is arbitrary.  recs and ids (or null): the sorted records
+// and visibility indices as two arrays, too (plan_splits).
 constexpr int kSortThreads = 512;
 constexpr int kMaxSortBins = 2 * 64 * 64;
 constexpr int kMaxBinsPerThread = kMaxSortBins / kSortThreads;
@@ -403,7 +404,7 @@ static int sort_keys(const DevParams &p)
 
 __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
     DevParams p, const WorkItem *items, const int32_t *nitems, const int32_t *mark,
-    Slot *__restrict__ slots)
+    Slot *__restrict__ slots, uint64_t *__restrict__ recs, int32_t *__restrict__ ids)
 {
     extern __shared__ int32_t hist[];  // per * kSortThreads bins
     __shared__ uint64_t s_rec[kChunk];
@@ -502,6 +503,10 @@ __global__ void __launch_bounds__(kSortThreads) item_sort_kernel(
         if (act) {
             const int dst = base + __popc(peers & lanemask_lt());
             store_slot(slots + it.start + dst, r, s_perm[q]);
+            if (recs) {
+                recs[it.start + dst] = r;
+                ids[it.start + dst] = s_perm[q];
+            }
         }
     }
     __syncthreads();  // shared memory is reused by the next item
@@ -667,7 +672,8 @@ cudaError_t launch_item_sort(const DevParams &p, const Plan &plan, int num_sms, 
     int32_t *const mark = (int32_t *)(plan.d_bin_base + kBinSortMark);
     const int nblk = std::max(1, std::min(plan.items_capacity, 16 * num_sms));
     e = launch_pdl(item_sort_kernel, nblk, kSortThreads, shm, s, p, plan.d_items, plan.d_nitems,
-                   marked ? mark : nullptr, plan.d_slots);
+                   marked ? mark : nullptr, plan.d_slots,
+                   plan_splits(plan) ? plan.d_rec0 : nullptr, plan.d_rank);
     if (e == cudaSuccess && marked)
         e = cudaMemsetAsync(mark, 1, sizeof(*mark), s);
     return e;

@@ -533,8 +533,10 @@ struct Plan {
     // tiled forms
     int32_t *d_tile = nullptr;      // [nvis] bin id per visibility (-1 dropped)
     int32_t *d_rank = nullptr;      // [nvis] rank of the visibility inside its bin
+                                    // (plan_splits: then visibility index, slot order)
     unsigned char *d_bin_base = nullptr;  // header, then [ntiles * nsub] counts, then slots
-    uint64_t *d_rec0 = nullptr;     // [nvis] record, input order
+    uint64_t *d_rec0 = nullptr;     // [nvis] record, input order (plan_splits: then
+                                    // in slot order)
     Slot *d_slots = nullptr;        // [nvis] records and visibility indices, slot order
     int32_t *d_tile_count = nullptr;   // [ntiles]
     void *d_blocks = nullptr;          // totals of the tile passes' blocks
@@ -554,6 +556,13 @@ struct Plan {
     // plain form: the coordinates are read directly
     const double *u = nullptr, *v = nullptr, *w = nullptr;
 };
+
+// TF32 plans: the sort leaves the records and visibility indices of the slots in
+// d_rec0 and d_rank as well, which the passes before it are done with.  The
+// TF32 gridder is bound by L1 and lost 2 to 6% by slots of 16 bytes (16M
+// visibilities on 1024^2: 1599 us with them, 1514 so; 32M on 4096^2 3249 and
+// 3113); writing the arrays costs the sort 3 to 6% of the plan.
+inline bool plan_splits(const Plan &plan) { return plan.form == SEPW_FORM_TC_TF32; }
 
 // Device-side parameters of a checked sepw_params (sepw_api.cu): derived
 // constants, and the tile edge resolved for the form when p->tile is 0.

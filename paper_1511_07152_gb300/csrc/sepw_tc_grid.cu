@@ -393,7 +393,8 @@ __device__ __forceinline__ bool cursor_seek(Cursor &c, int t, const WorkItem *__
 template <int PREC>
 __global__ void __launch_bounds__(Cfg<PREC>::kBlock, 1) grid_tc2_kernel(
     DevParams p, const WorkItem *__restrict__ items, const int32_t *__restrict__ nitems,
-    const Slot *__restrict__ slots,
+    const Slot *__restrict__ slots, const uint64_t *__restrict__ recs,
+    const int32_t *__restrict__ ids,
     const float2 *__restrict__ vis, const float *__restrict__ weight,
     const uint4 *__restrict__ vtab, const uint4 *__restrict__ utab,
     const float2 *__restrict__ taps, const int32_t *__restrict__ item_exp, float2 *grid,
@@ -461,9 +462,14 @@ __global__ void __launch_bounds__(Cfg<PREC>::kBlock, 1) grid_tc2_kernel(
                 const int e = (t_ - c.tb) * SV + slot0 + 32 * sl + lane;
                 vi_[sl] = -1;
                 if (e < c.count) {
-                    const Slot slot = load_slot_split(slots + c.start + e);
-                    r_[sl] = slot.rec;
-                    vi_[sl] = slot.vis;
+                    if constexpr (C::TF32) {  // plan_splits
+                        r_[sl] = __ldg(recs + c.start + e);
+                        vi_[sl] = __ldg(ids + c.start + e);
+                    } else {
+                        const Slot slot = load_slot_split(slots + c.start + e);
+                        r_[sl] = slot.rec;
+                        vi_[sl] = slot.vis;
+                    }
                 }
             }
 #pragma unroll
@@ -927,8 +933,8 @@ cudaError_t launch_prec(const DevParams &p, const Plan &plan, const float2 *vis,
     if (e != cudaSuccess)
         return e;
     grid_tc2_kernel<PREC><<<num_sms, C::kBlock, C::kSmem, s>>>(
-        p, plan.d_items, plan.d_nitems, plan.d_slots, vis, weight, vtab, utab, taps,
-        item_exp, grid, status, ctl);
+        p, plan.d_items, plan.d_nitems, plan.d_slots, plan.d_rec0, plan.d_rank, vis, weight,
+        vtab, utab, taps, item_exp, grid, status, ctl);
     return cudaGetLastError();
 }
 

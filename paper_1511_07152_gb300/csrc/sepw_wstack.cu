@@ -138,12 +138,16 @@ __global__ void __launch_bounds__(kWsThreads) wstack_scatter_kernel(
 // the caller's visibility indices
 __global__ void __launch_bounds__(256) wstack_compose_kernel(
     int64_t nvis, const unsigned long long *__restrict__ dropped,
-    const int32_t *__restrict__ part, Slot *slots, int32_t *drop_list)
+    const int32_t *__restrict__ part, Slot *slots, int32_t *ids, int32_t *drop_list)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nd = (int64_t)*dropped;
-    if (i < nvis - nd)
-        slots[i].vis = part[slots[i].vis];
+    if (i < nvis - nd) {
+        const int32_t id = part[slots[i].vis];
+        slots[i].vis = id;
+        if (ids)  // plan_splits
+            ids[i] = id;
+    }
     if (i < nd)
         drop_list[i] = part[drop_list[i]];
 }
@@ -185,7 +189,8 @@ cudaError_t launch_wstack_compose(int64_t nvis, const Plan &plan, const int32_t 
     if (nvis == 0)
         return cudaSuccess;
     wstack_compose_kernel<<<(unsigned)((nvis + 255) / 256), 256, 0, s>>>(
-        nvis, plan.d_dropped, part, plan.d_slots, plan.d_drop_list);
+        nvis, plan.d_dropped, part, plan.d_slots, plan_splits(plan) ? plan.d_rank : nullptr,
+        plan.d_drop_list);
     return cudaGetLastError();
 }
 

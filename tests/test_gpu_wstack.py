@@ -154,3 +154,29 @@ def test_wstack_rejects(env):
         with pytest.raises(S.SepwError) as e:
             S.sepw_wstack_plan(ctx, bad, d["u"], d["v"], d["w"])
         assert e.value.status == S.EINVAL
+
+
+def test_wstack_tf32(env):
+    """TF32 plans keep the visibility indices in an array of their own besides the
+    slots: both are in the caller's order (11-bit operands: the forms' 1.5e-3;
+    the prediction is the tiled FP32 form's)."""
+    torch, S = env
+    wl = _case()
+    ctx, taps, d, _ = _plan(torch, S, wl, S.FORM_TC_TF32)
+    N, L = wl.grid_size, len(CENTRES)
+    grids = torch.zeros((L, N, N), dtype=torch.complex64, device="cuda")
+    S.sepw_grid_planned(ctx, taps, d["vis"], d["weight"], grids)
+    p = _params(wl)
+    want, sl, wr = O.wstack_layer_grids(p, wl.u, wl.v, wl.w, wl.vis, wl.weight, CENTRES)
+    assert rel_l2(grids.cpu().numpy(), want) <= 1.5e-3
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((L, N, N, 2)).astype(np.float32).view(np.complex64)[..., 0]
+    out = torch.empty(wl.nvis, dtype=torch.complex64, device="cuda")
+    S.sepw_degrid_planned(ctx, taps, torch.from_numpy(X).cuda(), d["weight"], out)
+    sl, wr = O.wstack_assign(wl.w, CENTRES)
+    got, T = out.cpu().numpy(), O.taps(p)
+    for c in range(L):
+        m = sl == c
+        loc = O.locate(p, wl.u[m], wl.v[m], wr[m])
+        ref = O.degrid_separable(p, loc, X[c].astype(np.complex128), wl.weight[m], T)
+        assert rel_l2(got[m], ref) <= TOL
