@@ -182,9 +182,9 @@ SEPW_API int sepw_locate(sepw_ctx *ctx, int64_t nvis, const double *u, const dou
  * counting sort by tile and by block of footprint origins inside the tile,
  * cut into work items, each sorted by origin where the kernels need it).  The
  * plan is reused by sepw_grid_planned / sepw_degrid_planned until the next
- * sepw_plan; u, v, w need not stay alive.  A correction pass, and the second
- * prediction, sort the items of a plan that was made without (of many
- * visibilities a cell): that call does it, on its stream, and results do not
+ * sepw_plan; u, v, w need not stay alive.  A correction pass, and the first
+ * or second prediction, sort the items of a plan that was made without (by its
+ * visibilities per cell): that call does it, on its stream, and results do not
  * depend on it beyond FP32 rounding order.  Binning is amortisable over the
  * gridding/degridding calls of a major cycle (Sec. 6).  For the plain form
  * the plan only records the coordinates' pointers, which must then stay

@@ -706,18 +706,41 @@ static int sort_for_runs(sepw_ctx *ctx, cudaStream_t s)
     return sort_items(ctx, s);
 }
 
-// From the second prediction on one plan: a program that keeps its plan gets
-// the order that the column and block degridders gain by, one that does not
-// pays nothing.  6M visibilities on 2048^2 at S = 12: predictions 421 -> 318 us
-// on tracks, 439 -> 420 in random order, for one sort of 56 and 81 us; 1.5M on
-// 4096^2 at S = 14 251 -> 216 and 306 -> 305; 400k at S = 6 on 1000^2 52 -> 44.
-// Above S = 16 the window degridder is the faster one on any order.
+// Visibilities per cell from which on the first prediction of a plan of 2^20
+// visibilities or more is worth its sort, 0: none.  Steps without and with it on
+// tracks (t) and in random order (d):
+//   S = 6   1.4 a cell (6M on 2048^2) t 1075 and 982 us, d 1145 and 1171; 6 a
+//           cell (1000^2) t 1051 and 933, d 1130 and 1069
+//   S = 10  4 a cell (4M on 1000^2) d 853 and 895; 6 a cell t 1156 and 1094, d
+//           1244 and 1247; 122 a cell (8M on 256^2) t 1567 and 1479, d 1773 and 1648
+//   S = 12  1.4 a cell t 974 and 927, d 1054 and 1116; 6 a cell t 990 and 921,
+//           d 1027 and 1025
+//   S = 14  0.4 a cell (1.5M on 2048^2) t 474 and 448, d 511 and 542; 1.4 a cell
+//           t 1620 and 1455, d 1710 and 1706; 6 a cell t 1609 and 1436, d 1700
+//           and 1561
+//   S = 4   6 a cell t 531 and 577, d 615 and 687
+// (400k on 256^2, 6 a cell: S = 12 t 118 and 127, d 125 and 136.)
+static int sort_density(int S)
+{
+    return S == 6 || S == 14 ? 1 : S == 12 ? 4 : S == 10 ? 8 : 0;
+}
+
+// Before a prediction: the order that the column and block degridders gain by,
+// made by the first prediction where its step gains, else by the second: a
+// program that keeps its plan gets it, one that does not pays nothing.  6M
+// visibilities on 2048^2 at S = 12: predictions 421 -> 318 us on tracks, 439 ->
+// 420 in random order, for one sort of 56 and 81 us; 1.5M on 4096^2 at S = 14
+// 251 -> 216 and 306 -> 305; 400k at S = 6 on 1000^2 52 -> 44.  Above S = 16 the
+// window degridder is the faster one on any order.
 static int sort_for_predictions(sepw_ctx *ctx, cudaStream_t s)
 {
     Plan &pl = ctx->plan;
-    if (pl.form != SEPW_FORM_TILED || pl.predictions++ == 0 || ctx->dp.S > 16 ||
-        pl.nvis < (1 << 18) ||
-        16 * pl.nvis < (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N)
+    const int S = ctx->dp.S, density = sort_density(S);
+    const int64_t cells = (int64_t)pl.ngrids * ctx->dp.N * ctx->dp.N;
+    if (pl.form != SEPW_FORM_TILED || S > 16 || pl.nvis < (1 << 18) || 16 * pl.nvis < cells)
+        return SEPW_OK;
+    if (pl.predictions++ == 0 &&
+        (density == 0 || pl.nvis < (1 << 20) || pl.nvis < density * cells))
         return SEPW_OK;
     return sort_items(ctx, s);
 }

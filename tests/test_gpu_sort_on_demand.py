@@ -157,3 +157,21 @@ def test_few_cells_per_visibility_stay_unsorted(env):
     st.degrid()
     assert _sorts(st.torch, st.degrid) == 0
     st.check()
+
+
+@pytest.mark.parametrize("support,N,first", [
+    (4, 256, 0), (6, 1024, 1), (6, 1026, 0), (10, 362, 1), (10, 364, 0), (12, 512, 1),
+    (12, 514, 0), (14, 1024, 1), (14, 1026, 0), (18, 256, 0)])
+def test_first_prediction_sorts_dense_plans(env, support, N, first):
+    """2^20 visibilities at and just below the density from which on it does."""
+    st = Step(env, support, nvis=1 << 20, N=N)
+    st.plan()
+    assert _sorts(st.torch, st.degrid) == first
+    st.check()
+
+
+def test_first_prediction_of_fewer_visibilities_does_not_sort(env):
+    st = Step(env, 6, nvis=(1 << 20) - 1, N=256)
+    st.plan()
+    assert _sorts(st.torch, st.degrid) == 0
+    st.check()
