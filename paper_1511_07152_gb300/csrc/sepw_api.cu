@@ -83,8 +83,11 @@ int fail(sepw_ctx *ctx, int code, const char *fmt, ...)
     return code;
 }
 
+// (launch_pdl and the runtime's other calls leave the error set for the next
+// cudaGetLastError, which would refuse a later call)
 int cuda_fail(sepw_ctx *ctx, cudaError_t e, const char *where)
 {
+    cudaGetLastError();
     return fail(ctx, SEPW_ECUDA, "%s: %s", where, cudaGetErrorString(e));
 }
 
