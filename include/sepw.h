@@ -268,7 +268,8 @@ SEPW_API int sepw_set_wait_limit(sepw_ctx *ctx, uint64_t limit_ns);
  * Sec. 4.3): `chunk` visibilities per work item (64 .. 2048, a multiple of
  * 32; 0 = 2048, the default) and the number of parts the FP32 tiled
  * gridders cut an item into, one per warp at a time (1 .. 16; 0 = parts of 32
- * to 1024 visibilities by the plan's size, the default).  Takes
+ * to 1024 visibilities by the plan's size, the default; they are cut from a
+ * tile's visibilities, not item by item).  Takes
  * effect at the next sepw_plan (the current plan is invalidated); results
  * do not depend on it beyond FP32 rounding order.  Host only. */
 SEPW_API int sepw_set_schedule(sepw_ctx *ctx, int32_t chunk, int32_t grid_parts);
@@ -358,8 +359,9 @@ SEPW_API int sepw_taper(sepw_ctx *ctx, float *taper, sepw_stream_t stream);
  *   P * oversample_r^2 * support_r^2 (0 for invalid sizes).
  * sepw_make_residual / _f64: build it in float64 on the GPU (complex64 /
  * complex128 output, device).  Not in facet mode (SEPW_ENOTSUP).  Allocates
- * and frees a temporary of P * oversample_r * support_r * N complex128 and
- * synchronises `stream`: a set-up step, not for the hot loop.
+ * and frees a temporary of P * oversample_r * support_r * N complex128 and, up to
+ * N = 8192, 2 N^2 bytes (134 MB there), and synchronises `stream`: a set-up
+ * step, not for the hot loop.
  * sepw_grid_residual_planned: the correction pass, ADDS to grid the
  * W_i V_i res (conj(res) for w_i < 0) of every planned visibility; after
  * sepw_grid_planned with the full table (support_r = S, oversample_r = OS)

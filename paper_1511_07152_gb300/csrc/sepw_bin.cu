@@ -1,8 +1,9 @@
 // Plan construction for the tiled forms: locate every visibility, bin it by
 // the T x T tile that holds its footprint origin and, inside the tile, by the
-// block of origins (set_bins; counting sort with warp-aggregated atomics), cut each tile into work items of at most kChunk visibilities (and
-// into the smaller units of the tiled gridders), and, for the kernels that
-// walk runs of one origin, sort each item by (footprint origin, conj).
+// block of origins (set_bins; counting sort with warp-aggregated atomics), cut
+// each tile into work items of at most kChunk visibilities (and into the smaller
+// units of the tiled gridders), and, for the kernels that walk runs of one
+// origin, sort each item by (footprint origin, conj).
 //
 // The update structure this serves is Sec. 5: every visibility adds a
 // separable S x S block at its own offset; visibilities that share a tile

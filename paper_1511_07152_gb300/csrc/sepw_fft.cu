@@ -6,10 +6,10 @@
 //   image -> grid:  G[c] = sum_a' (-1)^a' I[a] exp(-2 pi i c a' / N),
 // so the shift is a reordering on the image side and a sign there: no pass
 // over the grids is needed for it.  The column transforms run on the grid
-// side, and the rows where the image side's reordering, sign, grid correction, slice phases and the sum over the slices
-// all fold into the one load or store of a row.  (sepw_image towards the grid
-// keeps its passes: predictions, and a float64 chi^2 of them, stay as they
-// were to the last bit.)
+// side, and the rows where the image side's reordering, sign, grid correction,
+// slice phases and the sum over the slices all fold into the one load or store
+// of a row.  (sepw_image towards the grid has no transform here: it runs cuFFT
+// between two passes over the grid.)
 //
 // What that saves: the passes are bound by memory.  Per direction the slice
 // grids were read and written by a sign pass, by the row transform and by the
@@ -362,8 +362,8 @@ __device__ __forceinline__ int index_out(int k)
 // Inverse rows in place, rows g and g + N/2 by one block (each lands in the
 // other's place): buf[b][a] = scale * transform.
 template <int R>
-__global__ void __launch_bounds__(Rows<R>::T, Rows<R>::BPS) rows_to_image_kernel(Pixels px, int mode, float2 *buf,
-                                                                   const float2 *__restrict__ tab)
+__global__ void __launch_bounds__(Rows<R>::T, Rows<R>::BPS) rows_to_image_kernel(
+    Pixels px, int mode, float2 *buf, const float2 *__restrict__ tab)
 {
     __shared__ float2 shm[Rows<R>::kShm];
     const int N = Rows<R>::N;

@@ -306,9 +306,9 @@ struct alignas(16) Slot {
 // are read again and again, stay there: window gridder at S = 12, 63M
 // visibilities, 6076 -> 5959 us; TF32 gridder, 32M, 3335 -> 3252 us; BF16 and
 // BF16 hi + lo gridders 0.1% and 0.2%, their degridders 0.5% by the slots alone.  The
-// hi + lo gridder (values loaded where they are used: 2504 -> 2578 us) and the
-// degridders' weights (neighbours share a sector: BF16 1597 -> 2026 us) keep
-// __ldg for theirs.
+// hi + lo gridder's values (loaded where they are used: 2504 -> 2578 us) and the
+// degridders' weights (neighbours share a sector: BF16 1597 -> 2026 us) go through
+// L1.
 __device__ __forceinline__ float2 load_once(const float2 *p)
 {
     float2 x;
@@ -474,7 +474,6 @@ constexpr int kMaxSubBins = 64;
 // items were sorted after it was made (launch_item_sort)
 constexpr size_t kBinHeader = 64, kBinTicket = 8, kBinSortMark = 12;
 
-// ceil(2^32 / T) for the tile edge T (8 <= T <= 64)
 // Bounds of locate_axis's integer path for grid size N and OS = 2^os_log2
 // (os_log2 < 0: path off): |y OS| < 2^elim with 2^elim <= N OS / 2 and
 // elim <= 21; margin (N OS) 2^-53 in units of 2^-32, rounded up, and 2 for the
@@ -493,6 +492,7 @@ inline void locate_fast_bounds(int N, int os_log2, int32_t &elim, int32_t &near)
     near = (int32_t)((((long long)N << os_log2) >> 21) + 3);
 }
 
+// ceil(2^32 / T) for the tile edge T (8 <= T <= 64)
 inline uint32_t tile_reciprocal(int T)
 {
     return (uint32_t)((0x100000000ull + (uint64_t)T - 1) / (uint64_t)T);

@@ -1,13 +1,13 @@
 // Tiled FP32 gridder and degridder (the separable update of Sec. 5, binned).
 //
 // Work items are <= kChunk visibilities of one T x T tile, sorted by
-// (footprint origin, conj) ("key").  A warp of a block gridder takes units of 32 to
-// 256 of a tile's visibilities from an atomic counter; a CTA of a degridder takes
-// parts of an item and keeps the tile's window of (T + S - 1)^2 cells in shared
-// memory.  Per batch of
-// visibilities a warp first decodes the records once (one per lane: tap-row
-// offsets, W V or the output index and weight, key) into shared memory; the
-// inner loop reads them as broadcasts.
+// (footprint origin, conj) ("key").  A warp of a block gridder takes units of a
+// tile's visibilities (32 to 256, see set_units, unless a schedule was set) from
+// an atomic counter; a CTA of a degridder takes parts of an item (degrid_parts)
+// and keeps the tile's window of (T + S - 1)^2 cells in shared memory.  Per
+// batch of visibilities a warp first decodes the records once (one per lane:
+// tap-row offsets, W V or the output index and weight, key) into shared memory;
+// the inner loop reads them as broadcasts.
 //
 // What limits these kernels is the load data returned to the registers, the
 // latency of those loads (gridder) and the instruction issue (degridder),
@@ -871,7 +871,8 @@ static cudaError_t launch_grid_S(const DevParams &p, const Plan &plan, const flo
             if (e != cudaSuccess)
                 return e;
             return launch_pdl(grid_tiled_block_kernel<S, true>, nb, kTiledThreads, 0, s, p,
-                              plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_slots, vis, weight, taps, planar, grid);
+                              plan.d_units, plan.d_nunits, plan.d_item_counter, plan.d_slots,
+                              vis, weight, taps, planar, grid);
         }
     }
     cudaError_t e = cudaMemsetAsync(plan.d_item_counter, 0, sizeof(int32_t), s);
@@ -887,7 +888,8 @@ static cudaError_t launch_grid_S(const DevParams &p, const Plan &plan, const flo
                           grid);
     else
         return launch_pdl(grid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, 0, s,
-                          p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_slots, vis, weight, taps, grid);
+                          p, plan.d_items, plan.d_nitems, plan.d_item_counter, plan.d_slots,
+                          vis, weight, taps, grid);
 }
 
 template <int S>
@@ -903,13 +905,15 @@ static cudaError_t launch_degrid_S(const DevParams &p, const Plan &plan,
         const int WP = W + ((4 - W % 8) + 8) % 8;
         const size_t shm = sizeof(float4) * (size_t)((W * WP + 1) / 2) +
                            (size_t)kTiledWarps * 2 * Blk<S>::MS * (sizeof(int4) + sizeof(int));
-        return launch_pdl(
-            degrid_tiled_block_kernel<S>, num_sms * Blk<S>::BPS, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_slots, grid, weight, taps, vis);
+        return launch_pdl(degrid_tiled_block_kernel<S>, num_sms * Blk<S>::BPS, kTiledThreads, shm,
+                          s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1,
+                          plan.d_slots, grid, weight, taps, vis);
     } else {
         const int WP = window_stride(W, S);
         const size_t shm = tiled_smem(W, WP);
-        return launch_pdl(
-            degrid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, shm, s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1, plan.d_slots, grid, weight, taps, vis);
+        return launch_pdl(degrid_tiled_kernel<S>, num_sms * kTiledBlocksPerSM, kTiledThreads, shm,
+                          s, p, WP, plan.d_items, plan.d_nitems, plan.d_item_counter + 1,
+                          plan.d_slots, grid, weight, taps, vis);
     }
 }
 
