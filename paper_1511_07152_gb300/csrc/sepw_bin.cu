@@ -10,6 +10,7 @@
 // share one shared-memory window, and visibilities that share an origin share
 // one register block.
 #include <algorithm>
+#include <limits>
 
 #include "sepw_internal.cuh"
 
@@ -108,11 +109,28 @@ __device__ __forceinline__ Totals operator-(const Totals &a, const Totals &b)
 }
 // How tiles are cut: items of `chunk`; units of a `parts`-th of the tile, at
 // most `unit` and a multiple of 32 (all of them `unit` when parts is 1).
+//
+// A cell's sum takes two steps, within a unit and over the units, and is the less
+// exact the longer either of them is.  Units of a tile of kHeavyTile or more are
+// no shorter than the root of its number, up to kLongUnit; windows from `dense`
+// visibilities a tile on are no longer than kDenseUnit.  Error of grids on tracks
+// with residuals that do not average out, units of 32, this rule, eighths of
+// items, and the gridder's time with the first two: 35k visibilities on 240^2 at
+// S = 6 1.8e-7, 1.3e-7, 1.4e-7 (15 and 32 us); 100k on 500^2 at S = 8 2.0e-7,
+// 1.8e-7, 1.8e-7 (15 and 27); 300k on 300^2 at S = 8 3.4e-7, 2.4e-7, 2.7e-7 (19
+// and 29).  Windows of 2048 at S = 6: 35k 5.7e-7, 1.5e-7 cut to 256; 300k on 700^2
+// 5.3e-7 and 1.3e-7.  Lighter tiles are as exact with units of 32 (20k on 400^2 at
+// S = 8 1.74e-7, 1.60e-7 with 64, 1.76e-7 with eighths), and faster (15 and 29 us).
+constexpr int kHeavyTile = 4096, kLongUnit = 128, kDenseUnit = 256;
 struct Cut {
-    int32_t chunk, unit, parts;
+    int32_t chunk, unit, parts, dense;
     __device__ __forceinline__ int unit_of(int n) const
     {
-        return parts > 1 ? max(32, min(unit, (n / parts + 31) & ~31)) : unit;
+        const int u = parts > 1 ? max(32, min(unit, (n / parts + 31) & ~31)) : unit;
+        if (n < min(dense, kHeavyTile))
+            return u;
+        const int root = n < kHeavyTile ? 0 : ((int)__fsqrt_rn((float)n) + 31) & ~31;
+        return max(n >= dense ? min(u, kDenseUnit) : u, min(root, kLongUnit));
     }
 };
 __device__ __forceinline__ Totals tile_totals(int n, const Cut &cut)
@@ -567,12 +585,13 @@ void set_units(const DevParams &p, int num_sms, Plan &plan)
             8, std::max<int64_t>(1, 640ll * num_sms / std::max(1, plan.ntiles)));
 }
 
-// units of any plan that set_units cuts: a full one takes unit visibilities or
-// more than a ninth of its tile
+// units of any plan that set_units cuts: a full one takes unit (kDenseUnit, where
+// that is less) visibilities or more than a ninth of its tile
 int64_t max_units(const Plan &plan)
 {
-    const int64_t cut = plan.nvis / (plan.unit_parts > 1 ? 32 : plan.unit);
-    return std::min(cut, plan.nvis / plan.unit + (int64_t)plan.unit_parts * plan.ntiles) +
+    const int unit = std::min(plan.unit, kDenseUnit);
+    const int64_t cut = plan.nvis / (plan.unit_parts > 1 ? 32 : unit);
+    return std::min(cut, plan.nvis / unit + (int64_t)plan.unit_parts * plan.ntiles) +
            plan.ntiles + 1;
 }
 
@@ -624,7 +643,8 @@ cudaError_t launch_plan(const DevParams &p, int64_t nvis, const double *u,
                         plan.d_tile, plan.d_rank, plan.d_rec0, bin, plan.d_dropped,
                         plan.d_drop_list, plan.ngrids, plan.d_offsets)) != cudaSuccess)
         return e;
-    const Cut cut{p.chunk, plan.unit, plan.unit_parts};
+    const Cut cut{p.chunk, plan.unit, plan.unit_parts,
+                  plan.window ? p.T * p.T : std::numeric_limits<int32_t>::max()};
     Totals *const blocks = (Totals *)plan.d_blocks;
     if (plan.ntiles <= kOneBlockTiles) {
         e = launch_pdl(tile_items_kernel<true>, 1, kPlanThreads, 0, s, plan.ntiles,
