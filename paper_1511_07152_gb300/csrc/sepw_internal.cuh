@@ -422,7 +422,7 @@ constexpr int kMaxWindow = 64;    // T + S - 1 <= kMaxWindow
 //     go, for grids of few tiles: locate_bin_kernel sends an atomic per warp
 //     and bin to the counters, and those of few bins lie in few L2 sectors,
 //     where they queue.
-//   kBinsTile: one bin, for the tensor-core forms, which take any order.
+//   kBinsTile: one bin, for the 16-bit tensor-core forms, which take any order.
 // Which one: plan_bins.
 enum PlanBins { kBinsWindow, kBinsSorted, kBinsFine, kBinsTile };
 inline void set_bins(DevParams &d, PlanBins b)
@@ -458,10 +458,18 @@ inline void set_bins(DevParams &d, PlanBins b)
 // 618; but 6241 tiles 630 and 596, and 256 tiles 935 and 693 (557 with edge
 // 4).  600k on 10404 tiles 306 and 314, 30k on 100 tiles 65 and 69 (tracks);
 // 100k on 400 tiles 80 and 73.
+//
+// Not for FP16 hi + lo, whose error is that of the FP32 sums in tensor memory:
+// an MMA adds its 16 visibilities to a cell at once, and in block order fewer MMAs
+// reach a cell.  Error with one bin and edge 8, tracks: 30k on 700^2 at S = 8
+// 1.4e-6 and 0.87e-6, 122k on 2162^2 at S = 6 8.1e-7 and 5.4e-7, 8M on 4096^2 at
+// S = 16 2.3e-6 and 2.1e-6 (step 1648 and 1714 us).  (BF16 hi + lo: 4.5e-6 either
+// way, by its operands.)
 inline PlanBins plan_bins(const DevParams &p, int form, int64_t nvis, int64_t ntiles)
 {
     const bool sorts = form == SEPW_FORM_TILED || form == SEPW_FORM_TC_TF32;
-    if (!sorts && (ntiles >= 16384 || nvis < 64 * ntiles || nvis <= 32768))
+    if (!sorts && form != SEPW_FORM_TC_FP16X2 &&
+        (ntiles >= 16384 || nvis < 64 * ntiles || nvis <= 32768))
         return kBinsTile;
     DevParams d = p;
     set_bins(d, kBinsSorted);
